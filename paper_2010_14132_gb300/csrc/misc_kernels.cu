@@ -470,122 +470,136 @@ cudaError_t launch_finalize(const float* p0, const float* q, double* p, long lon
 //   dL/drho_m = -sum_k (da_k/drho_m * Ma_k + dc_k/drho_m * Mc_k),
 //   Mc_k = Lo_k,  Ma_k = -Up_{k-1}.
 // Partials per (face, block) are reduced in a fixed order (deterministic).
+//
+// The double form is bound by the FP64 pipe: one subtraction and two FMAs a point, the level planes of
+// neighbouring faces coming from L2.  The block reduction costs as many FP64 instructions per warp as
+// some ten points do, so a thread takes at least kGrhoPoints points (one point a thread, as it was,
+// spent several times the work of the sums in the reductions: 512 x 512 x 64, both kernels together 831 ->
+// about 165 us).  The float
+// forms round the products to float and add them in pairs of floats (hi + lo, exact two-sums), so that
+// a longer sum per thread loses nothing.
 // ---------------------------------------------------------------------------
-template <typename TIO>
-__global__ void __launch_bounds__(256) k_grho_partial(const TIO* __restrict__ gS, const TIO* __restrict__ p,
-                                                      long long plane, double* __restrict__ partials) {
-  __shared__ double s0[256], s1[256];
+constexpr int kGrhoPoints = 32;
+
+struct GrhoSumD {   // FP64 fields
+  using V = double2;
+  double lo0 = 0, up0 = 0, lo1 = 0, up1 = 0;
+  __device__ __forceinline__ void add(V p0, V p1, V g0, V g1) {
+    const double d0 = p1.x - p0.x, d1 = p1.y - p0.y;
+    lo0 = fma(g0.x, d0, lo0);
+    up0 = fma(g1.x, d0, up0);
+    lo1 = fma(g0.y, d1, lo1);
+    up1 = fma(g1.y, d1, up1);
+  }
+  __device__ __forceinline__ double lo() const { return lo0 + lo1; }
+  __device__ __forceinline__ double up() const { return up0 + up1; }
+};
+struct GrhoSumF {   // float products, sums as float pairs
+  using V = float2;
+  float lh = 0, ll = 0, uh = 0, ul = 0;
+  __device__ __forceinline__ void one(float p0, float p1, float g0, float g1) {
+    const float d = p1 - p0;
+    float e;
+    two_sum(lh, __fmul_rn(g0, d), lh, e);
+    ll += e;
+    two_sum(uh, __fmul_rn(g1, d), uh, e);
+    ul += e;
+  }
+  __device__ __forceinline__ void add(V p0, V p1, V g0, V g1) {
+    one(p0.x, p1.x, g0.x, g1.x);
+    one(p0.y, p1.y, g0.y, g1.y);
+  }
+  __device__ __forceinline__ double lo() const { return (double)lh + (double)ll; }
+  __device__ __forceinline__ double up() const { return (double)uh + (double)ul; }
+};
+struct GrhoSumM : GrhoSumF {   // mixed: double fields, rounded to float with integer operations
+  using V = double2;
+  __device__ __forceinline__ void add(V p0, V p1, V g0, V g1) {
+    one(d2f_int(p0.x), d2f_int(p1.x), d2f_int(g0.x), d2f_int(g1.x));
+    one(d2f_int(p0.y), d2f_int(p1.y), d2f_int(g0.y), d2f_int(g1.y));
+  }
+};
+
+// half: pairs of points per level plane (nx is even, so the planes hold whole, aligned pairs)
+template <typename Sum>
+__global__ void __launch_bounds__(256) k_grho_partial(const typename Sum::V* __restrict__ gS,
+                                                      const typename Sum::V* __restrict__ p, long long half,
+                                                      double* __restrict__ partials) {
   const int f = blockIdx.y;
-  const TIO* g0 = gS + f * plane;
-  const TIO* g1 = g0 + plane;
-  const TIO* p0 = p + f * plane;
-  const TIO* p1 = p0 + plane;
-  TIO lo = 0, up = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (long long)gridDim.x * blockDim.x) {
-    const TIO d = p1[i] - p0[i];
-    lo += g0[i] * d;
-    up += g1[i] * d;
+  const typename Sum::V* g0 = gS + f * half;
+  const typename Sum::V* p0 = p + f * half;
+  Sum a;
+#pragma unroll 4
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < half; i += (long long)gridDim.x * blockDim.x)
+    a.add(p0[i], p0[i + half], g0[i], g0[i + half]);
+  double lo = a.lo(), up = a.up();
+  for (int o = 16; o > 0; o >>= 1) {
+    lo += __shfl_down_sync(0xffffffffu, lo, o);
+    up += __shfl_down_sync(0xffffffffu, up, o);
   }
+  __shared__ double s[2][8];
   const int t = threadIdx.x;
-  s0[t] = (double)lo;
-  s1[t] = (double)up;
-  __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (t < h) {
-      s0[t] += s0[t + h];
-      s1[t] += s1[t + h];
-    }
-    __syncthreads();
+  if ((t & 31) == 0) {
+    s[0][t >> 5] = lo;
+    s[1][t >> 5] = up;
   }
-  if (t == 0) {
-    partials[2 * ((long long)f * gridDim.x + blockIdx.x)] = s0[0];
-    partials[2 * ((long long)f * gridDim.x + blockIdx.x) + 1] = s1[0];
+  __syncthreads();
+  if (t < 2) {
+    double v = 0;
+    for (int w = 0; w < 8; ++w) v += s[t][w];
+    partials[2 * ((long long)f * gridDim.x + blockIdx.x) + t] = v;
   }
 }
 
-// Mixed dtype: double fields converted with integer operations, float products.
-__global__ void __launch_bounds__(256) k_grho_partial_mixed(const double* __restrict__ gS,
-                                                            const double* __restrict__ p, long long plane,
-                                                            double* __restrict__ partials) {
-  __shared__ double s0[256], s1[256];
-  const int f = blockIdx.y;
-  const double* g0 = gS + f * plane;
-  const double* g1 = g0 + plane;
-  const double* p0 = p + f * plane;
-  const double* p1 = p0 + plane;
-  float lo = 0, up = 0;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < plane; i += (long long)gridDim.x * blockDim.x) {
-    const float d = d2f_int(p1[i]) - d2f_int(p0[i]);
-    lo += d2f_int(g0[i]) * d;
-    up += d2f_int(g1[i]) * d;
-  }
-  const int t = threadIdx.x;
-  s0[t] = (double)lo;
-  s1[t] = (double)up;
+// One block per level m: warps 0..3 sum the (Lo, Up) partials of the faces m-1 and m in a fixed order
+// (a thread per level looping over every block's partials took 260 us at 512 x 512 x 64).
+__global__ void __launch_bounds__(128) k_grho_final(const double* __restrict__ partials, int nb, int nz,
+                                                    const double* __restrict__ dz, const double* __restrict__ rho,
+                                                    const double* __restrict__ a, const double* __restrict__ c,
+                                                    const double* __restrict__ W, double* __restrict__ grho) {
+  __shared__ double sum[4];
+  const int m = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int f = m - 1 + (w >> 1), which = w & 1;   // face and sum of this warp
+  double v = 0;
+  if (f >= 0 && f < nz - 1)
+    for (int b = lane; b < nb; b += 32) v += partials[2 * ((long long)f * nb + b) + which];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if (lane == 0) sum[w] = v;
   __syncthreads();
-  for (int h = 128; h > 0; h >>= 1) {
-    if (t < h) {
-      s0[t] += s0[t + h];
-      s1[t] += s1[t + h];
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    partials[2 * ((long long)f * gridDim.x + blockIdx.x)] = s0[0];
-    partials[2 * ((long long)f * gridDim.x + blockIdx.x) + 1] = s1[0];
-  }
-}
-
-// One thread per level m; each sums the partials of faces m-1 and m in fixed order.
-__global__ void k_grho_final(const double* __restrict__ partials, int nb, int nz, const double* __restrict__ dz,
-                             const double* __restrict__ rho, const double* __restrict__ a,
-                             const double* __restrict__ c, const double* __restrict__ W, double* __restrict__ grho) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  if (m >= nz) return;
-  auto face = [&](int f, int which) {
-    double s = 0;
-    for (int b = 0; b < nb; ++b) s += partials[2 * ((long long)f * nb + b) + which];
-    return s;
-  };
-  auto hf = [&](int f) { return 0.5 * (dz[f] + dz[f + 1]); };
+  if (threadIdx.x != 0) return;
+  const double lo_dn = sum[0], up_dn = sum[1], lo_up = sum[2], up_up = sum[3];
+  auto hf = [&](int face) { return 0.5 * (dz[face] + dz[face + 1]); };
   double acc = 0;
   // a-terms: k = m (face m-1) and k = m+1 (face m); Ma_k = -Up_{k-1}
-  if (m >= 1) {
-    const double Ma = -face(m - 1, 1);
-    acc += (0.5 / (W[m] * hf(m - 1)) - a[m] / rho[m]) * Ma;
-  }
-  if (m + 1 <= nz - 1) {
-    const double Ma = -face(m, 1);
-    acc += (0.5 / (W[m + 1] * hf(m))) * Ma;
-  }
+  if (m >= 1) acc += (0.5 / (W[m] * hf(m - 1)) - a[m] / rho[m]) * -up_dn;
+  if (m + 1 <= nz - 1) acc += (0.5 / (W[m + 1] * hf(m))) * -up_up;
   // c-terms: k = m (face m) and k = m-1 (face m-1); Mc_k = Lo_k
-  if (m <= nz - 2) {
-    const double Mc = face(m, 0);
-    acc += (0.5 / (W[m] * hf(m)) - c[m] / rho[m]) * Mc;
-  }
-  if (m >= 1) {
-    const double Mc = face(m - 1, 0);
-    acc += (0.5 / (W[m - 1] * hf(m - 1))) * Mc;
-  }
+  if (m <= nz - 2) acc += (0.5 / (W[m] * hf(m)) - c[m] / rho[m]) * lo_up;
+  if (m >= 1) acc += (0.5 / (W[m - 1] * hf(m - 1))) * lo_dn;
   grho[m] = -acc;
 }
 
 cudaError_t launch_grho(int kind, const void* g, const void* p, const Geom& g_, const Tables& tb, const double* dz,
                         const double* rho0, double* partials, int nparts_max, double* grho, cudaStream_t st) {
-  const long long plane = (long long)g_.nx * g_.ny;
-  int nb = (int)((plane + 255) / 256);
+  const long long half = (long long)g_.nx * g_.ny / 2;
+  // kGrhoPoints points a thread, fewer while that leaves less than about four blocks per SM
+  const int faces = g_.nz - 1;
+  long long nb = (2 * half + 256 * kGrhoPoints - 1) / (256 * kGrhoPoints);
+  const long long fill = (608 + faces - 1) / faces, most = (half + 255) / 256;
+  if (nb < fill) nb = fill;
+  if (nb > most) nb = most;
   if (nb > nparts_max) nb = nparts_max;
   if (nb < 1) nb = 1;
-  const dim3 grid(nb, g_.nz - 1);
+  const dim3 grid((unsigned)nb, faces);
   if (kind == 0)
-    k_grho_partial<double><<<grid, 256, 0, st>>>((const double*)g, (const double*)p, plane, partials);
+    k_grho_partial<GrhoSumD><<<grid, 256, 0, st>>>((const double2*)g, (const double2*)p, half, partials);
   else if (kind == 1)
-    k_grho_partial<float><<<grid, 256, 0, st>>>((const float*)g, (const float*)p, plane, partials);
+    k_grho_partial<GrhoSumF><<<grid, 256, 0, st>>>((const float2*)g, (const float2*)p, half, partials);
   else
-    k_grho_partial_mixed<<<grid, 256, 0, st>>>((const double*)g, (const double*)p, plane, partials);
+    k_grho_partial<GrhoSumM><<<grid, 256, 0, st>>>((const double2*)g, (const double2*)p, half, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_grho_final<<<(g_.nz + 127) / 128, 128, 0, st>>>(partials, nb, g_.nz, dz, rho0, tb.a_d, tb.c_d, tb.W_d, grho);
+  k_grho_final<<<g_.nz, 128, 0, st>>>(partials, (int)nb, g_.nz, dz, rho0, tb.a_d, tb.c_d, tb.W_d, grho);
   return cudaGetLastError();
 }
 
