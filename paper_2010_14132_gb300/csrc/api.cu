@@ -379,6 +379,14 @@ int poisson_plan_create(int nx, int ny, int nz, double dx, double dy, const doub
     ly[k] = -(4.0 / (dy * dy)) * sn * sn;
   }
 
+  // fixed-point twiddles of the FP64 transforms (empty where a length has no such kernel)
+  std::vector<int4> fxq, frq, fyq;
+  if (dtype == POISSON_FP64) {
+    fxq = fx_stage_table(n);
+    if (!fxq.empty()) frq = fx_unpack_table(nx);
+    fyq = fx_stage_table(ny);
+  }
+
   // ---- one device block for all tables
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -390,7 +398,9 @@ int poisson_plan_create(int nx, int ny, int nz, double dx, double dy, const doub
                o_aff = take(nz * 8), o_cff = take(nz * 8), o_lxd = take(pl->nxh * 8),
                o_lyd = take(ny * 8), o_lxf = take(pl->nxh * 4), o_lyf = take(ny * 4), o_twxd = take(n * 16),
                o_twrd = take(pl->nxh * 16), o_twyd = take(ny * 16), o_twxf = take(n * 8), o_twrf = take(pl->nxh * 8),
-               o_twyf = take(ny * 8), o_dz = take(nz * 8), o_rho = take(nz * 8), o_floor = take(32);
+               o_twyf = take(ny * 8), o_dz = take(nz * 8), o_rho = take(nz * 8), o_floor = take(32),
+               o_fxq = take(fxq.size() * sizeof(int4)), o_frq = take(frq.size() * sizeof(int4)),
+               o_fyq = take(fyq.size() * sizeof(int4));
   cudaError_t e = cudaMalloc(&pl->tables, off);
   if (e != cudaSuccess) {
     delete pl;
@@ -418,6 +428,9 @@ int poisson_plan_create(int nx, int ny, int nz, double dx, double dy, const doub
   if (ce == cudaSuccess) ce = upd(o_twxf, twxf.data(), n * 8);
   if (ce == cudaSuccess) ce = upd(o_twrf, twrf.data(), pl->nxh * 8);
   if (ce == cudaSuccess) ce = upd(o_twyf, twyf.data(), ny * 8);
+  if (ce == cudaSuccess && !fxq.empty()) ce = upd(o_fxq, fxq.data(), fxq.size() * sizeof(int4));
+  if (ce == cudaSuccess && !frq.empty()) ce = upd(o_frq, frq.data(), frq.size() * sizeof(int4));
+  if (ce == cudaSuccess && !fyq.empty()) ce = upd(o_fyq, fyq.data(), fyq.size() * sizeof(int4));
   if (ce == cudaSuccess) ce = upd(o_dz, dz, nz * 8);
   if (ce == cudaSuccess) ce = upd(o_rho, rho0, nz * 8);
   Tables& tb = pl->tb;
@@ -439,6 +452,9 @@ int poisson_plan_create(int nx, int ny, int nz, double dx, double dy, const doub
   tb.twr_f = (float2*)(base + o_twrf);
   tb.twy_f = (float2*)(base + o_twyf);
   tb.floor_d = (double*)(base + o_floor);
+  tb.twx_q = fxq.empty() ? nullptr : (int4*)(base + o_fxq);
+  tb.twr_q = frq.empty() ? nullptr : (int4*)(base + o_frq);
+  tb.twy_q = fyq.empty() ? nullptr : (int4*)(base + o_fyq);
   pl->dz_d = (double*)(base + o_dz);
   pl->rho_d = (double*)(base + o_rho);
   if (ce == cudaSuccess)
@@ -616,6 +632,11 @@ static int check_ws(const poisson_plan* pl, void* ws) {
 static cudaError_t ypass(poisson_plan* pl, const Geom& g, int sign, void* spec, const int* done, Stats* stats,
                          cudaStream_t st) {
   const bool t_double = pl->fp64();
+  if (t_double && pl->ykernel != 1 && pl->ykernel != 2) {
+    bool used = false;
+    cudaError_t e = launch_yfft_fx(sign, (double2*)spec, g, pl->ny, pl->tb, st, &used);
+    if (e != cudaSuccess || used) return e;
+  }
   if ((pl->ykernel == 0 || pl->ykernel == 3 || pl->ykernel == 4) && !t_double) {
     bool used = false;
     const int variant = pl->ykernel == 3 ? 1 : (pl->ykernel == 4 ? 2 : 0);
@@ -691,7 +712,9 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
       rparts += nb;
     } else {
       bool used = false;
-      if (!t_double && pl->xkernel == 0)
+      if (t_double && pl->xkernel == 0)
+        e = launch_xfwd_fx((const double*)in, (double2*)spec, gc, pl->nx / 2, pl->tb, st, &used);
+      else if (!t_double && pl->xkernel == 0)
         e = launch_xfwd_static(in_double, in, spec, gc, pl->fx, pl->tb, done, &stats->err, st, &used);
       if (e == cudaSuccess && !used) e = launch_xfwd(in_double, t_double, in, spec, gc, pl->fx, pl->tb, done, st);
     }
@@ -803,7 +826,9 @@ static cudaError_t inverse(poisson_plan* pl, char* ws, cudaStream_t st, const in
     // one chunk: the static kernel's last CTA runs the refinement control itself
     const bool fuse = control_fused && mode != XINV_PLAIN && lc >= pl->nz;
     if (!fuse) exs.ctl_stats = nullptr;
-    if (!t_double && pl->xkernel == 0)
+    if (t_double && pl->xkernel == 0)
+      e = launch_xinv_fx((const double2*)spec, (double*)out, gc, pl->nx / 2, pl->tb, st, &used);
+    else if (!t_double && pl->xkernel == 0)
       e = launch_xinv_static(to_double, mode, spec, out, gc, pl->fx, pl->tb, exs, &nb, st, &used);
     if (used && fuse) *control_fused = true;
     if (e == cudaSuccess && !used) e = launch_xinv(t_double, to_double, mode, spec, out, gc, pl->fx, pl->tb, ex, &nb, st);

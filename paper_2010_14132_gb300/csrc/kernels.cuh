@@ -141,6 +141,9 @@ struct Tables {
   // twiddles exp(-2 pi i m / n): x line (n = nx/2), R2C post (m = 0..nx/2 over nx), y line
   const double2* twx_d; const double2* twr_d; const double2* twy_d;
   const float2* twx_f; const float2* twr_f; const float2* twy_f;
+  // fixed-point twiddles of the FP64 transforms (null where the length has no such kernel): stage-ordered
+  // tables of the x and y lines, R2C post-twiddles (m = 0..nx/2)
+  const int4* twx_q; const int4* twr_q; const int4* twy_q;
   // limiting accuracy of the mixed refinement's error bound (one double, launch_accuracy_floor)
   const double* floor_d;
 };
@@ -214,6 +217,17 @@ cudaError_t launch_xfwd_residual(const ResidualArgs& R, void* spec, const Geom& 
                                  const Tables& tb, const int* done, int* nblocks_out, cudaStream_t st);
 cudaError_t launch_yfft(int t_is_double, int sign, void* spec, const Geom& g, const FftPlan& fy,
                         const Tables& tb, int tile, const int* done, cudaStream_t st);
+// FP64 passes in 64-bit block fixed point (fx_xpass.cu, fx_ypass.cu); *used = false when the plan has no
+// tables for them (a line length outside fx_supported).
+bool fx_supported(int n);
+std::vector<int4> fx_stage_table(int n);
+std::vector<int4> fx_unpack_table(int nx);
+cudaError_t launch_xfwd_fx(const double* in, double2* spec, const Geom& g, int n, const Tables& tb, cudaStream_t st,
+                           bool* used);
+cudaError_t launch_xinv_fx(const double2* spec, double* out, const Geom& g, int n, const Tables& tb, cudaStream_t st,
+                           bool* used);
+cudaError_t launch_yfft_fx(int sign, double2* spec, const Geom& g, int n, const Tables& tb, cudaStream_t st,
+                           bool* used);
 // 2-D tensor map over 8-byte elements (dim0 contiguous, dim1 rows of row_stride_bytes);
 // false when the driver entry point is unavailable or the shape is rejected.
 bool encode_tensor_2d(CUtensorMap* tm, void* base, size_t elem_bytes, unsigned long long dim0,
