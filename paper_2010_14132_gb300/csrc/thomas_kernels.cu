@@ -355,6 +355,157 @@ __global__ void __launch_bounds__(128) k_thomas_tw(float2* __restrict__ spec, Ge
 }
 
 // ---------------------------------------------------------------------------
+// FP64 column kernel: the twisted elimination with both halves of a column in one warp.
+//
+// Bound by the FP64 unit, which takes a warp's instruction in about 76 clocks whatever its lanes do: what counts
+// is the number of FP64 instructions per entry, that all lanes work, and (small grids) their number along
+// a column.  Hence
+//  * lanes 0-15 eliminate 16 columns upwards (levels 0..m-1), lanes 16-31 the same columns downwards (levels
+//    nz-1..m+1) with the same instructions, p and q being (a, c) for the one and (c, a) for the other:
+//        g_k = s + p_k (g/u)_prev,  u_k = g_k + q_k,  z_k = (b_k + e_k z_prev)/u_k,  w_k = r_k/u_k,
+//    forward e = p_k, r = q_k; adjoint (M^T: the couplings of the neighbouring rows) e_k = q_prev, r_k = p_next.
+//    They meet at m = nz/2 by a shuffle and substitute back outwards, x_k = z_k + w_k x_next.
+//  * the matrix is scaled by -nx ny instead of every entry by -1/(nx ny);
+//  * 1/u_k is the hardware's approximation (2^-20 or better) and one step of third order (Halley's iteration,
+//    e = 1 - u r, r (1 + e + e^2)): 3 instructions, half a unit in the last place;
+//  * NR = 4: a lane carries the columns (kx, ky) and (kx, ny - ky), which have the same pivots: 9.5 FP64
+//    instructions an entry, where one thread per column with a division per level took 17.  Grids with too few
+//    columns to fill the SMs take NR = 2 (one column a lane, 13 instructions per level) or NR = 1 (one real or
+//    imaginary part a lane, 10 per level): fewer along the chain.
+// The right-hand sides are read a level ahead straight from the spectrum and z is kept there in place (a level
+// takes over a thousand clocks); only the factors w stay in shared memory, so the levels do not limit
+// the warps per SM.  512 x 512 x 64: 337 -> 172 us, adjoint 326 -> 174; 256 x 256 x 64: 99 -> 57;
+// 32 x 32 x 32: 27 -> 18.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double rcp_halley(double u) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(u));
+  double e = fma(-u, r, 1.0);
+  e = fma(e, e, e);
+  return fma(r, e, r);
+}
+
+// NR values of one level of a lane's column(s); b is the second column's offset from the first (NR = 4)
+template <int NR> struct ColVals {
+  double v[NR];
+  __device__ __forceinline__ void load(const double* p, long long b) {
+    if constexpr (NR == 1) {
+      v[0] = *p;
+    } else {
+      const double2 x = *reinterpret_cast<const double2*>(p);
+      v[0] = x.x;
+      v[1] = x.y;
+      if constexpr (NR == 4) {
+        const double2 y = *reinterpret_cast<const double2*>(p + b);
+        v[2] = y.x;
+        v[3] = y.y;
+      }
+    }
+  }
+  __device__ __forceinline__ void store(double* p, long long b) const {
+    if constexpr (NR == 1) {
+      *p = v[0];
+    } else {
+      *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+      if constexpr (NR == 4) {
+        if (b) *reinterpret_cast<double2*>(p + b) = make_double2(v[2], v[3]);
+      }
+    }
+  }
+};
+
+template <int NR, bool ADJ>
+__global__ void __launch_bounds__(32) k_thomas_d(double2* __restrict__ spec, Geom g, const double* __restrict__ a,
+                                                const double* __restrict__ c, const double* __restrict__ lamx,
+                                                const double* __restrict__ lamy, int lowk_r2, Stats* stats, LowkArgs L) {
+  pdl_trigger();
+  extern __shared__ __align__(128) unsigned char smraw[];
+  if ((int)blockIdx.x < L.n) {
+    pdl_wait();
+    lowk_column<double, double, ADJ>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.lamx_d, L.lamy_d, L.scale,
+                                     L.cols[blockIdx.x], stats, L.target_mean, L.singular00 != 0, nullptr, L.inv_tab,
+                                     blockIdx.x);
+    return;
+  }
+  const int t = threadIdx.x, nz = g.nz, m = nz / 2;
+  double* cf = reinterpret_cast<double*>(smraw);   // -nx ny a_k, then -nx ny c_k
+  double* w = cf + 2 * nz + t;                     // [m][32] factors
+  const double ms = -(double)g.nx * (double)g.ny;
+  pdl_wait();   // also for a, c: poisson_plan_set_rho0 writes them on the stream
+  for (int k = t; k < nz; k += 32) {
+    cf[k] = ms * a[k];
+    cf[nz + k] = ms * c[k];
+  }
+  __syncwarp();
+  const int up = t >> 4;
+  const long long lane = (long long)(blockIdx.x - L.n) * 16 + (t & 15);
+  const long long cols = (long long)(NR == 4 ? g.ny / 2 + 1 : g.ny) * g.nxh;
+  long long col = NR == 1 ? lane >> 1 : lane;
+  bool valid = col < cols;
+  if (!valid) col = cols - 1;
+  const int ky = (int)(col / g.nxh), kx = (int)(col - (long long)ky * g.nxh);
+  const int kys = signed_ky(ky, g.ny);
+  valid = valid && kx * kx + kys * kys > lowk_r2;
+  const long long ld = 2 * g.plane;   // doubles from level to level
+  const long long second = NR == 4 ? 2ll * ((g.ny - ky) % g.ny - ky) * g.P : 0;   // 0: the row is its own pair
+  double* base = reinterpret_cast<double*>(spec + (long long)ky * g.P + kx) + (NR == 1 ? (lane & 1) : 0);
+  const double s = ms * -(lamx[kx] + lamy[ky]);
+  const double *pc = cf + up * nz, *qc = cf + (1 - up) * nz;   // couplings to the previous and the next level
+  const int n = up ? nz - 1 - m : m, dk = up ? -1 : 1;         // levels of this half, from k0 on
+  const int k0 = up ? nz - 1 : 0;
+  // before the first level: g/u = 1 and z = 0 (p is 0 below the bottom, the top face's coupling above the top)
+  double ratio = 1.0;
+  ColVals<NR> z, b;
+#pragma unroll
+  for (int r = 0; r < NR; ++r) z.v[r] = 0.0;
+  b.load(base + k0 * ld, second);   // the upper half of two levels has none of its own: level nz-1 = m, unused
+  for (int i = 0; i < m; ++i) {
+    const int k = k0 + i * dk;
+    ColVals<NR> bn;   // the next level (the last one read is level m or a neighbour of it)
+    bn.load(base + (long long)(k + dk) * ld, second);
+    if (i < n) {
+      const double q = qc[k];
+      const double gk = fma(pc[k], ratio, s);
+      const double inv = rcp_halley(gk + q);
+      const double e = ADJ ? (i ? qc[k - dk] : 0.0) : pc[k];
+      const double rr = ADJ ? pc[k + dk] : q;
+      ratio = gk * inv;
+      w[i * 32] = rr * inv;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) z.v[r] = fma(e, z.v[r], b.v[r]) * inv;
+      if (valid) z.store(base + k * ld, second);
+    }
+    b = bn;
+  }
+  // level m: both lanes of a column form the same sum
+  ColVals<NR> x;
+  x.load(base + m * ld, second);
+  {
+    const double own = pc[m] * ratio;
+    const double inv = rcp_halley(s + (own + __shfl_xor_sync(0xffffffffu, own, 16)));
+    const double e = ADJ ? (n ? qc[m - dk] : 0.0) : pc[m];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const double part = e * z.v[r];
+      x.v[r] = (x.v[r] + (part + __shfl_xor_sync(0xffffffffu, part, 16))) * inv;
+    }
+  }
+  __syncwarp();   // both lanes have read level m
+  if (valid && !up) x.store(base + m * ld, second);
+  ColVals<NR> zn;
+  if (n) z.load(base + (long long)(k0 + (n - 1) * dk) * ld, second);
+  for (int i = n - 1; i >= 0; --i) {
+    const int k = k0 + i * dk;
+    if (i) zn.load(base + (long long)(k - dk) * ld, second);
+    const double f = w[i * 32];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) x.v[r] = fma(f, x.v[r], z.v[r]);
+    if (valid) x.store(base + k * ld, second);
+    z = zn;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // launcher
 // ---------------------------------------------------------------------------
 // Columns per CTA: the requested width if its tile fits, else the largest of
@@ -453,6 +604,36 @@ static cudaError_t thomas_tw_launch(const ThomasArgs& A, const Geom& g, const Ta
                     A.kcut);
 }
 
+template <int NR, bool ADJ>
+static cudaError_t thomas_d_nr(const ThomasArgs& A, const Geom& g, const Tables& tb, long long lanes, cudaStream_t st) {
+  size_t smem = ((size_t)(g.nz / 2) * 32 + 2 * (size_t)g.nz) * sizeof(double);
+  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(double);
+  if (smem < lowk_smem) smem = lowk_smem;
+  auto kern = k_thomas_d<NR, ADJ>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const LowkArgs L{A.lowk_cols, A.n_lowk, tb.a_d, tb.c_d, tb.W_d, tb.lamx_d, tb.lamy_d, A.target_mean, A.scale,
+                   A.singular00, A.lowk_inv};
+  // Grids that fill the FP64 units take an ordinary launch: CTAs started while the y-pass drains would pile up on
+  // the SMs that finish first, and this kernel needs its warps spread evenly (256 x 256 x 64 solve: 226 us with
+  // the early launch, 162 without; 32 x 32 x 32: 34.6 with, 36.9 without).
+  const dim3 grid((unsigned)((lanes + 15) / 16 + A.n_lowk));
+  if (NR == 1)
+    return pdl_launch(kern, grid, dim3(32), smem, st, (double2*)A.spec, g, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d,
+                      A.lowk_r2, A.stats, L);
+  kern<<<grid, 32, smem, st>>>((double2*)A.spec, g, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, A.lowk_r2, A.stats, L);
+  return cudaGetLastError();
+}
+
+// Two columns a lane while that leaves a warp for each of the 608 FP64 units, then one column, then one part.
+template <bool ADJ>
+static cudaError_t thomas_d_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, cudaStream_t st) {
+  const long long pairs = (long long)(g.ny / 2 + 1) * g.nxh, cols = (long long)g.ny * g.nxh;
+  if (pairs >= 608 * 16) return thomas_d_nr<4, ADJ>(A, g, tb, pairs, st);
+  if (cols >= 608 * 16) return thomas_d_nr<2, ADJ>(A, g, tb, cols, st);
+  return thomas_d_nr<1, ADJ>(A, g, tb, 2 * cols, st);
+}
+
 template <typename T, typename TCm, bool ADJ>
 static cudaError_t thomas_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, const T* a, const T* c,
                                  const T* lx, const T* ly, cudaStream_t st) {
@@ -503,6 +684,8 @@ static cudaError_t thomas_launch(const ThomasArgs& A, const Geom& g, const Table
 }
 
 cudaError_t launch_thomas(const ThomasArgs& A, const Geom& g, const Tables& tb, cudaStream_t st) {
+  if (A.t_is_double && A.col_tile < 16 && !A.done)
+    return A.adjoint ? thomas_d_launch<true>(A, g, tb, st) : thomas_d_launch<false>(A, g, tb, st);
   if (A.t_is_double)
     return A.adjoint ? thomas_launch<double, double, true>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st)
                      : thomas_launch<double, double, false>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st);
