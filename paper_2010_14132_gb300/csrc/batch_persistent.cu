@@ -301,7 +301,7 @@ __device__ void item_x(const BDom& D, int type, int pass, int sub, unsigned char
   const long long rows = (long long)g.ny * g.nz;
   const long long r0 = (long long)sub * D.x_rows, r1 = min(rows, r0 + (long long)D.x_rows);
   float2* line = lines + (size_t)ty * LS;
-  const LineSync sync{1 + ty, nl};
+  const LineSyncT<nl> sync{1 + ty};
   const Swizzled sw{};
   const bool fwd = type == BP_XF0 || type == BP_XR;
   const bool has_q = pass > 1;

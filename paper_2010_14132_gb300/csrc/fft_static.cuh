@@ -65,13 +65,23 @@ template <int N, int E> __device__ __forceinline__ int st_out_index(int lane, in
   return lane + nl * (i / R) + (i % R) * Ns;
 }
 
-// Per-line barrier among the nl threads of a line.  Lines of at most 32 threads
-// live inside one warp; wider lines use a named barrier per line (ids 1..15).
-struct LineSync {
-  int id, nthreads;
+// Per-line barrier among the NL threads of a line: inside a warp, over whole warps (a named barrier per line, ids
+// 1..15), or, for lines that do not tile warps, the block's barrier (every line of the block then takes part).
+template <int NL> struct LineSyncT {
+  int id;
   __device__ __forceinline__ void operator()() const {
-    if (nthreads <= 32) __syncwarp();
-    else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+    if constexpr (NL <= 32 && 32 % NL == 0) __syncwarp();
+    else if constexpr (NL % 32 == 0) asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(NL) : "memory");
+    else __syncthreads();
+  }
+};
+
+// Slot of element idx of a line of N: swizzled where N is a multiple of 16 (the swizzle is a bijection within
+// blocks of 16), else plain: those lengths have a factor 3, and the first stage's stride of 3 already spreads.
+template <int N> struct LineAddr {
+  __device__ __forceinline__ int operator()(int idx) const {
+    if constexpr (N % 16 == 0) return idx ^ ((idx >> 4) & 15);
+    return idx;
   }
 };
 

@@ -281,16 +281,6 @@ __device__ __forceinline__ Fx2* fx_run_from(Fx2 (&v)[E], Fx2* cur, Fx2* nxt, Add
   }
 }
 
-// barrier of the threads that share one line of the x-pass: inside a warp, over whole warps, or the block
-template <int NL> struct FxLineSync {
-  int id;
-  __device__ __forceinline__ void operator()() const {
-    if constexpr (NL <= 32 && 32 % NL == 0) __syncwarp();
-    else if constexpr (NL % 32 == 0) asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(NL) : "memory");
-    else __syncthreads();
-  }
-};
-
 // opt a kernel in to its dynamic shared memory, once
 template <typename K> inline cudaError_t fx_allow_smem(K kernel, size_t bytes) {
   static std::mutex mu;

@@ -24,7 +24,7 @@ constexpr int fx_x_rows(int n) {   // rows per CTA: about 128 threads
 // shuffles; wider or odd ones through a shared word per line (zeroed before).
 template <int NL> struct FxLine {
   static constexpr bool kWarp = NL <= 32 && 32 % NL == 0;
-  static __device__ __forceinline__ int max_exp(int e, int* slot, FxLineSync<NL> sync) {
+  static __device__ __forceinline__ int max_exp(int e, int* slot, LineSyncT<NL> sync) {
     if constexpr (kWarp) {
 #pragma unroll
       for (int o = NL / 2; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xfwd_fx(cons
   const int lane = threadIdx.x, ty = threadIdx.y;
   const long long row = (long long)g.lev0 * g.ny + (long long)blockIdx.x * RB + ty;
   const bool valid = row < (long long)g.lev1 * g.ny;
-  const FxLineSync<nl> sync{1 + ty};
+  const LineSyncT<nl> sync{1 + ty};
   const Swizzled16 sw{};
   Fx2* la = lines + (size_t)ty * 2 * LS;
   if (lane == 0) {
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xinv_fx(cons
   const int lane = threadIdx.x, ty = threadIdx.y;
   const long long row = (long long)g.lev0 * g.ny + (long long)blockIdx.x * RB + ty;
   const bool valid = row < (long long)g.lev1 * g.ny;
-  const FxLineSync<nl> sync{1 + ty};
+  const LineSyncT<nl> sync{1 + ty};
   const Swizzled16 sw{};
   Fx2* la = lines + (size_t)ty * 2 * LS;
   if (lane == 0) {

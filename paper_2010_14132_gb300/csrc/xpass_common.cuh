@@ -1,4 +1,4 @@
-// Persistent x-pass kernels for FP32 transforms of power-of-two half lengths
+// Persistent x-pass kernels for FP32 transforms of half lengths 2^a 3^b (the list in PGB_XS_N_SWITCH)
 // (Section 2.1: the x transform of every row of every level).
 //
 // One CTA per SM slot walks groups of RB consecutive rows.  Each group's input
@@ -34,9 +34,12 @@
 namespace pgb {
 namespace {
 
-// CTA size: 256 threads with 8 elements per thread, 128 with 16 (one warp per
+// CTA size: at most 256 threads with 8 or 12 elements per thread, 128 with 16 (one warp per
 // 512-point line); with 16 elements the FFT runs radix-16 stages.
-__host__ __device__ constexpr int xs_threads(int E) { return E >= 16 ? 128 : 256; }
+__host__ __device__ constexpr int xs_max_threads(int E) { return E >= 16 ? 128 : 256; }
+// rows per CTA and threads of a CTA for lines of N packed points
+__host__ __device__ constexpr int xs_rows(int N, int E) { return xs_max_threads(E) / (N / E); }
+__host__ __device__ constexpr int xs_threads(int N, int E) { return xs_rows(N, E) * (N / E); }
 constexpr int kXsMaxStages = 4;
 
 template <typename T> struct V2s;
@@ -58,7 +61,7 @@ struct XsLayout {
 __host__ __device__ constexpr size_t xs_align(size_t x, size_t a) { return (x + a - 1) / a * a; }
 __host__ __device__ inline XsLayout xs_layout(int N, int RB, int ns, unsigned stage_bytes, bool alias) {
   XsLayout L{};
-  size_t off = (size_t)N * 8 + (size_t)(N + 2) * 8 + (alias ? 0 : (size_t)RB * 2 * swizzled_stride(N) * 8);
+  size_t off = (size_t)N * 8 + (size_t)(N + 2) * 8 + (alias ? 0 : (size_t)RB * 2 * N * 8);
   L.off_stage = xs_align(off, 128);
   L.off_bar = xs_align(L.off_stage + (size_t)ns * stage_bytes, 8);
   L.total = L.off_bar + (size_t)ns * 8;
@@ -84,7 +87,7 @@ __device__ __forceinline__ void r2c_unpack_store(const float2* fin, const float2
                                                  bool valid, int kmax = N) {
   using C = float2;
   constexpr int nl = N / E;
-  const Swizzled sw{};
+  const LineAddr<N> sw{};
 #pragma unroll
   for (int q = 0; q < E / 2; ++q) {
     const int k = lane + nl * q;   // k < N/2
@@ -136,7 +139,7 @@ struct XsConfig {
 // shared memory still allows two stages, then the deepest ring (up to four
 // stages) at that CTA count.
 XsConfig xs_config(int N, int E, unsigned stage_bytes, size_t static_smem, bool alias) {
-  const int RB = xs_threads(E) / (N / E);
+  const int RB = xs_rows(N, E);
   constexpr size_t kSmPerSm = 228 * 1024, kReserved = 1024, kMaxPerCta = 227 * 1024;
   XsConfig c{};
   c.stage_bytes = stage_bytes;
@@ -189,25 +192,28 @@ inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? kE3 : (plan_e == 16
     constexpr int EE = 8;                                       \
     __VA_ARGS__;                                                \
   }
-#define PGB_XS_E8_E3_SWITCH(E, ...)                             \
-  if ((E) == kE3) {                                             \
-    constexpr int EE = kE3;                                     \
-    __VA_ARGS__;                                                \
-  } else {                                                      \
-    constexpr int EE = 8;                                       \
-    __VA_ARGS__;                                                \
-  }
 #define PGB_XS_N_CASE(V, ...) \
   case V: { constexpr int NN = V; if constexpr (st_valid(NN, EE)) { __VA_ARGS__; } } break;
+// Half lengths with compile-time kernels.  The ones with factors 9, 27 and 81 ran the run-time engine (24 elements
+// and 190 registers a thread, index arithmetic by division): 432 x 324 x 37 in FP32, x 42 -> 22 us, inverse x
+// 40 -> 22, and the y-pass of 324 points 24 -> 17.
 #define PGB_XS_N_SWITCH(N, ...)                          \
   switch (N) {                                           \
     PGB_XS_N_CASE(32, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(36, __VA_ARGS__)                       \
     PGB_XS_N_CASE(64, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(72, __VA_ARGS__)                       \
     PGB_XS_N_CASE(96, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(108, __VA_ARGS__)                      \
     PGB_XS_N_CASE(128, __VA_ARGS__)                      \
+    PGB_XS_N_CASE(144, __VA_ARGS__)                      \
     PGB_XS_N_CASE(192, __VA_ARGS__)                      \
+    PGB_XS_N_CASE(216, __VA_ARGS__)                      \
     PGB_XS_N_CASE(256, __VA_ARGS__)                      \
+    PGB_XS_N_CASE(288, __VA_ARGS__)                      \
+    PGB_XS_N_CASE(324, __VA_ARGS__)                      \
     PGB_XS_N_CASE(384, __VA_ARGS__)                      \
+    PGB_XS_N_CASE(432, __VA_ARGS__)                      \
     PGB_XS_N_CASE(512, __VA_ARGS__)                      \
     PGB_XS_N_CASE(768, __VA_ARGS__)                      \
     PGB_XS_N_CASE(1024, __VA_ARGS__)                     \

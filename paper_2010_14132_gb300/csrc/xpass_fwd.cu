@@ -10,13 +10,13 @@ namespace {
 // forward x-pass
 // ---------------------------------------------------------------------------
 template <int N, int E, typename TI>
-__global__ void __launch_bounds__(xs_threads(E)) k_xfwd_s(const TI* __restrict__ in, float2* __restrict__ spec, Geom g,
+__global__ void __launch_bounds__(xs_max_threads(E)) k_xfwd_s(const TI* __restrict__ in, float2* __restrict__ spec, Geom g,
                                                       const float2* __restrict__ twx, const float2* __restrict__ twr,
                                                       const int* __restrict__ done, unsigned* __restrict__ err,
                                                       int ns, unsigned stage_bytes) {
   using C = float2;
   using TI2 = typename V2s<TI>::t;
-  constexpr int nl = N / E, RB = xs_threads(E) / nl, LS = swizzled_stride(N);
+  constexpr int nl = N / E, RB = xs_rows(N, E), LS = N;
   constexpr bool ALIAS = sizeof(TI) == 8;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -31,8 +31,8 @@ __global__ void __launch_bounds__(xs_threads(E)) k_xfwd_s(const TI* __restrict__
   const long long row_begin = (long long)g.lev0 * g.ny, row_end = (long long)g.lev1 * g.ny;
   const long long ngroups = (row_end - row_begin + RB - 1) / RB;
   constexpr unsigned row_bytes = (unsigned)(2 * N * sizeof(TI));
-  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(E));
-  for (int t = tid; t <= N / 2; t += xs_threads(E)) twr_s[t] = twr[t];
+  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(N, E));
+  for (int t = tid; t <= N / 2; t += xs_threads(N, E)) twr_s[t] = twr[t];
   Ring rg{};
   if (tid == 0) {
     for (int s = 0; s < ns; ++s) mbar_init(&bar[s], 1);
@@ -54,8 +54,8 @@ __global__ void __launch_bounds__(xs_threads(E)) k_xfwd_s(const TI* __restrict__
       const long long grp = blockIdx.x + (long long)s * gridDim.x;
       if (grp < ngroups) issue(grp, s);
     }
-  const LineSync sync{1 + ty, nl};
-  const Swizzled sw{};
+  const LineSyncT<nl> sync{1 + ty};
+  const LineAddr<N> sw{};
   C* la = lines + (size_t)ty * 2 * LS;
   C* lb = la + LS;
   bool ok = true;
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(xs_threads(E)) k_xfwd_s(const TI* __restrict__
 template <typename TI>
 cudaError_t xfwd_s(const TI* in, float2* spec, const Geom& g, int N, int E, const Tables& tb, const int* done,
                    unsigned* err, cudaStream_t st, bool* used) {
-  const int RB = xs_threads(E) / (N / E);
+  const int RB = xs_rows(N, E);
   const unsigned row_bytes = (unsigned)(g.nx * sizeof(TI));
   const XsConfig c = xs_config(N, E, RB * row_bytes, 0, sizeof(TI) == 8);
   if (c.ns == 0 || !aligned16(in) || row_bytes % 16) return cudaSuccess;

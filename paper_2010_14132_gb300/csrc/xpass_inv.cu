@@ -20,11 +20,11 @@ namespace {
 #endif
 constexpr int xinv_min_blocks(int e) { return e % 3 == 0 ? PGB_XINV_E3_BLOCKS : PGB_XINV_MIN_BLOCKS; }
 template <int N, int E, typename TO, int MODE>
-__global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(const float2* __restrict__ spec, TO* __restrict__ out, Geom g,
+__global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_s(const float2* __restrict__ spec, TO* __restrict__ out, Geom g,
                                                       const float2* __restrict__ twx, const float2* __restrict__ twr,
                                                       XinvExtra ex, int ns, unsigned stage_bytes) {
   using C = float2;
-  constexpr int nl = N / E, RB = xs_threads(E) / nl, LS = swizzled_stride(N);
+  constexpr int nl = N / E, RB = xs_rows(N, E), LS = N;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
   const XsLayout L = xs_layout(N, RB, ns, stage_bytes, false);
@@ -38,8 +38,8 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
   const long long row_begin = (long long)g.lev0 * g.ny, row_end = (long long)g.lev1 * g.ny;
   const long long ngroups = (row_end - row_begin + RB - 1) / RB;
   const unsigned row_bytes = (unsigned)xs_align((size_t)(N + 1) * sizeof(C), 16);
-  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(E));
-  for (int t = tid; t <= N; t += xs_threads(E)) twr_s[t] = twr[t];
+  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(N, E));
+  for (int t = tid; t <= N; t += xs_threads(N, E)) twr_s[t] = twr[t];
   Ring rg{};
   if (tid == 0) {
     for (int s = 0; s < ns; ++s) mbar_init(&bar[s], 1);
@@ -61,8 +61,8 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
       const long long grp = blockIdx.x + (long long)s * gridDim.x;
       if (grp < ngroups) issue(grp, s);
     }
-  const LineSync sync{1 + ty, nl};
-  const Swizzled sw{};
+  const LineSyncT<nl> sync{1 + ty};
+  const LineAddr<N> sw{};
   C* la = lines + (size_t)ty * 2 * LS;
   C* lb = la + LS;
   // per-lane partial sums (even / odd points): delta^2, p^2 and the double-float sum of p
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
   if constexpr (MODE != XINV_PLAIN) {
     // deterministic CTA partial sums: fixed-order tree over the CTA's threads, in the
     // line buffers (no longer in use: every thread is past its last transform)
-    constexpr int TH = xs_threads(E);
+    constexpr int TH = xs_threads(N, E);
     static_assert((size_t)TH * 40 <= (size_t)RB * 2 * LS * sizeof(C), "reduction does not fit the line buffers");
     __syncthreads();
     double* redd = reinterpret_cast<double*>(lines);
@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
     red[1][tid] = acc1.x + acc1.y;
     redd[tid] = (f2d_int(sh.x) + f2d_int(sl.x)) + (f2d_int(sh.y) + f2d_int(sl.y));
     __syncthreads();
-    for (int h = xs_threads(E) / 2; h > 0; h >>= 1) {
-      if (tid < h) {
+    for (int h = xs_max_threads(E) / 2; h > 0; h >>= 1) {
+      if (tid < h && tid + h < TH) {
         red[0][tid] += red[0][tid + h];
         red[1][tid] += red[1][tid + h];
         redd[tid] += redd[tid + h];
@@ -209,8 +209,8 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
       sums[3 * TH + tid] = a3;
       sums[4 * TH + tid] = a4;
       __syncthreads();
-      for (int h = TH / 2; h > 0; h >>= 1) {
-        if (tid < h) {
+      for (int h = xs_max_threads(E) / 2; h > 0; h >>= 1) {
+        if (tid < h && tid + h < TH) {
 #pragma unroll
           for (int v = 0; v < 5; ++v) sums[v * TH + tid] += sums[v * TH + tid + h];
         }
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(xs_threads(E), xinv_min_blocks(E)) k_xinv_s(co
 template <typename TO, int MODE>
 cudaError_t xinv_s(const float2* spec, TO* out, const Geom& g, int N, int E, const Tables& tb, const XinvExtra& ex,
                    int* nblocks_out, cudaStream_t st, bool* used) {
-  const int RB = xs_threads(E) / (N / E);
+  const int RB = xs_rows(N, E);
   const unsigned row_bytes = (unsigned)xs_align((size_t)(N + 1) * sizeof(float2), 16);
   if ((size_t)g.P * sizeof(float2) < row_bytes || (g.P * sizeof(float2)) % 16 || !aligned16(spec)) return cudaSuccess;
   const XsConfig c = xs_config(N, E, RB * row_bytes, 0, false);
@@ -245,7 +245,8 @@ cudaError_t xinv_s(const float2* spec, TO* out, const Geom& g, int N, int E, con
 
 bool xpass_static_supported(int n_half) {
   switch (n_half) {
-    case 32: case 64: case 96: case 128: case 192: case 256: case 384: case 512: case 768: case 1024: case 2048:
+    case 32: case 64: case 128: case 256: case 512: case 1024: case 2048:
+    case 36: case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 768:
       return true;
     default: return false;
   }

@@ -3,10 +3,14 @@
 // for the persistent staging scheme the kernels share.)
 #include "xpass_common.cuh"
 
-// This file is compiled twice: PGB_XRES_ISO 0 here (the general kernels and the dispatcher), and 1
-// from xpass_res_iso.cu (the dx == dy kernels), so that the two sets of instances build in parallel.
+// This file is compiled four times, so that the sets of instances build in parallel: PGB_XRES_ISO 0 and
+// PGB_XRES_E 8 here (the general kernels of power-of-two lines, and the dispatcher), PGB_XRES_ISO 1 from
+// the _iso files (dx == dy), PGB_XRES_E 12 from the xpass_res3 files (lines with a factor 3).
 #ifndef PGB_XRES_ISO
 #define PGB_XRES_ISO 0
+#endif
+#ifndef PGB_XRES_E
+#define PGB_XRES_E 8
 #endif
 
 namespace pgb {
@@ -34,12 +38,12 @@ constexpr int xres_min_blocks(int e, bool has_q, bool from_r0 = false) {
 // copy each per row, side by side in the row's slot, whose full width the line buffers need later) and
 // r = r0 - L q.
 template <int N, int E, bool HAS_Q, bool STAGE_P, bool ISO, bool FROM_R0 = false>
-__global__ void __launch_bounds__(xs_threads(E), xres_min_blocks(E, HAS_Q, FROM_R0)) k_xres_s(ResidualArgs R, float2* __restrict__ spec, Geom g,
+__global__ void __launch_bounds__(xs_max_threads(E), xres_min_blocks(E, HAS_Q, FROM_R0)) k_xres_s(ResidualArgs R, float2* __restrict__ spec, Geom g,
                                                       const float2* __restrict__ twx, const float2* __restrict__ twr,
                                                       const int* __restrict__ done, unsigned* __restrict__ err,
                                                       int ns, unsigned stage_bytes) {
   using C = float2;
-  constexpr int nl = N / E, RB = xs_threads(E) / nl, LS = swizzled_stride(N), NX = 2 * N;
+  constexpr int nl = N / E, RB = xs_rows(N, E), LS = N, NX = 2 * N;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
   const XsLayout L = xs_layout(N, RB, ns, stage_bytes, true);
@@ -53,8 +57,8 @@ __global__ void __launch_bounds__(xs_threads(E), xres_min_blocks(E, HAS_Q, FROM_
   const long long row_begin = (long long)g.lev0 * g.ny, row_end = (long long)g.lev1 * g.ny;
   const long long ngroups = (row_end - row_begin + RB - 1) / RB;
   constexpr unsigned s_bytes = RB * NX * 8, p_bytes = STAGE_P ? RB * NX * 4 : 0;
-  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(E));
-  for (int t = tid; t <= N / 2; t += xs_threads(E)) twr_s[t] = twr[t];
+  st_build_twiddles<N, E>(tw_s, twx, tid, xs_threads(N, E));
+  for (int t = tid; t <= N / 2; t += xs_threads(N, E)) twr_s[t] = twr[t];
   Ring rg{};
   if (tid == 0) {
     for (int s = 0; s < ns; ++s) mbar_init(&bar[s], 1);
@@ -90,8 +94,8 @@ __global__ void __launch_bounds__(xs_threads(E), xres_min_blocks(E, HAS_Q, FROM_
       const long long grp = blockIdx.x + (long long)s * gridDim.x;
       if (grp < ngroups) issue(grp, s);
     }
-  const LineSync sync{1 + ty, nl};
-  const Swizzled sw{};
+  const LineSyncT<nl> sync{1 + ty};
+  const LineAddr<N> sw{};
   (void)lines;
   const float2 cx = R.cx, cy = R.cy;   // double-float splits of 1/dx^2, 1/dy^2
   float2 racc = make_float2(0.f, 0.f), sacc = racc;   // per-lane sums of r^2 and S^2 (even / odd points)
@@ -215,15 +219,15 @@ __global__ void __launch_bounds__(xs_threads(E), xres_min_blocks(E, HAS_Q, FROM_
     ring_drain(rg, bar, ns);
   }
   // per-CTA sums of r^2 and S^2 (fixed-order tree) in the drained staging ring
-  constexpr int TH = xs_threads(E);
+  constexpr int TH = xs_threads(N, E);
   static_assert((size_t)TH * 8 <= (size_t)RB * NX * 8, "reduction does not fit the staging ring");
   __syncthreads();
   float (*red)[TH] = reinterpret_cast<float (*)[TH]>(stg);
   red[0][tid] = racc.x + racc.y;
   red[1][tid] = sacc.x + sacc.y;
   __syncthreads();
-  for (int h = TH / 2; h > 0; h >>= 1) {
-    if (tid < h) {
+  for (int h = xs_max_threads(E) / 2; h > 0; h >>= 1) {
+    if (tid < h && tid + h < TH) {
       red[0][tid] += red[0][tid + h];
       red[1][tid] += red[1][tid + h];
     }
@@ -236,15 +240,22 @@ __global__ void __launch_bounds__(xs_threads(E), xres_min_blocks(E, HAS_Q, FROM_
   }
 }
 
+// the lines of this compilation's element count
+#define PGB_XRES_SWITCH(N, ...)         \
+  {                                     \
+    constexpr int EE = PGB_XRES_E;      \
+    PGB_XS_N_SWITCH(N, __VA_ARGS__)     \
+  }
+
 template <bool HAS_Q, bool ISO>
 cudaError_t xres_s(const ResidualArgs& R, float2* spec, const Geom& g, int N, int E, const Tables& tb,
                    const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used) {
-  const int RB = xs_threads(E) / (N / E);
+  const int RB = xs_rows(N, E);
   // stage S, p0 (and q) rows while three CTAs per SM still fit, else S rows only
   const unsigned row_bytes_all = (unsigned)(g.nx * (8 + 4 + (HAS_Q ? 4 : 0)));
   const unsigned row_bytes_s = (unsigned)(g.nx * 8);
   const XsConfig c_all = xs_config(N, E, RB * row_bytes_all, 0, true);
-  const bool stage_p = c_all.ns > 0 && c_all.smem <= 75 * 1024 * (size_t)xs_threads(E) / 256;
+  const bool stage_p = c_all.ns > 0 && c_all.smem <= 75 * 1024 * (size_t)xs_max_threads(E) / 256;
   const XsConfig c = stage_p ? c_all : xs_config(N, E, RB * row_bytes_s, 0, true);
   const long long ngroups = ((long long)g.ny * (g.lev1 - g.lev0) + RB - 1) / RB;
   if constexpr (HAS_Q) {
@@ -253,54 +264,59 @@ cudaError_t xres_s(const ResidualArgs& R, float2* spec, const Geom& g, int N, in
       if (c0.ns == 0 || !aligned16(R.r0) || (R.r_ld * 4) % 16 || !aligned16(R.p0) || !aligned16(R.q) ||
           (g.nx * 4) % 16)
         return cudaSuccess;
-      PGB_XS_E8_E3_SWITCH(E, PGB_XS_N_SWITCH(N, {
+      PGB_XRES_SWITCH(N, {
         return xs_launch(k_xres_s<NN, EE, true, false, ISO, true>, NN / EE, RB, c0, ngroups, nblocks_out, st, used,
                          R, spec, g, tb.twx_f, tb.twr_f, done, err);
-      }));
+      });
       return cudaSuccess;
     }
   }
   if (c.ns == 0 || !aligned16(R.S) || !aligned16(R.p0) || (HAS_Q && !aligned16(R.q)) || (g.nx * 4) % 16)
     return cudaSuccess;
   if (stage_p) {
-    PGB_XS_E8_E3_SWITCH(E, PGB_XS_N_SWITCH(N, {
+    PGB_XRES_SWITCH(N, {
       return xs_launch(k_xres_s<NN, EE, HAS_Q, true, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
                        tb.twx_f, tb.twr_f, done, err);
-    }));
+    });
   } else {
-    PGB_XS_E8_E3_SWITCH(E, PGB_XS_N_SWITCH(N, {
+    PGB_XRES_SWITCH(N, {
       return xs_launch(k_xres_s<NN, EE, HAS_Q, false, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
                        tb.twx_f, tb.twr_f, done, err);
-    }));
+    });
   }
   return cudaSuccess;
 }
 
 }  // namespace
 
+static_assert(kE3 == 12, "the xpass_res3 files build the kernels of kE3 elements");
+#define PGB_XRES_ENTRY(NAME)                                                                                       \
+  cudaError_t NAME(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,            \
+                   const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used)
+PGB_XRES_ENTRY(launch_xres8);
+PGB_XRES_ENTRY(launch_xres8_iso);
+PGB_XRES_ENTRY(launch_xres12);
+PGB_XRES_ENTRY(launch_xres12_iso);
+#define PGB_XRES_CAT2(a, b) a##b
+#define PGB_XRES_CAT(a, b) PGB_XRES_CAT2(a, b)
 #if PGB_XRES_ISO
-cudaError_t launch_xres_static_iso(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx,
-                                   const Tables& tb, const int* done, unsigned* err, int* nblocks_out,
-                                   cudaStream_t st, bool* used) {
-  const int E = fx.n % 3 == 0 ? kE3 : 8;
-  if (R.q) return xres_s<true, true>(R, (float2*)spec, g, fx.n, E, tb, done, err, nblocks_out, st, used);
-  return xres_s<false, true>(R, (float2*)spec, g, fx.n, E, tb, done, err, nblocks_out, st, used);
-}
+PGB_XRES_ENTRY(PGB_XRES_CAT(PGB_XRES_CAT(launch_xres, PGB_XRES_E), _iso)) {
 #else
-cudaError_t launch_xres_static_iso(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx,
-                                   const Tables& tb, const int* done, unsigned* err, int* nblocks_out,
-                                   cudaStream_t st, bool* used);
+PGB_XRES_ENTRY(PGB_XRES_CAT(launch_xres, PGB_XRES_E)) {
+#endif
+  if (R.q)
+    return xres_s<true, PGB_XRES_ISO != 0>(R, (float2*)spec, g, fx.n, PGB_XRES_E, tb, done, err, nblocks_out, st, used);
+  return xres_s<false, PGB_XRES_ISO != 0>(R, (float2*)spec, g, fx.n, PGB_XRES_E, tb, done, err, nblocks_out, st, used);
+}
 
-cudaError_t launch_xres_static(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
-                               const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used) {
+#if !PGB_XRES_ISO && PGB_XRES_E == 8
+PGB_XRES_ENTRY(launch_xres_static) {
   *used = false;
   if (!xpass_static_supported(fx.n)) return cudaSuccess;
-  const int E = fx.n % 3 == 0 ? kE3 : 8;   // the residual kernel: 8 elements per thread for powers of two
   // dx == dy: the kernels with the merged horizontal term
-  if (R.cx.x == R.cy.x && R.cx.y == R.cy.y)
-    return launch_xres_static_iso(R, spec, g, fx, tb, done, err, nblocks_out, st, used);
-  if (R.q) return xres_s<true, false>(R, (float2*)spec, g, fx.n, E, tb, done, err, nblocks_out, st, used);
-  return xres_s<false, false>(R, (float2*)spec, g, fx.n, E, tb, done, err, nblocks_out, st, used);
+  const bool iso = R.cx.x == R.cy.x && R.cx.y == R.cy.y, three = fx.n % 3 == 0;
+  auto launch = three ? (iso ? launch_xres12_iso : launch_xres12) : (iso ? launch_xres8_iso : launch_xres8);
+  return launch(R, spec, g, fx, tb, done, err, nblocks_out, st, used);
 }
 #endif
 

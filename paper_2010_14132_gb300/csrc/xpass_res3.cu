@@ -1,0 +1,3 @@
+// Residual x-pass kernels for lines with a factor 3 (see xpass_res.cu).
+#define PGB_XRES_E 12
+#include "xpass_res.cu"

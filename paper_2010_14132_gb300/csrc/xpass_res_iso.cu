@@ -1,4 +1,3 @@
-// The dx == dy instances of the sweep's residual x-pass (see xpass_res.cu), in a
-// translation unit of their own so that they compile in parallel with the others.
+// Residual x-pass kernels for dx == dy, lines of powers of two (see xpass_res.cu).
 #define PGB_XRES_ISO 1
 #include "xpass_res.cu"

@@ -1,4 +1,4 @@
-// Persistent FP32 y-pass for power-of-two ny in [64, 2048] (Section 2.1: the
+// Persistent FP32 y-pass for ny = 2^a 3^b in [64, 2048] (the list in PGB_YS_N_SWITCH; Section 2.1: the
 // transform along y of every kx column of every level).
 //
 // A tile is one level and TK consecutive kx columns: ny rows of TK complex
@@ -23,9 +23,9 @@ namespace {
 
 // Column-interleaved tile addressing with the complex index swizzled inside
 // blocks of 16 (spreads the stride-R first-stage writes over the banks).
-struct SwStrided {
+template <int N> struct SwStrided {
   int es;
-  __device__ __forceinline__ int operator()(int idx) const { return (idx ^ ((idx >> 4) & 15)) * es; }
+  __device__ __forceinline__ int operator()(int idx) const { return LineAddr<N>{}(idx) * es; }
 };
 struct Plain {
   int es;
@@ -39,8 +39,9 @@ size_t ys_smem(int N, int TK, bool inplace) {
 
 constexpr int ys_max_threads(int E) { return E >= 16 || E % 3 == 0 ? 512 : 1024; }
 // the single-buffered kernel runs two CTAs per SM: 256 threads for the 12-element lengths keeps
-// their registers (128) free of spills
-constexpr int ys1_max_threads(int E) { return E % 3 == 0 ? 256 : ys_max_threads(E); }
+// their registers (128) free of spills (288 for 864 points, whose 72 threads a column would leave only two
+// columns otherwise)
+constexpr int ys1_max_threads(int N, int E) { return E % 3 == 0 ? (N == 864 ? 288 : 256) : ys_max_threads(E); }
 
 template <int N, int E, int SIGN, bool INPLACE>
 __global__ void __launch_bounds__(ys_max_threads(E)) k_ys(const __grid_constant__ CUtensorMap tm, Geom g,
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(ys_max_threads(E)) k_ys(const __grid_constant_
     if (t0 < ntiles) issue(t0, 0);
     if (t0 + (int)gridDim.x < ntiles) issue(t0 + gridDim.x, 1);
   }
-  const SwStrided sw{TK};
+  const SwStrided<N> sw{TK};
   bool ok = true;
   int it = 0;
   for (int t = t0; t < ntiles; t += gridDim.x, ++it) {
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(ys_max_threads(E)) k_ys(const __grid_constant_
 // The next tile's load is issued as soon as the transform has finished reading the
 // tile (its outputs are in registers), so it also overlaps this tile's stores.
 template <int N, int E, int SIGN>
-__global__ void __launch_bounds__(ys1_max_threads(E), 2) k_ys1(const __grid_constant__ CUtensorMap tm, Geom g,
+__global__ void __launch_bounds__(ys1_max_threads(N, E), 2) k_ys1(const __grid_constant__ CUtensorMap tm, Geom g,
                                                              const float2* __restrict__ twy,
                                                              float2* __restrict__ spec, int box_rows,
                                                              int tiles_per_level, int ntiles,
@@ -156,7 +157,7 @@ __global__ void __launch_bounds__(ys1_max_threads(E), 2) k_ys1(const __grid_cons
   __syncthreads();
   pdl_wait();   // the previous kernels of the stream are complete
   if (done && *done) return;
-  const SwStrided sw{TK};
+  const SwStrided<N> sw{TK};
   int it = 0, pending = 0;
   bool ok = true;
   auto issue = [&](int tt) {
@@ -209,13 +210,22 @@ int largest_divisor_upto(int n, int cap) {
 #define PGB_YS_N_SWITCH(N, ...)        \
   switch (N) {                         \
     PGB_YS_N_CASE(64, __VA_ARGS__)     \
+    PGB_YS_N_CASE(72, __VA_ARGS__)     \
     PGB_YS_N_CASE(96, __VA_ARGS__)     \
+    PGB_YS_N_CASE(108, __VA_ARGS__)    \
     PGB_YS_N_CASE(128, __VA_ARGS__)    \
+    PGB_YS_N_CASE(144, __VA_ARGS__)    \
     PGB_YS_N_CASE(192, __VA_ARGS__)    \
+    PGB_YS_N_CASE(216, __VA_ARGS__)    \
     PGB_YS_N_CASE(256, __VA_ARGS__)    \
+    PGB_YS_N_CASE(288, __VA_ARGS__)    \
+    PGB_YS_N_CASE(324, __VA_ARGS__)    \
     PGB_YS_N_CASE(384, __VA_ARGS__)    \
+    PGB_YS_N_CASE(432, __VA_ARGS__)    \
     PGB_YS_N_CASE(512, __VA_ARGS__)    \
+    PGB_YS_N_CASE(576, __VA_ARGS__)    \
     PGB_YS_N_CASE(768, __VA_ARGS__)    \
+    PGB_YS_N_CASE(864, __VA_ARGS__)    \
     PGB_YS_N_CASE(1024, __VA_ARGS__)   \
     PGB_YS_N_CASE(1536, __VA_ARGS__)   \
     PGB_YS_N_CASE(2048, __VA_ARGS__)   \
@@ -275,7 +285,7 @@ cudaError_t ys1_launch(float2* spec, const Geom& g, int N, const float2* twy, in
                        cudaStream_t st, bool* used) {
   const size_t smem = ys_tile_bytes(N, tk) + (size_t)N * sizeof(float2) + 64;
   const int nthreads = tk * (N / E);
-  if (smem > 110 * 1024 || nthreads > ys1_max_threads(E) || nthreads < 32) return cudaSuccess;
+  if (smem > 110 * 1024 || nthreads > ys1_max_threads(N, E) || nthreads < 32) return cudaSuccess;
   const int box_rows = largest_divisor_upto(N, 256);
   if (((size_t)box_rows * tk * sizeof(float2)) % 128 != 0 && box_rows != N) return cudaSuccess;
   CUtensorMap tm;
@@ -311,7 +321,9 @@ cudaError_t ys1_launch(float2* spec, const Geom& g, int N, const float2* twy, in
 
 bool ypass_static_supported(int ny) {
   switch (ny) {
-    case 64: case 96: case 128: case 192: case 256: case 384: case 512: case 768: case 1024: case 1536: case 2048:
+    case 64: case 128: case 256: case 512: case 1024: case 2048:
+    case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 576: case 768:
+    case 864: case 1536:
       return true;
     default: return false;
   }
@@ -327,7 +339,7 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   const int E = fy.n % 3 == 0 ? kE3 : (fy.E == 16 ? 16 : 8);
   if (variant == 2 && (E == 16 || E == kE3)) {   // single-buffered, in place, two CTAs per SM
     int tk1 = tk;
-    while (tk1 > 2 && tk1 * (fy.n / E) > ys1_max_threads(E)) tk1 >>= 1;
+    while (tk1 > 2 && tk1 * (fy.n / E) > ys1_max_threads(fy.n, E)) tk1 >>= 1;
     float2* sp = (float2*)spec;
     cudaError_t e;
     if (E == 16)
