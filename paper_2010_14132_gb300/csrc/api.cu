@@ -211,8 +211,9 @@ void layout_workspace(poisson_plan* pl) {
   off = align256(off + pl->stats_bytes);
   pl->off_part = off;
   off = align256(off + 3 * sizeof(double) * (size_t)(pl->xinv_blocks + pl->nz));   // + one per level chunk
-  pl->off_rpart = off;
-  off = align256(off + 2 * sizeof(double) * (size_t)(pl->xinv_blocks + pl->nz));
+  pl->off_rpart = off;   // residual norms: per row group of the tiled kernel, or as above
+  off = align256(off + 2 * sizeof(double) *
+                           (size_t)std::max(pl->xinv_blocks + pl->nz, xres_tile_groups(pl->ny, pl->nz, pl->nx / 2)));
   pl->off_sqn = off;   // per-CTA squared norms of a verification solve (column tiles of >= 16 columns)
   off = align256(off + sizeof(double) * (size_t)(pl->g.plane / 16 + 1 + pl->n_lowk));
   pl->off_lz = off;
@@ -702,7 +703,9 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
       }
       bool stat = false;
       if (e == cudaSuccess && !used && pl->xkernel == 0) {
-        e = launch_xres_static(Rc, spec, gc, pl->fx, pl->tb, done, &stats->err, &nb, st, &used);
+        e = launch_xres_tile(Rc, spec, gc, pl->fx, pl->tb, done, &stats->err, &nb, st, &used);
+        if (e == cudaSuccess && !used)
+          e = launch_xres_static(Rc, spec, gc, pl->fx, pl->tb, done, &stats->err, &nb, st, &used);
         stat = used;
       }
       if (Rc.r0 && !stat) return cudaErrorNotSupported;   // the r0 - L q form exists in the static pass only

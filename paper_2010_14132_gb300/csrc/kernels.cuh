@@ -426,6 +426,10 @@ cudaError_t launch_grho(int kind /*0 double, 1 float, 2 double fields float math
 bool xpass_static_supported(int n_half);
 cudaError_t launch_xfwd_static(int ti_is_double, const void* in, void* spec, const Geom& g, const FftPlan& fx,
                                const Tables& tb, const int* done, unsigned* err, cudaStream_t st, bool* used);
+cudaError_t launch_xres_tile(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
+                             const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used);
+// Row groups of that kernel over all levels (0: lines it does not take), an upper bound of its partial sums.
+int xres_tile_groups(int ny, int nz, int n_half);
 cudaError_t launch_xres_static(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
                                const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used);
 cudaError_t launch_xinv_static(int to_is_double, int mode, const void* spec, void* out, const Geom& g,

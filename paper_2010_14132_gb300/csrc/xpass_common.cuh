@@ -34,6 +34,11 @@
 namespace pgb {
 namespace {
 
+// Rows per CTA of the residual kernels that stage every stencil row (xpass_res_tile.cu), about 128 threads; lines
+// that leave fewer than two (1024 packed points and more) take the kernels that read neighbour rows through L2.
+__host__ __device__ constexpr int xrt_rows(int n) { return 128 / (n / (n % 3 == 0 ? kE3 : 8)); }
+__host__ __device__ constexpr bool xrt_length(int n) { return xrt_rows(n) >= 2; }
+
 // CTA size: at most 256 threads with 8 or 12 elements per thread, 128 with 16 (one warp per
 // 512-point line); with 16 elements the FFT runs radix-16 stages.
 __host__ __device__ constexpr int xs_max_threads(int E) { return E >= 16 ? 128 : 256; }

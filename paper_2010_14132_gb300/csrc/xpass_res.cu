@@ -265,8 +265,9 @@ cudaError_t xres_s(const ResidualArgs& R, float2* spec, const Geom& g, int N, in
           (g.nx * 4) % 16)
         return cudaSuccess;
       PGB_XRES_SWITCH(N, {
-        return xs_launch(k_xres_s<NN, EE, true, false, ISO, true>, NN / EE, RB, c0, ngroups, nblocks_out, st, used,
-                         R, spec, g, tb.twx_f, tb.twr_f, done, err);
+        if constexpr (!xrt_length(NN))   // the others: xpass_res_tile.cu
+          return xs_launch(k_xres_s<NN, EE, true, false, ISO, true>, NN / EE, RB, c0, ngroups, nblocks_out, st, used,
+                           R, spec, g, tb.twx_f, tb.twr_f, done, err);
       });
       return cudaSuccess;
     }
@@ -275,13 +276,15 @@ cudaError_t xres_s(const ResidualArgs& R, float2* spec, const Geom& g, int N, in
     return cudaSuccess;
   if (stage_p) {
     PGB_XRES_SWITCH(N, {
-      return xs_launch(k_xres_s<NN, EE, HAS_Q, true, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
-                       tb.twx_f, tb.twr_f, done, err);
+      if constexpr (HAS_Q || !xrt_length(NN))
+        return xs_launch(k_xres_s<NN, EE, HAS_Q, true, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
+                         tb.twx_f, tb.twr_f, done, err);
     });
   } else {
     PGB_XRES_SWITCH(N, {
-      return xs_launch(k_xres_s<NN, EE, HAS_Q, false, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
-                       tb.twx_f, tb.twr_f, done, err);
+      if constexpr (HAS_Q || !xrt_length(NN))
+        return xs_launch(k_xres_s<NN, EE, HAS_Q, false, ISO>, NN / EE, RB, c, ngroups, nblocks_out, st, used, R, spec, g,
+                         tb.twx_f, tb.twr_f, done, err);
     });
   }
   return cudaSuccess;
