@@ -1191,33 +1191,27 @@ int poisson_solve_adjoint(poisson_plan* pl, const void* gp, const void* p, void*
 // this plan's direct solve (its rho0 profile) as the preconditioner.
 // ---------------------------------------------------------------------------
 struct CgLayout {
-  size_t off_r, off_d, off_q, off_t, off_z, off_part, off_lv, off_ce, off_cn, off_cu, bytes;
+  size_t off_r, off_d, off_q, off_t, off_z, off_part, off_state, off_lv, off_rh, off_rl, bytes;
 };
 static CgLayout cg_layout(const poisson_plan* pl) {
   CgLayout L{};
-  const size_t f = align256(sizeof(double) * (size_t)pl->g.N);
   size_t off = align256(pl->ws_bytes);
-  L.off_r = off;
-  off += f;
-  L.off_d = off;
-  off += f;
-  L.off_q = off;
-  off += f;
-  L.off_t = off;
-  off += f;
-  L.off_z = off;
-  off += f;
-  L.off_part = off;
-  off += align256(2 * sizeof(double) * (size_t)cg_blocks());
-  L.off_lv = off;
-  off += align256(sizeof(CgLevel) * (size_t)pl->nz);
-  const size_t fc = align256(sizeof(float2) * (size_t)pl->g.N);   // face coefficients as float pairs
-  L.off_ce = off;
-  off += fc;
-  L.off_cn = off;
-  off += fc;
-  L.off_cu = off;
-  off += fc;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off += align256(bytes);
+    return o;
+  };
+  const size_t N = (size_t)pl->g.N;
+  L.off_r = take(sizeof(double) * N);
+  L.off_d = take(sizeof(double) * N);
+  L.off_q = take(sizeof(double) * N);
+  L.off_t = take(sizeof(double) * N);
+  L.off_z = take(sizeof(double) * N);
+  L.off_part = take(2 * sizeof(double) * (size_t)cg_blocks(pl->nz));
+  L.off_state = take(cg_state_bytes());
+  L.off_lv = take(sizeof(CgLevel) * (size_t)pl->nz);
+  L.off_rh = take(sizeof(float) * N);
+  L.off_rl = take(sizeof(float) * N);
   L.bytes = off;
   return L;
 }
@@ -1228,18 +1222,15 @@ int poisson_cg_workspace_bytes(const poisson_plan* pl, size_t* bytes) {
   return POISSON_OK;
 }
 
-// Sum the two-per-block partials of the last reduction on the host, in block order.
-static int cg_sums(const double* partials_dev, unsigned nb, cudaStream_t st, double* s0, double* s1) {
-  std::vector<double> h(2 * (size_t)nb);
-  PGB_CUDA(cudaMemcpyAsync(h.data(), partials_dev, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, st));
-  PGB_CUDA(cudaStreamSynchronize(st));
-  double a = 0, b = 0;
-  for (unsigned i = 0; i < nb; ++i) {
-    a += h[2 * i];
-    b += h[2 * i + 1];
-  }
-  *s0 = a;
-  if (s1) *s1 = b;
+// z = G t, the preconditioner.  The mixed plan without refinement sweeps transforms floats: its source is then
+// taken and its solution left in float (the values a double field would carry through its conversions).
+static bool cg_float_pc(const poisson_plan* pl) { return pl->mixed() && pl->max_sweeps == 0; }
+static int cg_precondition(poisson_plan* pl, const void* t, void* z, char* ws, cudaStream_t st) {
+  if (!cg_float_pc(pl)) return solve_fields(pl, t, z, ws, st);
+  PGB_CUDA(launch_zero_words(ws + pl->off_stats, pl->stats_bytes, st));
+  bool mid = false;
+  PGB_CUDA(forward_columns(pl, t, 0, ws, st, 0, nullptr, nullptr, nullptr, nullptr, 0, &mid));
+  PGB_CUDA(inverse(pl, ws, st, nullptr, 0, XINV_PLAIN, z, XinvExtra{}, nullptr, nullptr, mid));
   return POISSON_OK;
 }
 
@@ -1260,13 +1251,10 @@ int poisson_cg_solve(poisson_plan* pl, const double* rho3, const double* S, doub
     return POISSON_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   char* ws = (char*)workspace;
-  const CgKernels K = cg_kernels(pl->nx, pl->ny, pl->nz, pl->dx, pl->dy, pl->top_dirichlet());
-  const int nbmax = cg_blocks();
-  const unsigned nb = cg_grid(K, nbmax);
+  const CgGrid K{pl->nx, pl->ny, pl->nz, pl->top_dirichlet()};
   CgArgs a{};
   a.rho = rho3;
   a.S = S;
-  a.dz = pl->dz_d;
   {
     // per-level constants; the preconditioner's weights come from the plan's device table (set_rho0)
     const int nz = pl->nz;
@@ -1278,89 +1266,69 @@ int poisson_cg_solve(poisson_plan* pl, const double* rho3, const double* S, doub
       const double dzk = pl->dz[k];
       lv[k].dz = dzk;
       lv[k].idz = 1.0 / dzk;
-      lv[k].hup = (k + 1 < nz) ? 0.5 / (0.5 * (dzk + pl->dz[k + 1])) : (pl->top_dirichlet() ? 1.0 / (0.5 * dzk) : 0.0);
-      lv[k].hdn = (k > 0) ? 0.5 / (0.5 * (dzk + pl->dz[k - 1])) : 0.0;
       lv[k].iwbar = 1.0 / Wb[k];
+      lv[k].kx = split_host(0.5 / (pl->dx * pl->dx) * dzk);
+      lv[k].ky = split_host(0.5 / (pl->dy * pl->dy) * dzk);
+      lv[k].ku = split_host((k + 1 < nz) ? 0.5 / (0.5 * (dzk + pl->dz[k + 1]))
+                                         : (pl->top_dirichlet() ? 1.0 / (0.5 * dzk) : 0.0));
     }
     CgLevel* lv_d = (CgLevel*)(ws + L.off_lv);
     PGB_CUDA(cudaMemcpyAsync(lv_d, lv.data(), sizeof(CgLevel) * nz, cudaMemcpyHostToDevice, st));
     PGB_CUDA(cudaStreamSynchronize(st));   // lv is a local vector
     a.lv = lv_d;
   }
-  a.ce = (float2*)(ws + L.off_ce);
-  a.cn = (float2*)(ws + L.off_cn);
-  a.cu = (float2*)(ws + L.off_cu);
-  PGB_CUDA(cg_launch(CG_FACES, K, a, nbmax, st));
   a.p = p;
   a.r = (double*)(ws + L.off_r);
   a.d = (double*)(ws + L.off_d);
   a.q = (double*)(ws + L.off_q);
-  a.t = (double*)(ws + L.off_t);
-  a.z = (const double*)(ws + L.off_z);
+  a.t = ws + L.off_t;
+  a.z = ws + L.off_z;
+  a.rh = (float*)(ws + L.off_rh);
+  a.rl = (float*)(ws + L.off_rl);
+  a.float_pc = cg_float_pc(pl) ? 1 : 0;
   a.partials = (double*)(ws + L.off_part);
-  double* z = (double*)(ws + L.off_z);
-  double s0 = 0, s1 = 0;
-  // compatibility: with zero flux at the top remove mu_W = sum W S / sum W
-  double mu = 0;
-  if (!pl->top_dirichlet()) {
-    PGB_CUDA(cg_launch(CG_WMEAN, K, a, nbmax, st));
-    if ((rc = cg_sums(a.partials, nb, st, &s0, &s1)) != POISSON_OK) return rc;
-    mu = s1 > 0 ? s0 / s1 : 0.0;
-  }
-  a.scalar = mu;
-  PGB_CUDA(cg_launch(CG_START, K, a, nbmax, st));
-  if ((rc = cg_sums(a.partials, nb, st, &s0, nullptr)) != POISSON_OK) return rc;
-  const double snorm = std::sqrt(s0);
-  double rel = snorm > 0 ? 1.0 : 0.0;
-  a.inv_snorm = snorm > 0 ? 1.0 / snorm : 0.0;
+  a.state = ws + L.off_state;
+  void* z = ws + L.off_z;
+  CgReport rep{};
+  PGB_CUDA(launch_zero_words(a.state, align256(cg_state_bytes()), st));
+  PGB_CUDA(cg_launch(CG_PREP, K, a, st));   // with zero flux at the top mu_W = sum W S / sum W is removed
+  PGB_CUDA(cg_launch(CG_START, K, a, st));
+  PGB_CUDA(cg_read(a.state, &rep, st));
+  double rel = rep.ss > 0 ? 1.0 : 0.0;
   int it = 0;
-  bool conv = snorm == 0;
+  bool conv = rep.ss == 0;
+  a.step = 3;   // p = 0
   if (!conv) {
-    // z = M r, d = z, rz = r . z
-    if ((rc = solve_fields(pl, a.t, z, ws, st)) != POISSON_OK) return rc;
-    a.q = nullptr;
-    PGB_CUDA(cg_launch(CG_DOTS, K, a, nbmax, st));
-    a.q = (double*)(ws + L.off_q);
-    if ((rc = cg_sums(a.partials, nb, st, &s0, nullptr)) != POISSON_OK) return rc;
-    double rz = s0;
-    a.flag = 1;
-    PGB_CUDA(cg_launch(CG_DIR, K, a, nbmax, st));
-    a.flag = 0;
+    // z = M r, d = z, rz = r . z; the step lengths stay on the device
+    if ((rc = cg_precondition(pl, a.t, z, ws, st)) != POISSON_OK) return rc;
+    PGB_CUDA(cg_launch(CG_DOTS0, K, a, st));
+    a.step = 0;
+    PGB_CUDA(cg_launch(CG_DIR, K, a, st));
     for (it = 1; it <= max_iter; ++it) {
-      PGB_CUDA(cg_launch(CG_APPLY, K, a, nbmax, st));
-      if ((rc = cg_sums(a.partials, nb, st, &s0, nullptr)) != POISSON_OK) return rc;
-      if (!(s0 > 0)) break;   // d in the null space (or a breakdown): nothing left to reduce
-      const double alpha = rz / s0;
-      a.scalar = alpha;
-      PGB_CUDA(cg_launch(CG_UPDATE, K, a, nbmax, st));
-      if ((rc = cg_sums(a.partials, nb, st, &s0, nullptr)) != POISSON_OK) return rc;
-      rel = std::sqrt(s0);   // the update kernel's sum is already relative to ||S||
+      a.step = it == 1 ? 1 : 2;
+      PGB_CUDA(cg_launch(CG_APPLY, K, a, st));
+      PGB_CUDA(cg_launch(CG_UPDATE, K, a, st));
+      PGB_CUDA(cg_read(a.state, &rep, st));
+      if (!(rep.dq > 0)) break;   // d in the null space (or a breakdown): nothing left to reduce
+      rel = std::sqrt(rep.rel2);  // the update kernel's sum is already relative to ||S||
       if (rel <= tol) {
         conv = true;
         break;
       }
       if (it == max_iter) break;
-      if ((rc = solve_fields(pl, a.t, z, ws, st)) != POISSON_OK) return rc;
-      PGB_CUDA(cg_launch(CG_DOTS, K, a, nbmax, st));
-      if ((rc = cg_sums(a.partials, nb, st, &s0, &s1)) != POISSON_OK) return rc;
-      const double beta = -alpha * s1 / rz;   // Polak-Ribiere: z_new . (r_new - r_old) / (r_old . z_old)
-      rz = s0;
-      a.scalar = beta;
-      PGB_CUDA(cg_launch(CG_DIR, K, a, nbmax, st));
+      if ((rc = cg_precondition(pl, a.t, z, ws, st)) != POISSON_OK) return rc;
+      PGB_CUDA(cg_launch(CG_DOTS, K, a, st));
+      PGB_CUDA(cg_launch(CG_DIR, K, a, st));
     }
     if (it > max_iter) it = max_iter;
   }
-  if (!pl->top_dirichlet()) {   // plain mean zero, as the direct solve
-    PGB_CUDA(cg_launch(CG_SUM, K, a, nbmax, st));
-    if ((rc = cg_sums(a.partials, nb, st, &s0, nullptr)) != POISSON_OK) return rc;
-    a.scalar = s0 / (double)pl->g.N;
-    PGB_CUDA(cg_launch(CG_SHIFT, K, a, nbmax, st));
-  }
+  PGB_CUDA(cg_launch(CG_LAST, K, a, st));   // p += alpha d of the last step
+  if (!pl->top_dirichlet()) PGB_CUDA(cg_launch(CG_SHIFT, K, a, st));   // plain mean zero, as the direct solve
   if (info) {
     info->iterations = it;
     info->converged = conv ? 1 : 0;
     info->rel_residual = rel;
-    info->removed_weighted_mean = mu;
+    info->removed_weighted_mean = rep.mu;
   }
   return conv ? POISSON_OK : POISSON_ERR_NOT_CONVERGED;
 }

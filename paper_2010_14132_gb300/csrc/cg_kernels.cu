@@ -15,32 +15,105 @@
 // preconditioner is z = -G(r / Wbar): G is the plan's solve for the level density
 // rho0 (weights Wbar_k = rho0_k dz_k).  Polak-Ribiere beta = -alpha (q . z_new)/(r . z)
 // keeps the iteration robust to a preconditioner that is applied in reduced precision.
-// All vectors and reductions are FP64; the partial sums go to the host in block order.
-// The FP64 pipe (1/65 of the FP32 rate here) would bound these kernels, so no FP64
-// division runs per point: the level reciprocals come from small tables, and the
-// residual's weight 1/rho (needed only for the stopping test) is a float reciprocal.
-// The operator itself runs in double-float arithmetic: its six face coefficients are
-// formed once per solve in FP64 and stored as float pairs, and each application
-// splits the FP64 direction into float pairs with integer operations and forms
-// sum_f c_f (d_f - d_c) with error-free transformations, differences first.
+// All vectors and reductions are FP64, the partial sums added in block order by each launch's last block, which also
+// forms the step lengths on the device: the host waits once per iteration, for the stopping test.
+//
+// What bounds the kernels (GB300, 512 x 512 x 64, 16.8 M points): the FP64 unit does 1.7 operations a clock and SM, so
+// one FP64 operation per point costs as much as 11 bytes of HBM traffic, and each kernel keeps to two or so:
+//   k_cg_apply   instruction issue (the operator in double-float arithmetic, see below): 285 -> 185 us
+//   k_cg_update  r -= alpha q, t = -r/Wbar (float where the preconditioner transforms floats), the residual norm in
+//                the FP32 pipe; 32 bytes a point (64 with the step of p): 161 -> 103 us
+//   k_cg_dots    z.r and z.q; 20 bytes a point, bound by the FP64 unit: 73 us
+//   k_cg_dir     p += alpha d (of the step before, as d is read anyway) and d = z + beta d; 36 bytes a point: 93 us
+//                (57 without the step of p)
+// With the mixed plan's float preconditioner z stays the float field the inverse transform writes.
+// No FP64 division runs per point: the level reciprocals come from a small table, and the residual's weight
+// 1/rho (needed only for the stopping test) is a float reciprocal.
+//
+// The operator: q = -sum_f c_f (d_f - d_c) with c_f = const_k (rho_f + rho_c).  rho is split into float pairs once
+// per solve, d as it is read (integer operations); differences and sums are formed first and exactly
+// (two-sums), products by FMA-based two-products, on the two points of a pair at once (packed FP32).  A block
+// takes a tile of 64 x 8 points and marches up the levels: every value is read from memory once (24 bytes a
+// point with q, where three stored face coefficients made it 40), the x neighbours come by shuffles, the y
+// neighbours through shared memory, and the flux through the upper face is kept as the next level's lower one.
 #include "kernels.cuh"
 #include "residual2.cuh"
 
 namespace pgb {
 namespace {
 
+// The step lengths and sums of a solve, on the device.
+struct CgState {
+  double mu, ss, inv_snorm, rz, dq, alpha, beta, rel2, shift;
+  unsigned ticket;
+};
+
 struct CgDims {
   int nx, ny, nz;
   long long plane, n;
-  double hx2, hy2;     // 0.5/dx^2, 0.5/dy^2 (the 0.5 of the face-density mean folded in)
   int top_dirichlet;
 };
 
-__device__ __forceinline__ void block_sum2(double a, double b, double* partials) {
+// What a launch's sums (s0, s1) mean; run by one thread once every block's partials are added up.
+__device__ __forceinline__ void cg_finish(int op, CgState* c, double s0, double s1, const CgDims& D) {
+  switch (op) {
+    case CG_PREP: c->mu = (!D.top_dirichlet && s1 > 0) ? s0 / s1 : 0.0; break;
+    case CG_START:
+      c->ss = s0;
+      c->inv_snorm = s0 > 0 ? 1.0 / sqrt(s0) : 0.0;
+      break;
+    case CG_DOTS0: c->rz = s0; break;
+    case CG_APPLY:
+      c->dq = s0;
+      c->alpha = s0 > 0 ? c->rz / s0 : 0.0;   // otherwise d is in the null space (or a breakdown): no step
+      break;
+    case CG_UPDATE: c->rel2 = s0; break;
+    case CG_DOTS:
+      c->beta = -c->alpha * s1 / c->rz;       // Polak-Ribiere: z_new . (r_new - r_old) / (r_old . z_old)
+      c->rz = s0;
+      break;
+    case CG_LAST: c->shift = s0 / (double)D.n; break;
+    default: break;
+  }
+}
+
+// Sums a and b over the launch's blocks (256 threads each): per block a shuffle tree and the warps in order, over the
+// blocks by the last one to finish, in block order per thread and then a fixed tree.
+__device__ __forceinline__ void cg_reduce(int op, CgState* c, double a, double b, double* partials, const CgDims& D) {
   __shared__ double s0[256], s1[256];
+  __shared__ bool last;
   const int t = threadIdx.x;
-  s0[t] = a;
-  s1[t] = b;
+  const unsigned nb = gridDim.x * gridDim.y, blk = blockIdx.y * gridDim.x + blockIdx.x;
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_down_sync(0xffffffffu, a, o);
+    b += __shfl_down_sync(0xffffffffu, b, o);
+  }
+  if ((t & 31) == 0) {
+    s0[t >> 5] = a;
+    s1[t >> 5] = b;
+  }
+  __syncthreads();
+  if (t == 0) {
+    double x = 0, y = 0;
+    for (int w = 0; w < 8; ++w) {
+      x += s0[w];
+      y += s1[w];
+    }
+    partials[2 * blk] = x;
+    partials[2 * blk + 1] = y;
+    __threadfence();
+    last = atomicAdd(&c->ticket, 1u) == nb - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double x = 0, y = 0;
+  for (unsigned i = t; i < nb; i += 256) {
+    x += __ldcg(&partials[2 * i]);
+    y += __ldcg(&partials[2 * i + 1]);
+  }
+  s0[t] = x;
+  s1[t] = y;
   __syncthreads();
   for (int h = 128; h > 0; h >>= 1) {
     if (t < h) {
@@ -50,273 +123,428 @@ __device__ __forceinline__ void block_sum2(double a, double b, double* partials)
     __syncthreads();
   }
   if (t == 0) {
-    partials[2 * blockIdx.x] = s0[0];
-    partials[2 * blockIdx.x + 1] = s1[0];
+    c->ticket = 0u;   // ready for the next launch
+    cg_finish(op, c, s0[0], s1[0], D);
   }
 }
 
-// Face coefficients of W A, once per solve, as float pairs (hi, lo):
-//   ce = 0.5/dx^2 (rho_i + rho_{i+1}) dz_k (east face), cn = 0.5/dy^2 (rho_j + rho_{j+1}) dz_k (north),
-//   cu = (rho_k + rho_{k+1}) 0.5/h_{k+1/2} (upper; at the top rho_k 2/dz_k with p = 0 on the face, else 0).
-// x as a float pair (h, l) with integer operations (h + l within 2^-47 |x|), keeping the
-// conversions off the FP64 pipe; the sums and products above stay in FP64 (6 operations per point)
-__device__ __forceinline__ float2 split_int(double x) {
+// Flat kernels: grid (blocks per level, nz), pairs of points; pairs of block x of a level.
+#define CG_PAIRS(i, D)                                                                                      \
+  for (long long half = (D).plane / 2, off = (long long)blockIdx.y * half, i_ = blockIdx.x * 256ll + threadIdx.x, \
+                 i = off + i_;                                                                              \
+       i_ < half; i_ += gridDim.x * 256ll, i = off + i_)
+
+// rho as float pairs (within 2^-47), and sum W S, sum W for mu_W = sum W S / sum W
+__global__ void __launch_bounds__(256) k_cg_prep(const double2* __restrict__ rho, const double2* __restrict__ S,
+                                                 float2* __restrict__ rh, float2* __restrict__ rl,
+                                                 const CgLevel* __restrict__ lv, CgDims D, CgState* c,
+                                                 double* __restrict__ partials) {
+  double ws = 0, w = 0;
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 r = rho[i], s = S[i];
+    float2 h, l;
+    d2ff_trunc(r.x, h.x, l.x);
+    d2ff_trunc(r.y, h.y, l.y);
+    rh[i] = h;
+    rl[i] = l;
+    ws = fma(r.x, s.x, ws);
+    ws = fma(r.y, s.y, ws);
+    w += r.x + r.y;
+  }
+  const double dz = lv[blockIdx.y].dz;
+  cg_reduce(CG_PREP, c, ws * dz, w * dz, partials, D);
+}
+
+template <typename T> struct CgVec;
+template <> struct CgVec<double> {
+  using t = double2;
+  static __device__ __forceinline__ double2 in(double2 x) { return x; }
+  static __device__ __forceinline__ double2 out(double2 x) { return x; }
+};
+template <> struct CgVec<float> {
+  using t = float2;
+  static __device__ __forceinline__ double2 in(float2 x) { return make_double2(f2d_int(x.x), f2d_int(x.y)); }
+  static __device__ __forceinline__ float2 out(double2 x) { return make_float2(d2f_int(x.x), d2f_int(x.y)); }
+};
+
+// r = b = -W (S - mu), t = -r/Wbar (the preconditioner's source); sum S . S
+template <typename TT>
+__global__ void __launch_bounds__(256) k_cg_start(const double2* __restrict__ rho, const double2* __restrict__ S,
+                                                  double2* __restrict__ r, typename CgVec<TT>::t* __restrict__ t,
+                                                  const CgLevel* __restrict__ lv, CgDims D, CgState* c,
+                                                  double* __restrict__ partials) {
+  double ss = 0;
+  const CgLevel L = lv[blockIdx.y];
+  const double mu = c->mu, iw = -L.iwbar;
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 s = S[i], q = rho[i];
+    const double2 b = make_double2(-(q.x * L.dz) * (s.x - mu), -(q.y * L.dz) * (s.y - mu));
+    r[i] = b;
+    t[i] = CgVec<TT>::out(make_double2(b.x * iw, b.y * iw));
+    ss = fma(s.x, s.x, ss);
+    ss = fma(s.y, s.y, ss);
+  }
+  cg_reduce(CG_START, c, ss, 0.0, partials, D);
+}
+
+// Two points' d and rho as float pairs.
+struct CgPt {
+  float2 dh, dl, rh, rl;
+};
+// (rho_f + rho_c) (d_f - d_c) = ph - npl, an unnormalised float pair: sum and difference exact in their high parts,
+// the product of the high parts exact.  The low part comes negated, which saves the packed negations.
+__device__ __forceinline__ void cg_flux(const CgPt& f, const CgPt& c, float2& ph, float2& npl) {
+  float2 s, e, t, u;
+  two_diff2(f.dh, c.dh, s, e);
+  const float2 lo = add2(e, sub2(f.dl, c.dl));
+  two_sum2(f.rh, c.rh, t, u);
+  const float2 m1 = make_float2(-1.f, -1.f), nt = mul2(t, m1);
+  const float2 ntl = fma2(u, m1, mul2(add2(f.rl, c.rl), m1));
+  ph = mul2(t, s);
+  npl = fma2(nt, lo, fma2(ntl, s, fma2(nt, s, ph)));
+}
+// times a constant k = (h, l)
+__device__ __forceinline__ void cg_scale(float2& ph, float2& npl, float2 k) {
+  const float2 h = f2bc(k.x), nh = f2bc(-k.x), nl = f2bc(-k.y), p = mul2(h, ph);
+  npl = fma2(h, npl, fma2(nl, ph, fma2(nh, ph, p)));
+  ph = p;
+}
+// (H - L) += (ph - npl)
+__device__ __forceinline__ void cg_acc(float2& H, float2& L, float2 ph, float2 npl) {
+  float2 s, e;
+  two_sum2(H, ph, s, e);
+  H = s;
+  L = add2(L, sub2(npl, e));
+}
+__device__ __forceinline__ float2 cg_split(double x) {
   float h, l;
   d2ff_trunc(x, h, l);
   return make_float2(h, l);
 }
-
-__global__ void __launch_bounds__(256) k_cg_faces(const double* __restrict__ rho, float2* __restrict__ ce,
-                                                  float2* __restrict__ cn, float2* __restrict__ cu,
-                                                  const CgLevel* __restrict__ lv, CgDims D) {
-  const long long rows = (long long)D.nz * D.ny;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const int k = (int)(row / D.ny), j = (int)(row - (long long)k * D.ny);
-    const CgLevel L = lv[k];
-    const long long base = row * D.nx;
-    const long long dn_ = (j + 1 == D.ny ? (1 - D.ny) * (long long)D.nx : D.nx);
-    for (int i = threadIdx.x; i < D.nx; i += blockDim.x) {
-      const long long idx = base + i;
-      const long long e = idx + (i + 1 == D.nx ? 1 - D.nx : 1);
-      const double rc = rho[idx];
-      ce[idx] = split_int(D.hx2 * (rc + rho[e]) * L.dz);
-      cn[idx] = split_int(D.hy2 * (rc + rho[idx + dn_]) * L.dz);
-      double up = 0.0;
-      if (k + 1 < D.nz) up = (rc + rho[idx + D.plane]) * L.hup;
-      else if (D.top_dirichlet) up = rc * L.hup;
-      cu[idx] = split_int(up);
-    }
-  }
+__device__ __forceinline__ CgPt cg_point2(double2 d, float2 rh, float2 rl) {
+  const float2 a = cg_split(d.x), b = cg_split(d.y);
+  return {make_float2(a.x, b.x), make_float2(a.y, b.y), rh, rl};
 }
 
-// c (d_f - d_c) as an unnormalised float pair (ph, pl): the difference of the split values first
-// (exact high part), then the product with the split coefficient (exact high product).
-__device__ __forceinline__ void face_term(float fh, float fl, float ch, float cl, float2 c, float& ph, float& pl) {
-  float s, e;
-  two_sum(fh, -ch, s, e);
-  const float lo = e + (fl - cl);
-  two_prod(c.x, s, ph, pl);
-  pl = __fmaf_rn(c.x, lo, __fmaf_rn(c.y, s, pl));
-}
+constexpr int kCgTY = 8;    // rows of a tile (a warp each), 32 pairs of points wide
+constexpr int kCgZC = 16;   // levels a tile marches up
 
-// q = K d = -(W A d) = -sum_f c_f (d_f - d_c); partials: d . q
-__global__ void __launch_bounds__(256) k_cg_apply(const double* __restrict__ d, const float2* __restrict__ ce,
-                                                  const float2* __restrict__ cn, const float2* __restrict__ cu,
-                                                  double* __restrict__ q, CgDims D, double* __restrict__ partials) {
+// q = K d = -(W A d); sum d . q.  Tiles (x, y, level chunk) in grid-stride order.
+__global__ void __launch_bounds__(256) k_cg_apply(const double2* __restrict__ d, const float2* __restrict__ rh,
+                                                  const float2* __restrict__ rl, double2* __restrict__ q,
+                                                  const CgLevel* __restrict__ lv, CgDims D, CgState* c,
+                                                  double* __restrict__ partials) {
+  __shared__ float4 sd[2][kCgTY + 2][32], sr[2][kCgTY + 2][32];   // rows j0 - 1 .. j0 + 8 of a level
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nx2 = D.nx / 2, tx = (nx2 + 31) / 32, ty = (D.ny + kCgTY - 1) / kCgTY, tz = (D.nz + kCgZC - 1) / kCgZC;
   double acc = 0;
-  const long long rows = (long long)D.nz * D.ny;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {   // one x row per block step
-    const int k = (int)(row / D.ny), j = (int)(row - (long long)k * D.ny);
-    const long long base = row * D.nx;
-    const long long dn_ = (j + 1 == D.ny ? (1 - D.ny) * (long long)D.nx : D.nx);
-    const long long ds_ = (j == 0 ? (D.ny - 1) * (long long)D.nx : -(long long)D.nx);
-    const bool has_up = k + 1 < D.nz, has_dn = k > 0;
-    for (int i = threadIdx.x; i < D.nx; i += blockDim.x) {
-      const long long idx = base + i;
-      const long long w = idx + (i == 0 ? D.nx - 1 : -1), e = idx + (i + 1 == D.nx ? 1 - D.nx : 1);
-      const double dc = d[idx];
-      float ch, cl;
-      d2ff_trunc(dc, ch, cl);
-      float H = 0.f, Lo = 0.f;
-      auto add = [&](double df, float2 c) {
-        float fh, fl, ph, pl, s, t;
-        d2ff_trunc(df, fh, fl);
-        face_term(fh, fl, ch, cl, c, ph, pl);
-        two_sum(H, ph, s, t);
-        H = s;
-        Lo += t + pl;
+  for (long long tile = blockIdx.x; tile < (long long)tx * ty * tz; tile += gridDim.x) {
+    const int x0 = (int)(tile % tx) * 32, j0 = (int)(tile / tx % ty) * kCgTY, k0 = (int)(tile / tx / ty) * kCgZC;
+    const int k1 = min(D.nz, k0 + kCgZC), np = min(32, nx2 - x0), nr = min(kCgTY, D.ny - j0);
+    const bool act = lane < np && w < nr;
+    const int j = j0 + min(w, nr - 1), i = x0 + min(lane, np - 1);
+    // the row south (warp 0) or north (warp nr - 1) of the tile and the point west (lane 0) or east (lane np - 1; a
+    // tile is at least two pairs wide) of it, as element offsets within a level
+    const bool hs = w == 0, halo = hs || w == nr - 1, ew = lane == 0, edge = ew || lane == np - 1;
+    const unsigned half = (unsigned)(D.plane / 2);   // pairs of a level: at most 4096 x 4096 / 2
+    const unsigned own = (unsigned)(j * nx2 + i);
+    const unsigned js = (unsigned)((j0 == 0 ? D.ny - 1 : j0 - 1) * nx2 + i);
+    const unsigned jn = (unsigned)((j0 + nr == D.ny ? 0 : j0 + nr) * nx2 + i), jh = hs ? js : jn;
+    const unsigned ie = 2u * (unsigned)(j * nx2) +
+                        (unsigned)(ew ? (x0 == 0 ? D.nx - 1 : 2 * x0 - 1) : (x0 + np == nx2 ? 0 : 2 * (x0 + np)));
+    const double2* dk = d + (long long)k0 * half;
+    const float2 *hk = rh + (long long)k0 * half, *lk = rl + (long long)k0 * half;
+    const float2 z2 = make_float2(0.f, 0.f);
+    struct Raw {
+      double2 d;
+      float2 h, l;
+    };
+    auto load = [&](const double2* dp, const float2* hp, const float2* lp, unsigned at) {
+      return Raw{dp[at], hp[at], lp[at]};
+    };
+    auto split = [&](const Raw& v) { return cg_point2(v.d, v.h, v.l); };
+    double e_d = 0.0;   // the edge point
+    float e_h = 0.f, e_l = 0.f;
+    auto load_edge = [&](const double2* dp, const float2* hp, const float2* lp) {
+      e_d = reinterpret_cast<const double*>(dp)[ie];
+      e_h = reinterpret_cast<const float*>(hp)[ie];
+      e_l = reinterpret_cast<const float*>(lp)[ie];
+    };
+    // loaded ahead: this level's halo row and edge point, the next level's own pair
+    CgPt cur = split(load(dk, hk, lk, own));
+    Raw r_up{}, r_halo{};
+    if (k0 + 1 < D.nz) r_up = load(dk + half, hk + half, lk + half, own);
+    if (halo) r_halo = load(dk, hk, lk, jh);
+    if (edge) load_edge(dk, hk, lk);
+    float2 dnh = z2, dnl = z2;   // flux through the lower face, from the level below
+    if (k0 > 0) {
+      cg_flux(cur, split(load(dk - half, hk - half, lk - half, own)), dnh, dnl);
+      cg_scale(dnh, dnl, lv[k0 - 1].ku);
+    }
+    for (int k = k0, b = 0; k < k1; ++k, b ^= 1) {
+      // above the top: the face value 0 with the coefficient rho_k ku (ku = 0 with zero flux)
+      const CgPt up = k + 1 < D.nz ? split(r_up) : CgPt{z2, z2, z2, z2};
+      const CgPt hal = split(r_halo);
+      const float2 e_s = cg_split(e_d);
+      const float4 ev = make_float4(e_s.x, e_s.y, e_h, e_l);
+      auto publish = [&](int r, const CgPt& v) {
+        sd[b][r][lane] = make_float4(v.dh.x, v.dh.y, v.dl.x, v.dl.y);
+        sr[b][r][lane] = make_float4(v.rh.x, v.rh.y, v.rl.x, v.rl.y);
       };
-      add(d[e], ce[idx]);
-      add(d[w], ce[w]);
-      add(d[idx + dn_], cn[idx]);
-      add(d[idx + ds_], cn[idx + ds_]);
-      if (has_up) add(d[idx + D.plane], cu[idx]);
-      else add(0.0, cu[idx]);   // the face value 0 above the top (cu = 0 there with zero flux)
-      if (has_dn) add(d[idx - D.plane], cu[idx - D.plane]);
-      float s, t;
-      two_sum(H, Lo, s, t);
-      const double Kd = -ff2d_fast(s, t);
-      q[idx] = Kd;
-      acc += dc * Kd;
+      if (w < nr) publish(w + 1, cur);
+      if (halo) publish(hs ? 0 : nr + 1, hal);
+      if (hs && nr == 1) publish(2, split(load(dk, hk, lk, jn)));   // a tile of one row has both next to it
+      const double2* dn_ = dk + half;
+      const float2 *hn_ = hk + half, *ln_ = lk + half;
+      if (k + 1 < k1) {   // ahead of this level's arithmetic
+        if (halo) r_halo = load(dn_, hn_, ln_, jh);
+        if (edge) load_edge(dn_, hn_, ln_);
+        if (k + 2 < D.nz) r_up = load(dn_ + half, hn_ + half, ln_ + half, own);
+      }
+      __syncthreads();
+      const CgLevel& L = lv[k];
+      float2 H, Lo, ph, pl, eh, el;
+      // x: the faces (west, middle) and (middle, east) of the pair
+      float4 pw = make_float4(__shfl_up_sync(~0u, cur.dh.y, 1), __shfl_up_sync(~0u, cur.dl.y, 1),
+                              __shfl_up_sync(~0u, cur.rh.y, 1), __shfl_up_sync(~0u, cur.rl.y, 1));
+      float4 pe = make_float4(__shfl_down_sync(~0u, cur.dh.x, 1), __shfl_down_sync(~0u, cur.dl.x, 1),
+                              __shfl_down_sync(~0u, cur.rh.x, 1), __shfl_down_sync(~0u, cur.rl.x, 1));
+      if (ew) pw = ev;
+      if (edge && !ew) pe = ev;
+      const CgPt west = {make_float2(pw.x, cur.dh.x), make_float2(pw.y, cur.dl.x), make_float2(pw.z, cur.rh.x),
+                         make_float2(pw.w, cur.rl.x)};
+      const CgPt east = {make_float2(cur.dh.y, pe.x), make_float2(cur.dl.y, pe.y), make_float2(cur.rh.y, pe.z),
+                         make_float2(cur.rl.y, pe.w)};
+      cg_flux(west, cur, H, Lo);
+      cg_flux(east, cur, eh, el);
+      cg_acc(H, Lo, eh, el);
+      cg_scale(H, Lo, L.kx);
+      // y
+      auto row = [&](int r) {
+        const float4 a = sd[b][r][lane], e = sr[b][r][lane];
+        return CgPt{make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(e.x, e.y), make_float2(e.z, e.w)};
+      };
+      cg_flux(row(w), cur, ph, pl);
+      cg_flux(row(w + 2), cur, eh, el);
+      cg_acc(ph, pl, eh, el);
+      cg_scale(ph, pl, L.ky);
+      cg_acc(H, Lo, ph, pl);
+      // z
+      cg_flux(up, cur, ph, pl);
+      cg_scale(ph, pl, L.ku);
+      cg_acc(H, Lo, ph, pl);
+      {   // minus the flux through the lower face
+        float2 s, e;
+        two_diff2(H, dnh, s, e);
+        H = s;
+        Lo = sub2(Lo, add2(dnl, e));
+      }
+      dnh = ph;
+      dnl = pl;
+      float2 s, t;
+      two_diff2(Lo, H, s, t);   // K d = -(W A d)
+      if (act) {
+        const double2 Kd = make_double2(ff2d_fast(s.x, t.x), ff2d_fast(s.y, t.y)), dc = dk[own];
+        q[(long long)k * half + own] = Kd;
+        acc = fma(dc.x, Kd.x, acc);
+        acc = fma(dc.y, Kd.y, acc);
+      }
+      cur = up;
+      dk = dn_;
+      hk = hn_;
+      lk = ln_;
     }
+    __syncthreads();   // the buffers are reused by the next tile
   }
-  block_sum2(acc, 0.0, partials);
+  cg_reduce(CG_APPLY, c, acc, 0.0, partials, D);
 }
 
-// r = b = -W (S - mu), p = 0, t = -r/Wbar (the preconditioner's source); partials: S . S
-__global__ void __launch_bounds__(256) k_cg_start(const double* __restrict__ rho, const double* __restrict__ S,
-                                                  double mu, double* __restrict__ r, double* __restrict__ p,
-                                                  double* __restrict__ t, const double* __restrict__ dz,
-                                                  const CgLevel* __restrict__ lv, CgDims D,
-                                                  double* __restrict__ partials) {
-  double ss = 0;
-  const long long rows = (long long)D.nz * D.ny;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const CgLevel L = lv[(int)(row / D.ny)];
-    for (int i = threadIdx.x; i < D.nx; i += blockDim.x) {
-      const long long idx = row * D.nx + i;
-      const double s = S[idx];
-      const double b = -(rho[idx] * L.dz) * (s - mu);
-      r[idx] = b;
-      p[idx] = 0.0;
-      t[idx] = -b * L.iwbar;
-      ss += s * s;
-    }
-  }
-  block_sum2(ss, 0.0, partials);
-}
-
-// partials: W S, W (for the compatibility projection mu_W = sum W S / sum W)
-__global__ void __launch_bounds__(256) k_cg_wmean(const double* __restrict__ rho, const double* __restrict__ S,
-                                                  const double* __restrict__ dz, CgDims D,
-                                                  double* __restrict__ partials) {
-  double ws = 0, w = 0;
-  const long long rows = (long long)D.nz * D.ny;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const double dzk = dz[(int)(row / D.ny)];
-    for (int i = threadIdx.x; i < D.nx; i += blockDim.x) {
-      const long long idx = row * D.nx + i;
-      const double wk = rho[idx] * dzk;
-      ws += wk * S[idx];
-      w += wk;
-    }
-  }
-  block_sum2(ws, w, partials);
-}
-
-// p += alpha d, r -= alpha q, t = -r/Wbar; partials: (r/(W ||S||))^2 (the relative residual of A p = S - mu)
-__global__ void __launch_bounds__(256) k_cg_update(const double* __restrict__ rho, double alpha, float inv_snorm,
-                                                   const double* __restrict__ d, const double* __restrict__ q,
-                                                   double* __restrict__ p, double* __restrict__ r,
-                                                   double* __restrict__ t, const CgLevel* __restrict__ lv, CgDims D,
+// r -= alpha q, t = -r/Wbar; sum (r/(W ||S||))^2 (the relative residual of A p = S - mu)
+template <typename TT>
+__global__ void __launch_bounds__(256) k_cg_update(const float2* __restrict__ rh, const double2* __restrict__ q,
+                                                   double2* __restrict__ r, typename CgVec<TT>::t* __restrict__ t,
+                                                   const CgLevel* __restrict__ lv, CgDims D, CgState* c,
                                                    double* __restrict__ partials) {
+  const CgLevel L = lv[blockIdx.y];
+  const double na = -c->alpha, iw = -L.iwbar;
+  const float idz = (float)L.idz * (float)c->inv_snorm;   // the norm comes out relative to ||S||
   float rr = 0.f;
-  const long long rows = (long long)D.nz * D.ny;
-  for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-    const CgLevel L = lv[(int)(row / D.ny)];
-    const float idz = (float)L.idz * inv_snorm;   // the norm comes out relative to ||S||
-  for (int i = threadIdx.x; i < D.nx; i += blockDim.x) {
-    const long long idx = row * D.nx + i;
-    p[idx] += alpha * d[idx];
-    const double rn = r[idx] - alpha * q[idx];
-    r[idx] = rn;
-    t[idx] = -rn * L.iwbar;
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 qv = q[i], rv = r[i];
+    const float2 h = rh[i];
+    const double2 rn = make_double2(fma(na, qv.x, rv.x), fma(na, qv.y, rv.y));
+    r[i] = rn;
+    t[i] = CgVec<TT>::out(make_double2(rn.x * iw, rn.y * iw));
     // residual of A p = S - mu: r / (rho dz), to float accuracy (a stopping test), in the FP32 pipe
-    float rh, rl, h, l;
-    d2ff_trunc(rn, rh, rl);
-    d2ff_trunc(rho[idx], h, l);
-    const float ra = rh * idz * __frcp_rn(h);
-    rr = __fmaf_rn(ra, ra, rr);
+    const float ax = d2f_int(rn.x) * idz * __frcp_rn(h.x), ay = d2f_int(rn.y) * idz * __frcp_rn(h.y);
+    rr = __fmaf_rn(ax, ax, __fmaf_rn(ay, ay, rr));
   }
-  }
-  block_sum2((double)rr, 0.0, partials);
+  cg_reduce(CG_UPDATE, c, (double)rr, 0.0, partials, D);
 }
 
-// partials: z . r, z . q
-__global__ void __launch_bounds__(256) k_cg_dots(const double* __restrict__ z, const double* __restrict__ r,
-                                                 const double* __restrict__ q, CgDims D,
-                                                 double* __restrict__ partials) {
+// z . r and, from the second preconditioner solve on, z . q
+template <typename TT, bool FIRST>
+__global__ void __launch_bounds__(256) k_cg_dots(const typename CgVec<TT>::t* __restrict__ z,
+                                                 const double2* __restrict__ r, const double2* __restrict__ q, CgDims D,
+                                                 CgState* c, double* __restrict__ partials) {
   double zr = 0, zq = 0;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < D.n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const double zv = z[idx];
-    zr += zv * r[idx];
-    if (q) zq += zv * q[idx];
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 zv = CgVec<TT>::in(z[i]), rv = r[i];
+    zr = fma(zv.x, rv.x, zr);
+    zr = fma(zv.y, rv.y, zr);
+    if (!FIRST) {
+      const double2 qv = q[i];
+      zq = fma(zv.x, qv.x, zq);
+      zq = fma(zv.y, qv.y, zq);
+    }
   }
-  block_sum2(zr, zq, partials);
+  cg_reduce(FIRST ? CG_DOTS0 : CG_DOTS, c, zr, zq, partials, D);
 }
 
-// d = z + beta d (beta_is_zero: d = z, whatever d held)
-__global__ void __launch_bounds__(256) k_cg_dir(const double* __restrict__ z, double beta, int beta_is_zero,
-                                                double* __restrict__ d, long long n) {
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x)
-    d[idx] = beta_is_zero ? z[idx] : z[idx] + beta * d[idx];
+// STEP 0: d = z.  1: p = alpha d, d = z + beta d.  2: p += alpha d, d = z + beta d.
+template <typename TT, int STEP>
+__global__ void __launch_bounds__(256) k_cg_dir(const typename CgVec<TT>::t* __restrict__ z, double2* __restrict__ d,
+                                                double2* __restrict__ p, CgDims D, const CgState* __restrict__ c) {
+  const double alpha = STEP ? c->alpha : 0.0, beta = STEP ? c->beta : 0.0;
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 zv = CgVec<TT>::in(z[i]);
+    if (STEP == 0) {
+      d[i] = zv;
+    } else {
+      const double2 dv = d[i], po = STEP == 2 ? p[i] : make_double2(0.0, 0.0);
+      p[i] = STEP == 2 ? make_double2(fma(alpha, dv.x, po.x), fma(alpha, dv.y, po.y))
+                       : make_double2(alpha * dv.x, alpha * dv.y);
+      d[i] = make_double2(fma(beta, dv.x, zv.x), fma(beta, dv.y, zv.y));
+    }
+  }
 }
 
-// partials: sum p; then (second launch) p -= shift
-__global__ void __launch_bounds__(256) k_cg_sum(const double* __restrict__ p, long long n,
-                                                double* __restrict__ partials) {
+// the last step's p (STEP as above; 3: p = 0), and sum p
+template <int STEP>
+__global__ void __launch_bounds__(256) k_cg_last(const double2* __restrict__ d, double2* __restrict__ p, CgDims D,
+                                                 CgState* c, double* __restrict__ partials) {
+  const double alpha = c->alpha;
   double s = 0;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x)
-    s += p[idx];
-  block_sum2(s, 0.0, partials);
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    double2 v = make_double2(0.0, 0.0);
+    if (STEP != 3) {
+      const double2 dv = d[i];
+      if (STEP == 2) v = p[i];
+      v = STEP == 2 ? make_double2(fma(alpha, dv.x, v.x), fma(alpha, dv.y, v.y))
+                    : make_double2(alpha * dv.x, alpha * dv.y);
+    }
+    p[i] = v;
+    s += v.x + v.y;
+  }
+  cg_reduce(CG_LAST, c, s, 0.0, partials, D);
 }
-__global__ void __launch_bounds__(256) k_cg_shift(double* __restrict__ p, double shift, long long n) {
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x)
-    p[idx] -= shift;
+// p -= its mean
+__global__ void __launch_bounds__(256) k_cg_shift(double2* __restrict__ p, CgDims D, const CgState* __restrict__ c) {
+  const double m = c->shift;
+#pragma unroll 2
+  CG_PAIRS(i, D) {
+    const double2 v = p[i];
+    p[i] = make_double2(v.x - m, v.y - m);
+  }
 }
 
 }  // namespace
 
 // Host side ---------------------------------------------------------------------
 
-int cg_blocks() {
+static int cg_sms() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return (sms > 0 ? sms : 1) * 8;
+  return sms > 0 ? sms : 1;
 }
-
-CgKernels cg_kernels(int nx, int ny, int nz, double dx, double dy, int top_dirichlet) {
-  CgKernels K{};
-  K.nx = nx;
-  K.ny = ny;
-  K.nz = nz;
-  K.idx2 = 1.0 / (dx * dx);
-  K.idy2 = 1.0 / (dy * dy);
-  K.top_dirichlet = top_dirichlet;
-  return K;
+// blocks of the largest launch: eight a SM, and at least one per level
+int cg_blocks(int nz) {
+  const int b = cg_sms() * 8;
+  return b > nz ? b : nz;
 }
+size_t cg_state_bytes() { return sizeof(CgState); }
 
-static CgDims dims_of(const CgKernels& K) {
+cudaError_t cg_launch(int op, const CgGrid& K, const CgArgs& a, cudaStream_t st) {
   CgDims D{};
   D.nx = K.nx;
   D.ny = K.ny;
   D.nz = K.nz;
   D.plane = (long long)K.nx * K.ny;
   D.n = D.plane * K.nz;
-  D.hx2 = 0.5 * K.idx2;
-  D.hy2 = 0.5 * K.idy2;
   D.top_dirichlet = K.top_dirichlet;
-  return D;
-}
-
-// the row kernels step over x rows, the flat ones over points
-static unsigned grid_for(long long n, int nb) {
-  long long g = (n + 255) / 256;
-  if (g > nb) g = nb;
-  return (unsigned)(g < 1 ? 1 : g);
-}
-
-// blocks of every CG kernel: one x row per block step (at most nb blocks)
-unsigned cg_grid(const CgKernels& K, int nb) { return grid_for((long long)K.nz * K.ny * 256, nb); }
-
-cudaError_t cg_launch(int op, const CgKernels& K, const CgArgs& a, int nb, cudaStream_t st) {
-  const CgDims D = dims_of(K);
-  const unsigned g = cg_grid(K, nb), gr = g;   // every kernel: the same grid, so the host sums g partials
+  CgState* c = (CgState*)a.state;
+  const int sms = cg_sms();
+  long long bx = (D.plane / 2 + 255) / 256;
+  const long long per_level = sms * 8 / K.nz > 1 ? sms * 8 / K.nz : 1;
+  if (bx > per_level) bx = per_level;
+  const dim3 g((unsigned)bx, (unsigned)K.nz);
+  const long long tiles = (long long)((K.nx / 2 + 31) / 32) * ((K.ny + kCgTY - 1) / kCgTY) * ((K.nz + kCgZC - 1) / kCgZC);
+  const unsigned ga = (unsigned)(tiles < sms * 8 ? tiles : sms * 8);
+  const double2 *rho = (const double2*)a.rho, *S = (const double2*)a.S;
+  double2 *r = (double2*)a.r, *d = (double2*)a.d, *q = (double2*)a.q, *p = (double2*)a.p;
+  float2 *rh = (float2*)a.rh, *rl = (float2*)a.rl;
+  double* P = a.partials;
+  if (a.float_pc) {
+    float2* t = (float2*)a.t;
+    const float2* z = (const float2*)a.z;
+    switch (op) {
+      case CG_START: k_cg_start<float><<<g, 256, 0, st>>>(rho, S, r, t, a.lv, D, c, P); return cudaGetLastError();
+      case CG_UPDATE: k_cg_update<float><<<g, 256, 0, st>>>(rh, q, r, t, a.lv, D, c, P); return cudaGetLastError();
+      case CG_DOTS0: k_cg_dots<float, true><<<g, 256, 0, st>>>(z, r, q, D, c, P); return cudaGetLastError();
+      case CG_DOTS: k_cg_dots<float, false><<<g, 256, 0, st>>>(z, r, q, D, c, P); return cudaGetLastError();
+      case CG_DIR:
+        if (a.step == 0) k_cg_dir<float, 0><<<g, 256, 0, st>>>(z, d, p, D, c);
+        else if (a.step == 1) k_cg_dir<float, 1><<<g, 256, 0, st>>>(z, d, p, D, c);
+        else k_cg_dir<float, 2><<<g, 256, 0, st>>>(z, d, p, D, c);
+        return cudaGetLastError();
+      default: break;
+    }
+  } else {
+    double2* t = (double2*)a.t;
+    const double2* z = (const double2*)a.z;
+    switch (op) {
+      case CG_START: k_cg_start<double><<<g, 256, 0, st>>>(rho, S, r, t, a.lv, D, c, P); return cudaGetLastError();
+      case CG_UPDATE: k_cg_update<double><<<g, 256, 0, st>>>(rh, q, r, t, a.lv, D, c, P); return cudaGetLastError();
+      case CG_DOTS0: k_cg_dots<double, true><<<g, 256, 0, st>>>(z, r, q, D, c, P); return cudaGetLastError();
+      case CG_DOTS: k_cg_dots<double, false><<<g, 256, 0, st>>>(z, r, q, D, c, P); return cudaGetLastError();
+      case CG_DIR:
+        if (a.step == 0) k_cg_dir<double, 0><<<g, 256, 0, st>>>(z, d, p, D, c);
+        else if (a.step == 1) k_cg_dir<double, 1><<<g, 256, 0, st>>>(z, d, p, D, c);
+        else k_cg_dir<double, 2><<<g, 256, 0, st>>>(z, d, p, D, c);
+        return cudaGetLastError();
+      default: break;
+    }
+  }
   switch (op) {
-    case CG_WMEAN: k_cg_wmean<<<gr, 256, 0, st>>>(a.rho, a.S, a.dz, D, a.partials); break;
-    case CG_START:
-      k_cg_start<<<gr, 256, 0, st>>>(a.rho, a.S, a.scalar, a.r, a.p, a.t, a.dz, a.lv, D, a.partials);
+    case CG_PREP: k_cg_prep<<<g, 256, 0, st>>>(rho, S, rh, rl, a.lv, D, c, P); break;
+    case CG_APPLY: k_cg_apply<<<ga, 256, 0, st>>>(d, rh, rl, q, a.lv, D, c, P); break;
+    case CG_LAST:
+      if (a.step == 1) k_cg_last<1><<<g, 256, 0, st>>>(d, p, D, c, P);
+      else if (a.step == 2) k_cg_last<2><<<g, 256, 0, st>>>(d, p, D, c, P);
+      else k_cg_last<3><<<g, 256, 0, st>>>(d, p, D, c, P);
       break;
-    case CG_FACES: k_cg_faces<<<gr, 256, 0, st>>>(a.rho, a.ce, a.cn, a.cu, a.lv, D); break;
-    case CG_APPLY: k_cg_apply<<<gr, 256, 0, st>>>(a.d, a.ce, a.cn, a.cu, a.q, D, a.partials); break;
-    case CG_UPDATE:
-      k_cg_update<<<gr, 256, 0, st>>>(a.rho, a.scalar, (float)a.inv_snorm, a.d, a.q, a.p, a.r, a.t, a.lv, D,
-                                      a.partials);
-      break;
-    case CG_DOTS: k_cg_dots<<<g, 256, 0, st>>>(a.z, a.r, a.q, D, a.partials); break;
-    case CG_DIR: k_cg_dir<<<g, 256, 0, st>>>(a.z, a.scalar, a.flag, a.d, D.n); break;
-    case CG_SUM: k_cg_sum<<<g, 256, 0, st>>>(a.p, D.n, a.partials); break;
-    case CG_SHIFT: k_cg_shift<<<g, 256, 0, st>>>(a.p, a.scalar, D.n); break;
+    case CG_SHIFT: k_cg_shift<<<g, 256, 0, st>>>(p, D, c); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
 
-
+cudaError_t cg_read(const void* state, CgReport* out, cudaStream_t st) {
+  CgState h{};
+  cudaError_t e = cudaMemcpyAsync(&h, state, sizeof(h), cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  out->mu = h.mu;
+  out->ss = h.ss;
+  out->dq = h.dq;
+  out->rel2 = h.rel2;
+  return e;
+}
 
 }  // namespace pgb

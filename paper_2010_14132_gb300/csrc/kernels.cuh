@@ -321,42 +321,43 @@ cudaError_t launch_zero_words(void* p, size_t bytes, cudaStream_t st);
 // Four ints from src to dst by a one-thread kernel (dst may be mapped host memory).
 cudaError_t launch_copy_status(const int* src, int* dst, cudaStream_t st);
 // Conjugate gradients for a density varying in x, y and z (cg_kernels.cu).
-enum CgOp { CG_WMEAN = 0, CG_START, CG_APPLY, CG_UPDATE, CG_DOTS, CG_DIR, CG_SUM, CG_SHIFT, CG_FACES };
+enum CgOp { CG_PREP = 0, CG_START, CG_APPLY, CG_UPDATE, CG_DOTS0, CG_DOTS, CG_DIR, CG_LAST, CG_SHIFT };
 struct CgLevel {      // per-level constants, so that no FP64 division runs per point
   double dz;          // dz_k
   double idz;         // 1/dz_k
-  double hup;         // 0.5/h_{k+1/2}; at the top 2/dz_k with p = 0 on the face, else 0
-  double hdn;         // 0.5/h_{k-1/2}; 0 at the bottom
   double iwbar;       // 1/(rho0_k dz_k), the preconditioner's weight
+  float2 kx, ky;      // 0.5 dz_k/dx^2, 0.5 dz_k/dy^2 as float pairs (the 0.5 of the face-density mean folded in)
+  float2 ku;          // 0.5/h_{k+1/2}; at the top 2/dz_k with p = 0 on the face, else 0
 };
-struct CgKernels {
+struct CgGrid {
   int nx, ny, nz;
-  double idx2, idy2;
   int top_dirichlet;
 };
 struct CgArgs {
   const double* rho;    // [nz][ny][nx] density
   const double* S;      // source
-  const double* dz;     // level thicknesses (device)
   const CgLevel* lv;    // per-level constants (device, nz entries)
-  float2* ce;           // face coefficients of W A as float pairs: east, north, upper (CG_FACES writes them)
-  float2* cn;
-  float2* cu;
+  float* rh;            // rho as float pairs, high and low parts (CG_PREP writes them)
+  float* rl;
   double* p;            // iterate
   double* r;            // residual of K p = b
   double* d;            // search direction
   double* q;            // K d
-  double* t;            // preconditioner source -r/Wbar
-  const double* z;      // preconditioned residual
+  void* t;              // preconditioner source -r/Wbar (float or double)
+  const void* z;        // preconditioned residual (float or double)
+  int float_pc;         // 1: t and z are float fields
+  void* state;          // step lengths and sums (device, cg_state_bytes(), zeroed at the start)
   double* partials;     // 2 doubles per block
-  double scalar;        // mu, alpha, beta or shift
-  double inv_snorm;     // 1/||S|| (CG_UPDATE: the residual norm comes out relative)
-  int flag;             // CG_DIR: beta is zero
+  int step;             // CG_DIR, CG_LAST: 0 the first direction, 1 the first step of p, 2 a later one, 3 none
 };
-CgKernels cg_kernels(int nx, int ny, int nz, double dx, double dy, int top_dirichlet);
-cudaError_t cg_launch(int op, const CgKernels& K, const CgArgs& a, int nb, cudaStream_t st);
-int cg_blocks();
-unsigned cg_grid(const CgKernels& K, int nb);
+struct CgReport {
+  double mu, ss, dq, rel2;   // removed mean, ||S||^2, d . K d, squared relative residual
+};
+cudaError_t cg_launch(int op, const CgGrid& K, const CgArgs& a, cudaStream_t st);
+int cg_blocks(int nz);
+size_t cg_state_bytes();
+// Copies the state's report to the host; waits for the stream.
+cudaError_t cg_read(const void* state, CgReport* out, cudaStream_t st);
 
 // dst[b][m][a] = src[a][m][b]: [nx][ny][nz] <-> [nz][ny][nx] field layouts (elem_bytes 4 or 8).
 cudaError_t launch_swap_outer_inner(const void* src, void* dst, int A, int M, int B, int elem_bytes,
