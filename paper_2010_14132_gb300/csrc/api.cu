@@ -106,7 +106,7 @@ struct poisson_plan {
   double* rho_d = nullptr;
   void* tables = nullptr;
   int2* lowk_d = nullptr;
-  double* lowk_inv_d = nullptr;   // pivot reciprocals of the listed columns [n_lowk][nz] (launch_lowk_pivots)
+  double* lowk_inv_d = nullptr;   // pivot reciprocals of the listed columns [2][n_lowk][nz] (launch_lowk_pivots)
   int n_lowk = 0;
   std::vector<int> lowk_kx;     // kx of every listed low-|k| column (host copy)
   int* mid_d = nullptr;         // item list of the fused spectral middle (device)
@@ -174,9 +174,9 @@ int build_lowk(poisson_plan* pl) {
   for (const int2& c : cols) pl->lowk_kx.push_back(c.x);
   if (pl->lowk_inv_d) cudaFree(pl->lowk_inv_d);
   pl->lowk_inv_d = nullptr;
-  PGB_CUDA(cudaMalloc(&pl->lowk_inv_d, (size_t)pl->n_lowk * pl->nz * sizeof(double)));
-  PGB_CUDA(launch_lowk_pivots(pl->lowk_d, pl->n_lowk, pl->tb.a_d, pl->tb.c_d, pl->tb.lamx_d, pl->tb.lamy_d, pl->nz,
-                              !pl->top_dirichlet(), pl->lowk_inv_d, 0));
+  PGB_CUDA(cudaMalloc(&pl->lowk_inv_d, (2 * (size_t)pl->n_lowk * pl->nz + 1) * sizeof(double)));
+  PGB_CUDA(launch_lowk_pivots(pl->lowk_d, pl->n_lowk, pl->tb.a_d, pl->tb.c_d, pl->tb.lamx_d, pl->tb.lamy_d,
+                              pl->tb.W_d, pl->nz, !pl->top_dirichlet(), pl->lowk_inv_d, 0));
   PGB_CUDA(cudaStreamSynchronize(0));
   return POISSON_OK;
 }
@@ -617,8 +617,8 @@ int poisson_plan_set_rho0(poisson_plan* pl, const double* rho0_dev, void* stream
   if (pl->mixed())
     PGB_CUDA(launch_accuracy_floor(tb.a_d, tb.c_d, tb.W_d, pl->nz, pl->nx, pl->ny, pl->g.dx, pl->g.dy,
                                    pl->top_dirichlet(), (double*)tb.floor_d, st));
-  PGB_CUDA(launch_lowk_pivots(pl->lowk_d, pl->n_lowk, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, pl->nz,
-                              !pl->top_dirichlet(), pl->lowk_inv_d, st));
+  PGB_CUDA(launch_lowk_pivots(pl->lowk_d, pl->n_lowk, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d,
+                              tb.W_d, pl->nz, !pl->top_dirichlet(), pl->lowk_inv_d, st));
   return POISSON_OK;
 }
 
@@ -737,9 +737,8 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
   A.adjoint = adjoint;
   A.scale = 1.0 / ((double)pl->nx * pl->ny);
   A.lowk_r2 = pl->mixed() ? pl->lowk_r2 : 0;
-  A.lowk_double = pl->mixed() || t_double;
   A.lowk_cols = pl->lowk_d;
-  A.lowk_inv = A.lowk_double ? pl->lowk_inv_d : nullptr;
+  A.lowk_inv = pl->lowk_inv_d + (size_t)pl->n_lowk * pl->nz;   // the twisted ones
   A.singular00 = !pl->top_dirichlet();
   A.n_lowk = pl->n_lowk;
   A.lowk_z = (double2*)(ws + pl->off_lz);

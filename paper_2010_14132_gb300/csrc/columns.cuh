@@ -29,8 +29,7 @@ struct LowkArgs {
   const double* target_mean;
   double scale;   // 1/(nx ny) in double for the double-precision columns
   int singular00; // zero flux at the top: the (0,0) column is singular
-  const double* inv_tab;   // nullable: [n][nz] pivot reciprocals 1/u_k of the listed columns (double
-                           // columns only), from lowk_pivots; the recurrence then reads them
+  const double* inv_tab;   // [n][nz] twisted pivot reciprocals of the listed columns, then 1/sum W (launch_lowk_pivots)
 };
 
 // One step of the low-|k| pivot recurrence (rounded step by step, so that the table built ahead by
@@ -52,8 +51,7 @@ __device__ __forceinline__ TCm lowk_pivot_step(int k, TCm s, TCm ak, TCm ck, TCm
 }
 
 // ---------------------------------------------------------------------------
-// Low-|k| and singular columns: one thread per listed column, compute type TCm
-// (double in the mixed path), scratch in global memory.  The (0,0) column, when
+// Low-|k| and singular columns, in double.  The (0,0) column, when
 // zero flux at the top makes it singular:
 //   forward: remove the W-weighted mean of the right-hand side (compatibility),
 //            pin x_{nz-1} = 0, back-substitute, shift to zero mean;
@@ -164,154 +162,131 @@ __device__ __forceinline__ void lowk_recurrence(TCm* zx, TCm* zy, TCm* w, int ld
   }
 }
 
-// Shared memory (in units of the compute type) of one low-|k| column solved by a block.
+// Shared memory (in doubles) of one low-|k| column solved by a block.
 __host__ __device__ constexpr size_t lowk_smem_elems(int nz) { return 6 * (size_t)nz + 96; }
 
-// Fixed-order sum of three values over the block (every thread gets the result): each thread's
-// values, then a shuffle tree in each warp, then the warps in order.  scratch: 3 doubles per warp.
-__device__ __forceinline__ double3 lowk_block_sum3(double v0, double v1, double v2, double* scratch) {
-  for (int o = 16; o > 0; o >>= 1) {
-    v0 += __shfl_down_sync(0xffffffffu, v0, o);
-    v1 += __shfl_down_sync(0xffffffffu, v1, o);
-    v2 += __shfl_down_sync(0xffffffffu, v2, o);
-  }
+// Fixed-order sum over the block (every thread gets the result): a shuffle tree in each warp, then the warps in
+// order.  scratch: a double per warp.
+__device__ __forceinline__ double lowk_block_sum(double v, double* scratch) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   const int wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   __syncthreads();   // scratch may still be read from an earlier sum
-  if ((threadIdx.x & 31) == 0) {
-    scratch[3 * wid] = v0;
-    scratch[3 * wid + 1] = v1;
-    scratch[3 * wid + 2] = v2;
-  }
+  if ((threadIdx.x & 31) == 0) scratch[wid] = v;
   __syncthreads();
-  double3 r = make_double3(0.0, 0.0, 0.0);
-  for (int w = 0; w < nw; ++w) {
-    r.x += scratch[3 * w];
-    r.y += scratch[3 * w + 1];
-    r.z += scratch[3 * w + 2];
-  }
+  double r = scratch[0];
+  for (int w = 1; w < nw; ++w) r += scratch[w];
   return r;
 }
 
-// One low-|k| or singular column in double precision from the plan's pivot table (inv_col: 1/u_k,
-// 0 for the pinned singular top), solved by the whole block (at most 1024 threads).  The FP64 units
-// issue a warp's instruction at the same cost however few of its lanes are active, so the serial
-// part is kept to the two recurrences alone: the real parts run on lane 0 and the imaginary parts on
-// lane 1 of the first warp (one double FMA instruction per level and sweep), and everything that
-// does not depend on the previous level (the scaled right-hand side, the elimination and
-// back-substitution factors, the means and sums) runs across the block.
-//   forward  (M x = b):   y_k = b_k + (a_k/u_{k-1}) y_{k-1},  z_k = y_k/u_k,  x_k = z_k + (c_k/u_k) x_{k+1}
-//   adjoint (M^T x = b):  v_k = (b_k + c_{k-1} v_{k-1})/u_k,                  x_k = v_k + (a_{k+1}/u_k) x_{k+1}
+// One low-|k| or singular column in double precision from the plan's table of twisted pivot reciprocals (inv_col,
+// k_lowk_pivots: 1/u_k below level m = nz/2, 1/v_k above it, the meeting pivot's at m, 0 where it is singular and
+// pinned), solved by the whole block (at most 1024 threads).  The FP64 units take a warp's instruction in about 76
+// clocks however few of its lanes are active, so what counts is the length of the serial part: the column is
+// eliminated from both ends at once, real and imaginary parts on lanes 0-1 (upwards) and 2-3 (downwards) of the first
+// warp, one FMA per level and sweep, nz/2 levels each way (eliminated from the bottom alone, twice that: the
+// column kernel of a 64 x 64 x 48 solve 16 -> 10 us, of the first try at 1024 x 1024 x 128 32 -> 27).  Everything
+// that does not depend on the previous level runs across the block:
+//   z_k = b_k/u_k + (e_k/u_k) z_prev,  x_m = (b_m + e_m z_{m-1} + e'_m z_{m+1})/u_m,  x_k = z_k + (r_k/u_k) x_next,
+// with the couplings e (to the eliminated neighbour) and r (to the other): forward e_k = a_k, r_k = c_k below m and
+// c_k, a_k above; adjoint (transposed) e_k = c_{k-1}, r_k = a_{k+1} below and a_{k+1}, c_{k-1} above.
 template <typename TS, bool ADJ>
 __device__ __forceinline__ void lowk_column_tab(unsigned char* smraw, typename CT<TS>::t* __restrict__ spec,
                                                 const Geom& g, const double* __restrict__ ag,
                                                 const double* __restrict__ cg, const double* __restrict__ Wg,
-                                                const double* __restrict__ lamx, const double* __restrict__ lamy,
                                                 double scale, int2 colk, Stats* stats,
                                                 const double* __restrict__ target_mean, bool singular00,
-                                                double* sq_out, const double* __restrict__ inv_col) {
+                                                double* sq_out, const double* __restrict__ inv_col, double inv_sumw) {
   using CS = typename CT<TS>::t;
-  const int nz = g.nz, t = threadIdx.x, nt = blockDim.x;
+  const int nz = g.nz, m = nz / 2, t = threadIdx.x, nt = blockDim.x;
   double* z = reinterpret_cast<double*>(smraw);   // [2][nz]: real parts, imaginary parts
-  double* inv = z + 2 * nz;                        // 1/u_k, then the back-substitution factors
-  double* F = inv + nz;                            // forward factors
-  double* scratch = F + nz;                        // [3 per warp]
+  double* F = z + 2 * nz;                          // elimination factors
+  double* w = F + nz;                              // back-substitution factors
+  double* scratch = w + nz;                        // [3 per warp]
   const int kx = colk.x, ky = colk.y;
   const bool singular = singular00 && kx == 0 && ky == 0;   // nonsingular with p = 0 on the top face
   CS* colp = spec + (long long)ky * g.P + kx;
   // the column is read at L2 (not through L1), so that a persistent kernel that produced it earlier
   // in the same launch on another SM is seen
-  double mx = 0.0, my = 0.0, sw = 0.0;
+  // The mean column is real (it is the horizontal mean of a real field), so only its real part has a mean.  No
+  // division here: 1/nz early, 1/sum W from the table.
+  const double inv_nz = singular ? 1.0 / (double)nz : 0.0;
+  double mean = 0.0;
   for (int k = t; k < nz; k += nt) {
     const CS v = __ldcg(&colp[(long long)k * g.plane]);
     z[k] = (double)v.x;
     z[nz + k] = (double)v.y;
-    inv[k] = __ldg(inv_col + k);
-    if (singular) {   // compatibility: the W-weighted (adjoint: plain) mean of the right-hand side
-      const double wk = ADJ ? 1.0 : __ldg(Wg + k);
-      mx += wk * (double)v.x;
-      my += wk * (double)v.y;
-      sw += wk;
-    }
+    if (singular) mean += (ADJ ? 1.0 : __ldg(Wg + k)) * (double)v.x;
   }
-  double mean_x = 0.0, mean_y = 0.0;
-  if (singular) {
-    const double3 m = lowk_block_sum3(mx, my, sw, scratch);
-    mean_x = m.x / m.z;
-    mean_y = m.y / m.z;
+  if (singular) {   // compatibility: the W-weighted (adjoint: plain) mean of the right-hand side
+    mean = lowk_block_sum(mean, scratch) * (ADJ ? inv_nz : inv_sumw);
     // only the first solve records mu_W (a refinement correction solve has a target mean)
-    if (!ADJ && t == 0 && stats && !target_mean) stats->mu_w = mean_x * scale;
+    if (!ADJ && t == 0 && stats && !target_mean) stats->mu_w = mean * scale;
   }
-  __syncthreads();
   const double ms = -scale;
-  for (int k = t; k < nz; k += nt) {
-    z[k] = ms * (z[k] - mean_x);
-    z[nz + k] = ms * (z[nz + k] - mean_y);
-    F[k] = k == 0 ? 0.0 : (ADJ ? __ldg(cg + k - 1) : __ldg(ag + k) * inv[k - 1]);
+  for (int k = t; k < nz; k += nt) {   // each thread its own levels: no barrier since they were stored
+    const double u = __ldg(inv_col + k), f = k == m ? ms : ms * u;   // b_m is scaled after the meeting
+    z[k] = f * (z[k] - mean);
+    z[nz + k] *= f;
+    const bool up = k > m;
+    // at the ends e is 0 (a_0, and the flux coupling above the top, which has no level to couple to)
+    const double e = ADJ ? (up ? (k + 1 < nz ? __ldg(ag + k + 1) : 0.0) : (k > 0 ? __ldg(cg + k - 1) : 0.0))
+                         : (up ? (k + 1 < nz ? __ldg(cg + k) : 0.0) : __ldg(ag + k));
+    const double r = ADJ ? (up ? __ldg(cg + k - 1) : (k + 1 < nz ? __ldg(ag + k + 1) : 0.0))
+                         : (up ? __ldg(ag + k) : __ldg(cg + k));
+    F[k] = k == m ? e : e * u;    // level m: the couplings themselves (below: F, above: w)
+    w[k] = k == m ? (ADJ ? r : (k + 1 < nz ? r : 0.0)) : r * u;
   }
   __syncthreads();
-  if (t < 2) {   // forward elimination: lane 0 the real parts, lane 1 the imaginary parts
-    double* zp = z + t * nz;
-    double y = ADJ ? zp[0] * inv[0] : zp[0];
-    zp[0] = y;
-    for (int k = 1; k < nz; ++k) {
-      y = fma(F[k], y, zp[k]);
-      if (ADJ) y *= inv[k];
-      zp[k] = y;
+  if (t < 32) {   // lanes 0-3: (part, direction); the others keep the shuffles whole
+    const int part = t & 1, up = (t >> 1) & 1, n = t < 4 ? (up ? nz - 1 - m : m) : 0;
+    double* zp = z + part * nz;
+    const int k0 = up ? nz - 1 : 0, dk = up ? -1 : 1;
+    double y = 0.0;
+    if (n > 0) {
+      double f = F[k0], b = zp[k0];
+      for (int i = 0; i < n; ++i) {
+        const int k = k0 + i * dk;
+        const double fn = F[k + dk], bn = zp[k + dk];   // ahead of this level's store (level m at the end)
+        y = fma(f, y, b);
+        zp[k] = y;
+        f = fn;
+        b = bn;
+      }
+    }
+    const double term = (up ? w[m] : F[m]) * y;
+    const double both = term + __shfl_xor_sync(0xffffffffu, term, 2);
+    double x = (zp[m] + both) * __ldg(inv_col + m);
+    __syncwarp();
+    if (t < 2) zp[m] = x;
+    if (n > 0) {
+      int k = k0 + (n - 1) * dk;
+      double f = w[k], b = zp[k];
+      for (int i = n - 1; i >= 0; --i) {
+        const int kn = i > 0 ? k - dk : k;
+        const double fn = w[kn], bn = zp[kn];
+        x = fma(f, x, b);
+        zp[k] = x;
+        k = kn;
+        f = fn;
+        b = bn;
+      }
     }
   }
   __syncthreads();
-  for (int k = t; k < nz; k += nt) {
-    const double u = inv[k];
-    if (!ADJ) {
-      z[k] *= u;
-      z[nz + k] *= u;
-      inv[k] = __ldg(cg + k) * u;
-    } else {
-      inv[k] = k + 1 < nz ? __ldg(ag + k + 1) * u : 0.0;
-    }
-  }
-  __syncthreads();
-  if (t < 2) {   // back substitution
-    double* zp = z + t * nz;
-    double x = zp[nz - 1];
-    for (int k = nz - 2; k >= 0; --k) {
-      x = fma(inv[k], x, zp[k]);
-      zp[k] = x;
-    }
-  }
-  __syncthreads();
-  double shx = 0.0, shy = 0.0, fx = 0.0, fy = 0.0;
+  double shift = 0.0;   // off the mean column's levels (adjoint: times W_k)
   if (singular) {
-    double sx = 0.0, sy = 0.0, swt = 0.0;
-    for (int k = t; k < nz; k += nt) {
-      sx += z[k];
-      sy += z[nz + k];
-      if (ADJ) swt += __ldg(Wg + k);
-    }
-    const double3 r = lowk_block_sum3(sx, sy, swt, scratch);
-    if (!ADJ) {
-      shx = r.x / (double)nz;
-      shy = r.y / (double)nz;
-      // refinement sweep: the correction also removes the mean of the current iterate
-      if (target_mean) shx += __ldcg(target_mean);
-    } else {   // remove the W direction (the null vector of the transposed column)
-      fx = r.x / r.z;
-      fy = r.y / r.z;
-    }
+    double sx = 0.0;
+    for (int k = t; k < nz; k += nt) sx += z[k];
+    sx = lowk_block_sum(sx, scratch);
+    // adjoint: remove the W direction (the null vector of the transposed column); refinement sweep: the
+    // correction also removes the mean of the current iterate
+    shift = ADJ ? sx * inv_sumw : sx * inv_nz + (target_mean ? __ldcg(target_mean) : 0.0);
   }
   double sq = 0.0;
   for (int k = t; k < nz; k += nt) {
-    double ox = z[k], oy = z[nz + k];
-    if (singular) {
-      if (!ADJ) {
-        ox -= shx;
-        oy -= shy;
-      } else {
-        const double wk = __ldg(Wg + k);
-        ox -= wk * fx;
-        oy -= wk * fy;
-      }
-    }
+    double ox = z[k];
+    const double oy = z[nz + k];
+    if (singular) ox -= ADJ ? __ldg(Wg + k) * shift : shift;
     if (!ADJ && sq_out) sq += ox * ox + oy * oy;
     CS o;
     o.x = (TS)ox;
@@ -319,76 +294,20 @@ __device__ __forceinline__ void lowk_column_tab(unsigned char* smraw, typename C
     colp[(long long)k * g.plane] = o;
   }
   if (!ADJ && sq_out) {
-    const double3 r = lowk_block_sum3(sq, 0.0, 0.0, scratch);
-    if (t == 0) *sq_out = r.x;
+    sq = lowk_block_sum(sq, scratch);
+    if (t == 0) *sq_out = sq;
   }
 }
 
-// One low-|k| or singular column, solved by the whole block.  With the plan's pivot table (double
-// columns) this is lowk_column_tab; otherwise the strided loads and stores of the column and the
-// coefficient tables go through shared memory in parallel and thread 0 runs the sequential
-// recurrence out of shared memory.  sq_out (nullable): the solution's sum of |x_k|^2 over the
-// levels (forward solve), stored by thread 0.  Shared memory: lowk_smem_elems(nz) of TCm.
-template <typename TS, typename TCm, bool ADJ>
+// Listed column `index`, solved by the whole block.  sq_out (nullable): the solution's sum of |x_k|^2 over the levels
+// (forward solve), stored by thread 0.  Shared memory: lowk_smem_elems(nz) doubles.
+template <typename TS, bool ADJ>
 __device__ __forceinline__ void lowk_column(unsigned char* smraw, typename CT<TS>::t* __restrict__ spec,
-                                            const Geom& g, const double* __restrict__ ag,
-                                            const double* __restrict__ cg, const double* __restrict__ Wg,
-                                            const double* __restrict__ lamx, const double* __restrict__ lamy,
-                                            double scale, int2 colk, Stats* stats,
-                                            const double* __restrict__ target_mean, bool singular00,
-                                            double* sq_out = nullptr, const double* inv_tab = nullptr,
-                                            int col_index = 0) {
-  using CS = typename CT<TS>::t;
-  const int nz = g.nz;
-  TCm* zx = reinterpret_cast<TCm*>(smraw);   // right-hand side, then z, then x (real parts)
-  TCm* zy = zx + nz;                          // imaginary parts
-  TCm* w = zy + nz;                           // back-substitution factors
-  TCm* a = w + nz;                            // coefficient tables
-  TCm* c = a + nz;
-  TCm* W = c + nz;
-  TCm* red = W + nz;                          // shift_x, shift_y, sumw, sum_x, sum_y
-  const int kx = colk.x, ky = colk.y;
-  const bool singular = singular00 && kx == 0 && ky == 0;   // nonsingular with p = 0 on the top face
-  CS* colp = spec + (long long)ky * g.P + kx;
-  if (inv_tab && sizeof(TCm) == 8) {   // the plan's pivot table holds double pivots
-    lowk_column_tab<TS, ADJ>(smraw, spec, g, ag, cg, Wg, lamx, lamy, scale, colk, stats, target_mean, singular00,
-                             sq_out, inv_tab + (size_t)col_index * nz);
-    return;
-  }
-  // the column and the target mean are read at L2 (not through L1), so a persistent kernel that
-  // produced them earlier in the same launch on another SM is seen
-  for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-    const CS v = __ldcg(&colp[(long long)k * g.plane]);
-    zx[k] = (TCm)v.x;
-    zy[k] = (TCm)v.y;
-    a[k] = (TCm)ag[k];
-    c[k] = (TCm)cg[k];
-    W[k] = (TCm)Wg[k];
-  }
-  __syncthreads();
-  if (threadIdx.x == 0)
-    lowk_recurrence<TCm, ADJ>(zx, zy, w, 1, a, c, W, nz, kx, ky, singular, lamx, lamy, scale, target_mean, stats,
-                              red, sq_out);
-  __syncthreads();
-  const TCm shift_x = red[0], shift_y = red[1], sumw = red[2], sum_x = red[3], sum_y = red[4];
-  for (int k = threadIdx.x; k < nz; k += blockDim.x) {
-    TCm ox = zx[k], oy = zy[k];
-    if (singular) {
-      if (!ADJ) {
-        ox -= shift_x;
-        oy -= shift_y;
-      } else {
-        // remove the W direction (the null vector of the transposed column)
-        const TCm f = (TCm)W[k] / sumw;
-        ox -= f * sum_x;
-        oy -= f * sum_y;
-      }
-    }
-    CS o;
-    o.x = (TS)ox;
-    o.y = (TS)oy;
-    colp[(long long)k * g.plane] = o;
-  }
+                                            const Geom& g, const LowkArgs& L, int index, Stats* stats,
+                                            double* sq_out = nullptr) {
+  lowk_column_tab<TS, ADJ>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.scale, L.cols[index], stats, L.target_mean,
+                           L.singular00 != 0, sq_out, L.inv_tab + (size_t)index * g.nz,
+                           __ldg(L.inv_tab + (size_t)L.n * g.nz));
 }
 
 // ---------------------------------------------------------------------------
@@ -404,7 +323,9 @@ __device__ __forceinline__ void lowk_column(unsigned char* smraw, typename CT<TS
 // entry in the spectrum (levels plane entries apart).  wp/colp: the column's
 // factor and tile slots.  Shared: ac [nz] (a_k, c_k), meet [TC], xm_s [TC].
 // Returns the sum of |x_k|^2 over the levels the thread wrote (0 when it wrote none).
+// ADJ: the transposed columns (couplings c_{k-1}, a_{k+1} of the neighbouring rows, the same pivots).
 // ---------------------------------------------------------------------------
+template <bool ADJ = false>
 __device__ __forceinline__ float tw_solve_tile(float2* colp, float* wp, const float2* __restrict__ ac, float4* meet,
                                                float2* xm_s, int TC, int nz, int col_t, int upper, bool part,
                                                bool valid, float s, float ms, float2* out, long long plane) {
@@ -419,16 +340,23 @@ __device__ __forceinline__ float tw_solve_tile(float2* colp, float* wp, const fl
       const float f = (k == 0) ? 0.f : akc.x * inv_prev;
       const float gk = (k == 0) ? s : s + f * g_prev;
       const float inv = rcp(gk + akc.y);
-      y = make_float2(fmaf(ms, d.x, f * y.x), fmaf(ms, d.y, f * y.y));
-      colp[(size_t)k * TC] = make_float2(y.x * inv, y.y * inv);
-      wp[(size_t)k * TC] = akc.y * inv;
+      if constexpr (ADJ) {
+        const float cm = (k == 0) ? 0.f : ac[k - 1].y;
+        y = make_float2(fmaf(ms, d.x, cm * y.x) * inv, fmaf(ms, d.y, cm * y.y) * inv);
+        colp[(size_t)k * TC] = y;
+        wp[(size_t)k * TC] = ac[k + 1].x * inv;
+      } else {
+        y = make_float2(fmaf(ms, d.x, f * y.x), fmaf(ms, d.y, f * y.y));
+        colp[(size_t)k * TC] = make_float2(y.x * inv, y.y * inv);
+        wp[(size_t)k * TC] = akc.y * inv;
+      }
       g_prev = gk;
       inv_prev = inv;
     }
     // the level-m terms of the lower part: a_m g_{m-1}/u_{m-1} and a_m z_{m-1}
-    const float am = ac[m].x;
+    const float am = ac[m].x, zm = ADJ ? (m > 0 ? ac[m - 1].y : 0.f) : am;   // adjoint: c_{m-1} z_{m-1}
     const float2 z = (m > 0) ? colp[(size_t)(m - 1) * TC] : make_float2(0.f, 0.f);
-    meet[col_t] = (m > 0) ? make_float4(am * g_prev * inv_prev, am * z.x, am * z.y, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+    meet[col_t] = (m > 0) ? make_float4(am * g_prev * inv_prev, zm * z.x, zm * z.y, 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
   } else if (part) {
     // levels nz-1..m+1, downward elimination with the mirror recurrence
     float h_prev = s, inv_prev = 0.f;
@@ -439,9 +367,16 @@ __device__ __forceinline__ float tw_solve_tile(float2* colp, float* wp, const fl
       const float f = (k == nz - 1) ? 0.f : akc.y * inv_prev;   // c_k / v_{k+1}
       const float hk = (k == nz - 1) ? s + akc.y : s + f * h_prev;
       const float inv = rcp(hk + akc.x);
-      y = make_float2(fmaf(ms, d.x, f * y.x), fmaf(ms, d.y, f * y.y));
-      colp[(size_t)k * TC] = make_float2(y.x * inv, y.y * inv);
-      wp[(size_t)k * TC] = akc.x * inv;
+      if constexpr (ADJ) {
+        const float am = (k == nz - 1) ? 0.f : ac[k + 1].x;
+        y = make_float2(fmaf(ms, d.x, am * y.x) * inv, fmaf(ms, d.y, am * y.y) * inv);
+        colp[(size_t)k * TC] = y;
+        wp[(size_t)k * TC] = ac[k - 1].y * inv;
+      } else {
+        y = make_float2(fmaf(ms, d.x, f * y.x), fmaf(ms, d.y, f * y.y));
+        colp[(size_t)k * TC] = make_float2(y.x * inv, y.y * inv);
+        wp[(size_t)k * TC] = akc.x * inv;
+      }
       h_prev = hk;
       inv_prev = inv;
     }
@@ -456,7 +391,8 @@ __device__ __forceinline__ float tw_solve_tile(float2* colp, float* wp, const fl
     const float4 lo = meet[col_t];
     const float2 dm = colp[(size_t)m * TC];
     const float den = s + lo.x + hterm;
-    const float2 num = make_float2(fmaf(ms, dm.x, lo.y + cm * zt.x), fmaf(ms, dm.y, lo.z + cm * zt.y));
+    const float zu = ADJ ? (m + 1 < nz ? ac[m + 1].x : 0.f) : cm;   // adjoint: a_{m+1} z_{m+1}
+    const float2 num = make_float2(fmaf(ms, dm.x, lo.y + zu * zt.x), fmaf(ms, dm.y, lo.z + zu * zt.y));
     const float2 xm = make_float2(__fdiv_rn(num.x, den), __fdiv_rn(num.y, den));
     xm_s[col_t] = xm;   // this thread has read the h-term; no other thread touches the slot before the barrier
   }

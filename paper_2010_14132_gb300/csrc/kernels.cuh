@@ -249,7 +249,6 @@ struct ThomasArgs {
   int adjoint;
   double scale;           // 1/(nx ny)
   int lowk_r2;            // columns with kx^2+ky'^2 <= lowk_r2 go to the low-k kernel (>= 0)
-  int lowk_double;        // low-k kernel computes in double
   const int2* lowk_cols;  // (kx, ky) list, (0,0) first
   int n_lowk;
   double2* lowk_z;        // scratch nz * n_lowk
@@ -262,7 +261,7 @@ struct ThomasArgs {
   double* sqnorm;             // nullable: per-CTA w-weighted sums of |x|^2 of the solved spectrum (the
                               // two-threads-per-column kernel only); *sqnorm_blocks receives their count
   int* sqnorm_blocks;
-  const double* lowk_inv;     // nullable: the plan's pivot table of the listed columns (double columns only)
+  const double* lowk_inv;     // the plan's twisted pivot table of the listed columns
   int kcut;                   // >= 0 (two-threads-per-column kernel): solve only the columns with kx <= kcut
                               // and |ky'| <= kcut (ky' signed); -1: every column
 };
@@ -406,11 +405,12 @@ int batch_persistent_build(BatchPersistent* bp, const std::vector<BatchDomIn>& d
 cudaError_t batch_persistent_launch(const BatchPersistent& bp, cudaStream_t st);
 void batch_persistent_free(BatchPersistent* bp);
 
-// Pivot reciprocals 1/u_k of the listed low-|k| columns ([n][nz], double), which depend only on the
-// column's wavenumbers and the levels: built once per plan (and per poisson_plan_set_rho0) so that the
-// double column solves run their recurrences without a division on the dependency chain.
+// Pivot reciprocals of the listed low-|k| columns ([2][n][nz], double: eliminated from the bottom, and from both
+// ends; then 1/sum W), which depend only on the column's wavenumbers and the levels: built once per plan (and per
+// poisson_plan_set_rho0) so that the double column solves run their recurrences without a division on the chain.
 cudaError_t launch_lowk_pivots(const int2* cols, int n, const double* a_d, const double* c_d, const double* lamx_d,
-                               const double* lamy_d, int nz, int singular00, double* inv_tab, cudaStream_t st);
+                               const double* lamy_d, const double* W_d, int nz, int singular00, double* inv_tab,
+                               cudaStream_t st);
 // Limiting accuracy F of the mixed refinement from the plan's coefficients (one block; nz <= 512):
 // the relative error that the double-float residual's rounding leaves after any number of sweeps,
 // added to every error bound.  Written to out[0]; out[1] = max_k W_k / min_k W_k (the bound on the

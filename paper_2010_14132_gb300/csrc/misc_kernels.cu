@@ -207,31 +207,63 @@ cudaError_t launch_accuracy_floor(const double* a_d, const double* c_d, const do
 }
 
 // ---------------------------------------------------------------------------
-// Pivot reciprocals of the listed low-|k| columns, one thread per column, with the step the column
-// solves use (lowk_pivot_step), so that reading the table gives the same solution bit for bit.
+// Pivot reciprocals of the listed low-|k| columns, a block per column: tab[0][n][nz], 1/u_k eliminated from the bottom
+// (with the step the sequential column solves use, lowk_pivot_step, so that reading the table gives the same solution
+// bit for bit), and tab[1][n][nz], the twisted ones of lowk_column_tab: 1/u_k below m = nz/2, from the top
+// 1/v_k (h_{nz-1} = s + c_{nz-1}, h_k = s + c_k h_{k+1}/v_{k+1}, v_k = h_k + a_k) above it, and
+// 1/(s + a_m g_{m-1}/u_{m-1} + c_m h_{m+1}/v_{m+1}) at m (0 for the singular column).  A column without row
+// sum (the mean column) has g = h = 0 but for the top coupling: its levels are independent.  After both: 1/sum W.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_lowk_pivots(const int2* __restrict__ cols, int n,
-                                                     const double* __restrict__ a, const double* __restrict__ c,
-                                                     const double* __restrict__ lamx,
-                                                     const double* __restrict__ lamy, int nz, int singular00,
-                                                     double* __restrict__ inv_tab) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
+__global__ void __launch_bounds__(64) k_lowk_pivots(const int2* __restrict__ cols, int n, const double* __restrict__ a,
+                                                    const double* __restrict__ c, const double* __restrict__ lamx,
+                                                    const double* __restrict__ lamy, const double* __restrict__ W,
+                                                    int nz, int singular00, double* __restrict__ tab) {
+  const int j = blockIdx.x, t = threadIdx.x, m = nz / 2;
+  if (j == 0 && t < 32) {
+    double sw = 0.0;
+    for (int k = t; k < nz; k += 32) sw += W[k];
+    for (int o = 16; o > 0; o >>= 1) sw += __shfl_down_sync(0xffffffffu, sw, o);
+    if (t == 0) tab[2 * (size_t)n * nz] = 1.0 / sw;
+  }
   const int2 ck = cols[j];
   const bool singular = singular00 && ck.x == 0 && ck.y == 0;
   const double s = singular ? 0.0 : -(lamx[ck.x] + lamy[ck.y]);
-  double g_prev = s, inv_prev = 0.0;
-  for (int k = 0; k < nz; ++k) {
-    const double inv = lowk_pivot_step<double>(k, s, a[k], c[k], g_prev, inv_prev, singular && (k == nz - 1));
-    inv_tab[(size_t)j * nz + k] = inv;
-    inv_prev = inv;
+  double* lower = tab + (size_t)j * nz;
+  double* tw = tab + (size_t)(n + j) * nz;
+  __shared__ double meet[2];   // g_{m-1}/u_{m-1}, h_{m+1}/v_{m+1}
+  if (s == 0.0) {
+    for (int k = t; k < nz; k += blockDim.x) lower[k] = singular && k == nz - 1 ? 0.0 : 1.0 / c[k];
+    if (t == 0) meet[0] = 0.0;
+  } else if (t == 0) {
+    double g_prev = s, inv_prev = 0.0;
+    for (int k = 0; k < nz; ++k) {
+      const double inv = lowk_pivot_step<double>(k, s, a[k], c[k], g_prev, inv_prev, false);
+      lower[k] = inv;
+      inv_prev = inv;
+      if (k == m - 1) meet[0] = g_prev * inv;
+    }
   }
+  if (singular) {   // h = 0 throughout
+    for (int k = m + 1 + t; k < nz; k += blockDim.x) tw[k] = 1.0 / a[k];
+    if (t == 32) meet[1] = m + 1 < nz ? 0.0 : 1.0;
+  } else if (t == 32) {
+    double ratio = 1.0;   // above the top: the face's coupling enters the top row's sum
+    for (int k = nz - 1; k > m; --k) {
+      const double h = s + c[k] * ratio, inv = 1.0 / (h + a[k]);
+      tw[k] = inv;
+      ratio = h * inv;
+    }
+    meet[1] = ratio;
+  }
+  __syncthreads();
+  for (int k = t; k < m; k += blockDim.x) tw[k] = lower[k];
+  if (t == 0) tw[m] = singular ? 0.0 : 1.0 / (s + a[m] * meet[0] + c[m] * meet[1]);
 }
-
 cudaError_t launch_lowk_pivots(const int2* cols, int n, const double* a_d, const double* c_d, const double* lamx_d,
-                               const double* lamy_d, int nz, int singular00, double* inv_tab, cudaStream_t st) {
+                               const double* lamy_d, const double* W_d, int nz, int singular00, double* inv_tab,
+                               cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_lowk_pivots<<<(n + 127) / 128, 128, 0, st>>>(cols, n, a_d, c_d, lamx_d, lamy_d, nz, singular00, inv_tab);
+  k_lowk_pivots<<<n, 64, 0, st>>>(cols, n, a_d, c_d, lamx_d, lamy_d, W_d, nz, singular00, inv_tab);
   return cudaGetLastError();
 }
 
@@ -301,16 +333,17 @@ __global__ void __launch_bounds__(256) k_control(Stats* st, const double* __rest
 // Verification of the current iterate by the next correction's norm (see launch_verify in
 // kernels.cuh).  One block; fixed-order sums.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_verify(Stats* st, const double* __restrict__ sq, int nsq,
-                                                 const double* __restrict__ res_partials, int res_nblocks, int pass,
-                                                 double tol, const double* __restrict__ floor, double nxny,
-                                                 int p_stored, double inv_lcut2, int from_r0) {
-  __shared__ double sh[3][1024];
+constexpr int kVerifyThreads = 256;
+__global__ void __launch_bounds__(kVerifyThreads) k_verify(Stats* st, const double* __restrict__ sq, int nsq,
+                                                           const double* __restrict__ res_partials, int res_nblocks,
+                                                           int pass, double tol, const double* __restrict__ floor,
+                                                           double nxny, int p_stored, double inv_lcut2, int from_r0) {
+  __shared__ double sh[3][kVerifyThreads];
   if (st->done) return;   // an earlier pass already ended the refinement
   const int t = threadIdx.x;
   double a = 0, b = 0, c = 0;
-  for (int i = t; i < nsq; i += blockDim.x) a += sq[i];
-  for (int i = t; i < res_nblocks; i += blockDim.x) {
+  for (int i = t; i < nsq; i += kVerifyThreads) a += sq[i];
+  for (int i = t; i < res_nblocks; i += kVerifyThreads) {
     b += res_partials[2 * i];
     c += res_partials[2 * i + 1];
   }
@@ -318,14 +351,17 @@ __global__ void __launch_bounds__(1024) k_verify(Stats* st, const double* __rest
   sh[1][t] = b;
   sh[2][t] = c;
   __syncthreads();
-  for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-    if (t < h) {
-      sh[0][t] += sh[0][t + h];
-      sh[1][t] += sh[1][t + h];
-      sh[2][t] += sh[2][t + h];
-    }
-    __syncthreads();
+  // one warp per sum: the FP64 unit takes a warp's addition in 76 clocks, so what counts is their number in a row
+  // (a tree over 1024 threads: 8.7 -> 7.2 us at 64 x 64 x 48)
+  if (t < 96) {
+    const int q = t >> 5;
+    double x = 0.0;
+    for (int i = t & 31; i < kVerifyThreads; i += 32) x += sh[q][i];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    __syncwarp();
+    if ((t & 31) == 0) sh[q][0] = x;
   }
+  __syncthreads();
   if (t != 0) return;
   double sd = nxny * sh[0][0];
   // low wavenumbers only: every other column of the correction is (lambda_h + T)^{-1} of the residual's
@@ -348,7 +384,7 @@ __global__ void __launch_bounds__(1024) k_verify(Stats* st, const double* __rest
 cudaError_t launch_verify(Stats* st_dev, const double* sq, int nsq, const double* res_partials, int res_nblocks,
                           int pass, double tol, const double* floor, double nxny, int p_stored, double inv_lcut2,
                           int from_r0, cudaStream_t st) {
-  k_verify<<<1, 1024, 0, st>>>(st_dev, sq, nsq, res_partials, res_nblocks, pass, tol, floor, nxny, p_stored,
+  k_verify<<<1, kVerifyThreads, 0, st>>>(st_dev, sq, nsq, res_partials, res_nblocks, pass, tol, floor, nxny, p_stored,
                                inv_lcut2, from_r0);
   return cudaGetLastError();
 }

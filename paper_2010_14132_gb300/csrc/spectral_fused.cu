@@ -87,7 +87,7 @@ __host__ __device__ constexpr size_t mid_buf_bytes(int N, int nz, int TC, size_t
   return y > c ? (y > l ? y : l) : (c > l ? c : l);
 }
 
-template <int N, int TC, typename TCm>
+template <int N, int TC>
 __global__ void __launch_bounds__(kMidTK * (N / kMidE), 2)
     k_mid(const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmc, MidArgs A) {
   using C = float2;
@@ -203,9 +203,7 @@ __global__ void __launch_bounds__(kMidTK * (N / kMidE), 2)
         tw_solve_tile(tile + col_t, wv + col_t, ac, meet, xm_s, TC, nz, col_t, upper, part, valid, sv, -A.scale,
                       A.spec + (valid ? (long long)ky * g.P + kx : 0), g.plane);
       } else {   // MID_L
-        lowk_column<float, TCm, false>(buf, A.spec, g, A.L.a_d, A.L.c_d, A.L.W_d, A.L.lamx_d, A.L.lamy_d, A.L.scale,
-                                       A.L.cols[sub], A.stats, A.L.target_mean, A.L.singular00 != 0, nullptr,
-                                       A.L.inv_tab, sub);
+        lowk_column<float, false>(buf, A.spec, g, A.L, sub, A.stats);
       }
     }
     // the item's shared-memory accesses precede the next TMA write into the buffer, and its spectrum
@@ -319,7 +317,7 @@ cudaError_t launch_spectral_fused(const ThomasArgs& T, const Geom& g, const FftP
   A.box_z = box_z;
   A.done = T.done;
   A.stats = T.stats;
-  const size_t lowk_elem = T.lowk_double ? 8 : 4;
+  const size_t lowk_elem = sizeof(double);
   const size_t smem = mid_buf_offset(g.ny, g.nz) + mid_buf_bytes(g.ny, g.nz, tc, lowk_elem);
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -351,9 +349,9 @@ cudaError_t launch_spectral_fused(const ThomasArgs& T, const Geom& g, const FftP
   case NN: {                                                                                              \
     constexpr int nt = kMidTK * (NN / kMidE);                                                             \
     if (tc == 64 && 2 * 64 <= nt)                                                                         \
-      e = T.lowk_double ? run(k_mid<NN, 64, double>, nt) : run(k_mid<NN, 64, float>, nt);                 \
+      e = run(k_mid<NN, 64>, nt);                 \
     else                                                                                                  \
-      e = T.lowk_double ? run(k_mid<NN, 32, double>, nt) : run(k_mid<NN, 32, float>, nt);                 \
+      e = run(k_mid<NN, 32>, nt);                 \
   } break;
   switch (g.ny) {
     PGB_MID_CASE(256)

@@ -27,10 +27,10 @@ namespace pgb {
 // Main column kernel: one thread per column, a tile of TC consecutive columns
 // (flattened (ky, kx) index with pitch P) staged for all nz levels.
 // Shared layout: tile [nz][TC] complex, wv [nz][TC] real, one mbarrier.
-// Blocks [0, L.n) solve the listed low-|k| / singular columns (precision TCm);
+// Blocks [0, L.n) solve the listed low-|k| / singular columns (double);
 // the others solve tiles of TC consecutive columns.  The two sets of columns are
 // disjoint (the tile blocks skip listed columns), so they run concurrently.
-template <typename T, typename TCm, bool ADJ>
+template <typename T, bool ADJ>
 __global__ void __launch_bounds__(128) k_thomas(typename CT<T>::t* __restrict__ spec, Geom g,
                                                 const T* __restrict__ a, const T* __restrict__ c,
                                                 const T* __restrict__ lamx, const T* __restrict__ lamy, T scale,
@@ -41,9 +41,7 @@ __global__ void __launch_bounds__(128) k_thomas(typename CT<T>::t* __restrict__ 
   if (done && *done) return;
   extern __shared__ __align__(128) unsigned char smraw[];
   if ((int)blockIdx.x < L.n) {
-    lowk_column<T, TCm, ADJ>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.lamx_d, L.lamy_d, L.scale,
-                             L.cols[blockIdx.x], stats, L.target_mean, L.singular00 != 0, nullptr, L.inv_tab,
-                             blockIdx.x);
+    lowk_column<T, ADJ>(smraw, spec, g, L, blockIdx.x, stats);
     return;
   }
   const int TC = blockDim.x, t = threadIdx.x, nz = g.nz;
@@ -202,7 +200,7 @@ __device__ __forceinline__ void column_solve_pair(float2* ca, float2* cb, float*
   }
 }
 
-template <typename TCm, bool ADJ>
+template <bool ADJ>
 __global__ void __launch_bounds__(64) k_thomas_pair(float2* __restrict__ spec, Geom g, const float* __restrict__ a,
                                                     const float* __restrict__ c, const float* __restrict__ lamx,
                                                     const float* __restrict__ lamy, float scale, int lowk_r2,
@@ -212,9 +210,7 @@ __global__ void __launch_bounds__(64) k_thomas_pair(float2* __restrict__ spec, G
   if (done && *done) return;
   extern __shared__ __align__(128) unsigned char smraw[];
   if ((int)blockIdx.x < L.n) {
-    lowk_column<float, TCm, ADJ>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.lamx_d, L.lamy_d, L.scale,
-                                 L.cols[blockIdx.x], stats, L.target_mean, L.singular00 != 0, nullptr, L.inv_tab,
-                                 blockIdx.x);
+    lowk_column<float, ADJ>(smraw, spec, g, L, blockIdx.x, stats);
     return;
   }
   const int TC = blockDim.x, t = threadIdx.x, nz = g.nz;
@@ -260,7 +256,8 @@ __global__ void __launch_bounds__(64) k_thomas_pair(float2* __restrict__ spec, G
 
 
 // ---------------------------------------------------------------------------
-// Twisted FP32 column kernel (forward solves): two threads per column.  The
+// Twisted FP32 column kernel: two threads per column (forward and adjoint; the adjoint with paired columns and
+// one chain each took 40 us at 512 x 512 x 64, so 29.6).  The
 // lower thread eliminates levels 0..m-1 upward with the pivots above
 // (g_k, u_k = g_k + c_k), the upper thread eliminates levels nz-1..m+1 downward
 // with the mirror recurrence h_{nz-1} = s + c_{nz-1} (the top row's sum: c_{nz-1} = 0
@@ -280,7 +277,7 @@ __global__ void __launch_bounds__(64) k_thomas_pair(float2* __restrict__ spec, G
 // |ky'| <= kcut are solved; the grid then holds just their tiles, ceil((kcut + 1)/TC) from the start
 // of each of the rows ky = 0..kcut and ny - kcut..ny - 1 (P, a multiple of 16, keeps every tile's
 // first entry 16-byte aligned for the TMA box).
-template <typename TCm>
+template <bool ADJ>
 __global__ void __launch_bounds__(128) k_thomas_tw(float2* __restrict__ spec, Geom g, const float* __restrict__ a,
                                                   const float* __restrict__ c, const float* __restrict__ lamx,
                                                   const float* __restrict__ lamy, float scale, int lowk_r2,
@@ -294,8 +291,7 @@ __global__ void __launch_bounds__(128) k_thomas_tw(float2* __restrict__ spec, Ge
   if ((int)blockIdx.x < L.n) {
     double sq = 0.0;
     const int2 ck = L.cols[blockIdx.x];
-    lowk_column<float, TCm, false>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.lamx_d, L.lamy_d, L.scale, ck, stats,
-                                   L.target_mean, L.singular00 != 0, sqn ? &sq : nullptr, L.inv_tab, blockIdx.x);
+    lowk_column<float, ADJ>(smraw, spec, g, L, blockIdx.x, stats, sqn ? &sq : nullptr);
     if (sqn && threadIdx.x == 0) sqn[blockIdx.x] = (ck.x == 0 || ck.x == g.nxh - 1 ? 1.0 : 2.0) * sq;
     return;
   }
@@ -337,7 +333,7 @@ __global__ void __launch_bounds__(128) k_thomas_tw(float2* __restrict__ spec, Ge
   const bool valid = col < g.plane && kx < g.nxh && (kx * kx + kys * kys > lowk_r2) &&
                      (kcut < 0 || (kx <= kcut && low_row(ky)));
   const float s = valid ? -(lamx[kx] + lamy[ky]) : 1.f;
-  const float sq = tw_solve_tile(tile + col_t, wv + col_t, ac, meet, xm_s, TC, nz, col_t, upper, true, valid, s,
+  const float sq = tw_solve_tile<ADJ>(tile + col_t, wv + col_t, ac, meet, xm_s, TC, nz, col_t, upper, true, valid, s,
                                  -scale, spec + (valid ? col : 0), g.plane);
   if (sqn) {   // fixed-order CTA sum of the weighted squares (in the drained tile's shared memory)
     float v = (kx == 0 || kx == g.nxh - 1) ? sq : 2.f * sq;
@@ -422,9 +418,7 @@ __global__ void __launch_bounds__(32) k_thomas_d(double2* __restrict__ spec, Geo
   extern __shared__ __align__(128) unsigned char smraw[];
   if ((int)blockIdx.x < L.n) {
     pdl_wait();
-    lowk_column<double, double, ADJ>(smraw, spec, g, L.a_d, L.c_d, L.W_d, L.lamx_d, L.lamy_d, L.scale,
-                                     L.cols[blockIdx.x], stats, L.target_mean, L.singular00 != 0, nullptr, L.inv_tab,
-                                     blockIdx.x);
+    lowk_column<double, ADJ>(smraw, spec, g, L, blockIdx.x, stats);
     return;
   }
   const int t = threadIdx.x, nz = g.nz, m = nz / 2;
@@ -520,8 +514,8 @@ static int thomas_tile(int nz, size_t entry_bytes, int request) {
   return 0;
 }
 
-// Paired FP32 column kernel (col_tile = 0, the default); *used = false when it does not fit.
-template <typename TCm, bool ADJ>
+// Paired FP32 column kernel (col_tile = 3); *used = false when it does not fit.
+template <bool ADJ>
 static cudaError_t thomas_pair_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, cudaStream_t st,
                                       bool* used) {
   *used = false;
@@ -540,7 +534,7 @@ static cudaError_t thomas_pair_launch(const ThomasArgs& A, const Geom& g, const 
   }
   size_t smem = 2 * (size_t)g.nz * tc * sizeof(float2) + (((size_t)g.nz * tc * sizeof(float) + 15) & ~(size_t)15) +
                 ((size_t)g.nz + 1) * sizeof(float2) + 16;
-  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(TCm);
+  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(double);
   if (smem < lowk_smem) smem = lowk_smem;
   int box_rows = 1;
   for (int d = 256; d >= 1; --d)
@@ -553,7 +547,7 @@ static cudaError_t thomas_pair_launch(const ThomasArgs& A, const Geom& g, const 
   if (!encode_tensor_2d(&tm, A.spec, 8, (unsigned long long)g.plane, (unsigned long long)g.nz,
                         (unsigned long long)g.plane * sizeof(float2), (unsigned)tc, (unsigned)box_rows))
     return cudaSuccess;
-  auto kern = k_thomas_pair<TCm, ADJ>;
+  auto kern = k_thomas_pair<ADJ>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int kx_chunks = (g.nxh + tc - 1) / tc;
@@ -568,14 +562,14 @@ static cudaError_t thomas_pair_launch(const ThomasArgs& A, const Geom& g, const 
   return cudaGetLastError();
 }
 
-// Twisted FP32 column kernel for forward solves; *used = false when it does not fit.
-template <typename TCm>
+// Twisted FP32 column kernel (col_tile = 0, the default); *used = false when it does not fit.
+template <bool ADJ>
 static cudaError_t thomas_tw_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, int tc, cudaStream_t st,
                                     bool* used) {
   *used = false;
   size_t smem = (((size_t)g.nz * tc * (sizeof(float2) + sizeof(float)) + 15) & ~(size_t)15) +
                 ((size_t)g.nz + 1) * sizeof(float2) + (size_t)tc * (sizeof(float4) + sizeof(float2)) + 16;
-  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(TCm);
+  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(double);
   if (smem < lowk_smem) smem = lowk_smem;
   if (smem > 200 * 1024) return cudaSuccess;
   int box_rows = 1;
@@ -589,7 +583,7 @@ static cudaError_t thomas_tw_launch(const ThomasArgs& A, const Geom& g, const Ta
   if (!encode_tensor_2d(&tm, A.spec, 8, (unsigned long long)g.plane, (unsigned long long)g.nz,
                         (unsigned long long)g.plane * sizeof(float2), (unsigned)tc, (unsigned)box_rows))
     return cudaSuccess;
-  auto kern = k_thomas_tw<TCm>;
+  auto kern = k_thomas_tw<ADJ>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // every tile of the plane, or (kcut >= 0) the low rows' first ceil((kcut + 1)/tc) tiles
@@ -634,31 +628,31 @@ static cudaError_t thomas_d_launch(const ThomasArgs& A, const Geom& g, const Tab
   return thomas_d_nr<1, ADJ>(A, g, tb, 2 * cols, st);
 }
 
-template <typename T, typename TCm, bool ADJ>
+template <typename T, bool ADJ>
 static cudaError_t thomas_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, const T* a, const T* c,
                                  const T* lx, const T* ly, cudaStream_t st) {
   using C = typename CT<T>::t;
   if constexpr (sizeof(T) == 4) {
-    if (!ADJ && (A.col_tile <= 2 || A.col_tile == 4)) {
+    if (A.col_tile <= 2 || A.col_tile == 4) {
       // twisted two-thread columns: 32 columns per CTA by default (col_tile 0 or 2), 16 (1) or 64 (4)
       const int tc = A.col_tile == 1 ? 16 : (A.col_tile == 4 ? 64 : 32);
       bool used = false;
-      cudaError_t e = thomas_tw_launch<TCm>(A, g, tb, tc, st, &used);
+      cudaError_t e = thomas_tw_launch<ADJ>(A, g, tb, tc, st, &used);
       if (e != cudaSuccess || used) return e;
     }
     if (A.col_tile == 0 || A.col_tile == 3) {
       bool used = false;
-      cudaError_t e = thomas_pair_launch<TCm, ADJ>(A, g, tb, st, &used);
+      cudaError_t e = thomas_pair_launch<ADJ>(A, g, tb, st, &used);
       if (e != cudaSuccess || used) return e;
     }
   }
   const int tc = thomas_tile(g.nz, sizeof(C) + sizeof(T), A.col_tile);
   if (tc == 0) return cudaErrorInvalidValue;
   size_t smem = (((size_t)g.nz * tc * (sizeof(C) + sizeof(T)) + 15) & ~(size_t)15) + 16;
-  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(TCm);
+  const size_t lowk_smem = lowk_smem_elems(g.nz) * sizeof(double);
   if (smem < lowk_smem) smem = lowk_smem;
   const long long nb = (g.plane + tc - 1) / tc;
-  auto kern = k_thomas<T, TCm, ADJ>;
+  auto kern = k_thomas<T, ADJ>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // the spectrum as a 2-D tensor: a level's ny*P entries per row, nz rows
@@ -687,13 +681,10 @@ cudaError_t launch_thomas(const ThomasArgs& A, const Geom& g, const Tables& tb, 
   if (A.t_is_double && A.col_tile < 16 && !A.done)
     return A.adjoint ? thomas_d_launch<true>(A, g, tb, st) : thomas_d_launch<false>(A, g, tb, st);
   if (A.t_is_double)
-    return A.adjoint ? thomas_launch<double, double, true>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st)
-                     : thomas_launch<double, double, false>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st);
-  if (A.lowk_double)
-    return A.adjoint ? thomas_launch<float, double, true>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st)
-                     : thomas_launch<float, double, false>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st);
-  return A.adjoint ? thomas_launch<float, float, true>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st)
-                   : thomas_launch<float, float, false>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st);
+    return A.adjoint ? thomas_launch<double, true>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st)
+                     : thomas_launch<double, false>(A, g, tb, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, st);
+  return A.adjoint ? thomas_launch<float, true>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st)
+                   : thomas_launch<float, false>(A, g, tb, tb.a_f, tb.c_f, tb.lamx_f, tb.lamy_f, st);
 }
 
 }  // namespace pgb

@@ -209,13 +209,17 @@ __global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_
       sums[3 * TH + tid] = a3;
       sums[4 * TH + tid] = a4;
       __syncthreads();
-      for (int h = xs_max_threads(E) / 2; h > 0; h >>= 1) {
-        if (tid < h && tid + h < TH) {
-#pragma unroll
-          for (int v = 0; v < 5; ++v) sums[v * TH + tid] += sums[v * TH + tid + h];
-        }
-        __syncthreads();
+      // one warp per sum: TH/32 values a lane, then a shuffle tree (12 FP64 instructions one after the other and two
+      // barriers; a tree over the block took 40 and eight)
+      constexpr int NW = TH / 32;
+      for (int q = tid >> 5; q < 5 && tid < NW * 32; q += NW) {
+        double x = 0.0;
+        for (int i = tid & 31; i < TH; i += 32) x += sums[q * TH + i];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+        __syncwarp();
+        if ((tid & 31) == 0) sums[q * TH] = x;
       }
+      __syncthreads();
       if (tid == 0) {
         ex.ctl_stats->control_ticket = 0u;   // ready for the next pass
         control_decide(ex.ctl_stats, sums[0], sums[TH], sums[2 * TH], sums[3 * TH], sums[4 * TH], ex.ctl_pass,
