@@ -55,18 +55,23 @@ template <typename TI> __device__ __forceinline__ float to_f(TI x);
 template <> __device__ __forceinline__ float to_f<float>(float x) { return x; }
 template <> __device__ __forceinline__ float to_f<double>(double x) { return d2f_int(x); }
 
-// Shared layout: twiddles (n/2), unpack twiddles (n/2 + 2), RB rows x 2 line
-// buffers (none when the lines alias the staged rows), then the staging ring
-// (128-byte aligned) and its mbarriers.  A staged row of nx doubles holds
-// exactly the two n/2-point line buffers of its own row, so kernels that stage
-// double rows run the transform inside the consumed row.
+// Shared layout: twiddles (n/2), unpack twiddles (half a line of them for the forward kernels, a line for the inverse),
+// the line buffers that do not fit the staged rows, then the
+// staging ring (128-byte aligned) and its mbarriers.  A staged row of nx doubles holds exactly the two n/2-point line
+// buffers of its own row (XS_ALIAS_TWO); a row of nx floats, or of n/2 + 1 spectrum bins, holds one of them, the
+// one that the second stage writes, when every input has long been read (XS_ALIAS_ONE; lines with a factor 3, whose
+// registers allow two CTAs per SM either way, keep both buffers).  What that saves makes room for a fourth
+// CTA per SM or a deeper ring (FP32 solve of 256 x 256 x 64: 53.1 -> 50.3 us; forward pass at 1024 x 1024 x 128 232 ->
+// 211).  The mixed path's inverse epilogues are held to three CTAs by their registers and keep both buffers.
+enum XsAlias { XS_ALIAS_NONE = 0, XS_ALIAS_ONE = 1, XS_ALIAS_TWO = 2 };
 struct XsLayout {
   size_t off_stage, off_bar, total;
 };
 __host__ __device__ constexpr size_t xs_align(size_t x, size_t a) { return (x + a - 1) / a * a; }
-__host__ __device__ inline XsLayout xs_layout(int N, int RB, int ns, unsigned stage_bytes, bool alias) {
+__host__ __device__ constexpr XsAlias xs_alias_float(int E) { return E % 3 == 0 ? XS_ALIAS_NONE : XS_ALIAS_ONE; }
+__host__ __device__ inline XsLayout xs_layout(int N, int RB, int ns, unsigned stage_bytes, XsAlias alias, bool inverse) {
   XsLayout L{};
-  size_t off = (size_t)N * 8 + (size_t)(N + 2) * 8 + (alias ? 0 : (size_t)RB * 2 * N * 8);
+  size_t off = (size_t)N * 8 + (size_t)((inverse ? N : N / 2) + 2) * 8 + (size_t)RB * (2 - (int)alias) * N * 8;
   L.off_stage = xs_align(off, 128);
   L.off_bar = xs_align(L.off_stage + (size_t)ns * stage_bytes, 8);
   L.total = L.off_bar + (size_t)ns * 8;
@@ -140,24 +145,24 @@ struct XsConfig {
   size_t smem = 0;
 };
 
-// Staging depth and CTAs per SM: the most CTAs per SM (up to three) whose
+// Staging depth and CTAs per SM: the most CTAs per SM (up to max_ctas) whose
 // shared memory still allows two stages, then the deepest ring (up to four
 // stages) at that CTA count.
-XsConfig xs_config(int N, int E, unsigned stage_bytes, size_t static_smem, bool alias) {
+XsConfig xs_config(int N, int E, unsigned stage_bytes, size_t static_smem, XsAlias alias, bool inverse, int max_ctas) {
   const int RB = xs_rows(N, E);
   constexpr size_t kSmPerSm = 228 * 1024, kReserved = 1024, kMaxPerCta = 227 * 1024;
   XsConfig c{};
   c.stage_bytes = stage_bytes;
-  for (int ctas = 3; ctas >= 1 && c.ns == 0; --ctas) {
+  for (int ctas = max_ctas; ctas >= 1 && c.ns == 0; --ctas) {
     size_t budget = kSmPerSm / ctas - kReserved - static_smem;
     if (budget > kMaxPerCta - static_smem) budget = kMaxPerCta - static_smem;
     for (int ns = kXsMaxStages; ns >= 2; --ns)
-      if (xs_layout(N, RB, ns, stage_bytes, alias).total <= budget) {
+      if (xs_layout(N, RB, ns, stage_bytes, alias, inverse).total <= budget) {
         c.ns = ns;
         break;
       }
   }
-  if (c.ns) c.smem = xs_layout(N, RB, c.ns, stage_bytes, alias).total;
+  if (c.ns) c.smem = xs_layout(N, RB, c.ns, stage_bytes, alias, inverse).total;
   return c;
 }
 

@@ -17,13 +17,13 @@ __global__ void __launch_bounds__(xs_max_threads(E)) k_xfwd_s(const TI* __restri
   using C = float2;
   using TI2 = typename V2s<TI>::t;
   constexpr int nl = N / E, RB = xs_rows(N, E), LS = N;
-  constexpr bool ALIAS = sizeof(TI) == 8;
+  constexpr XsAlias ALIAS = sizeof(TI) == 8 ? XS_ALIAS_TWO : xs_alias_float(E);
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
-  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, ALIAS);
+  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, ALIAS, false);
   C* tw_s = reinterpret_cast<C*>(smraw);
   C* twr_s = tw_s + N;
-  C* lines = twr_s + N + 2;
+  C* lines = twr_s + N / 2 + 2;
   unsigned char* stg = smraw + L.off_stage;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + L.off_bar);
 
@@ -56,15 +56,18 @@ __global__ void __launch_bounds__(xs_max_threads(E)) k_xfwd_s(const TI* __restri
     }
   const LineSyncT<nl> sync{1 + ty};
   const LineAddr<N> sw{};
-  C* la = lines + (size_t)ty * 2 * LS;
+  C* la = lines + (size_t)ty * (ALIAS == XS_ALIAS_ONE ? 1 : 2) * LS;
   C* lb = la + LS;
   bool ok = true;
   int it = 0;
   for (long long grp = blockIdx.x; grp < ngroups; grp += gridDim.x, ++it) {
     const int s = it % ns;
-    if constexpr (ALIAS) {   // this row's two line buffers are its staged row
-      la = reinterpret_cast<C*>(stg + (size_t)s * stage_bytes + (size_t)ty * row_bytes);
-      lb = la + LS;
+    if constexpr (ALIAS != XS_ALIAS_NONE) {   // one or both of this row's line buffers are its staged row
+      lb = reinterpret_cast<C*>(stg + (size_t)s * stage_bytes + (size_t)ty * row_bytes);
+      if constexpr (ALIAS == XS_ALIAS_TWO) {
+        la = lb;
+        lb = la + LS;
+      }
     }
     const bool got = mbar_wait_bounded(&bar[s], (unsigned)((it / ns) & 1), kWaitPolls);
     if (!__syncthreads_and(got)) {
@@ -90,11 +93,11 @@ __global__ void __launch_bounds__(xs_max_threads(E)) k_xfwd_s(const TI* __restri
       const TI2 x = srow[st_in_index<N, E, 0>(lane, i)];
       v[i] = make_float2(to_f<TI>(x.x), to_f<TI>(x.y));
     }
-    if constexpr (ALIAS) sync();   // the line's threads have read the row before it is overwritten
+    if constexpr (ALIAS == XS_ALIAS_TWO) sync();   // the line's threads have read the row before it is overwritten
     const C* fin = st_fft<N, E, -1, false, float>(v, la, lb, sw, lane, tw_s, sync);
     r2c_unpack_store<N, E>(fin, twr_s, spec + (valid ? row : 0) * g.P, lane, valid);
     // the staged row was written through the generic proxy; order that before its refill by TMA
-    if constexpr (ALIAS) fence_proxy_async_smem();
+    if constexpr (ALIAS != XS_ALIAS_NONE) fence_proxy_async_smem();
   }
   if (tid == 0) {
     if (!ok) atomicOr(err, (unsigned)ERR_WAIT_TIMEOUT);
@@ -107,7 +110,8 @@ cudaError_t xfwd_s(const TI* in, float2* spec, const Geom& g, int N, int E, cons
                    unsigned* err, cudaStream_t st, bool* used) {
   const int RB = xs_rows(N, E);
   const unsigned row_bytes = (unsigned)(g.nx * sizeof(TI));
-  const XsConfig c = xs_config(N, E, RB * row_bytes, 0, sizeof(TI) == 8);
+  const XsConfig c = xs_config(N, E, RB * row_bytes, 0, sizeof(TI) == 8 ? XS_ALIAS_TWO : xs_alias_float(E), false,
+                               4);
   if (c.ns == 0 || !aligned16(in) || row_bytes % 16) return cudaSuccess;
   const long long ngroups = ((long long)g.ny * (g.lev1 - g.lev0) + RB - 1) / RB;
   PGB_XS_E_SWITCH(E, PGB_XS_N_SWITCH(N, {

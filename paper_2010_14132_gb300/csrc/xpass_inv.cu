@@ -18,16 +18,24 @@ namespace {
 #ifndef PGB_XINV_E3_BLOCKS
 #define PGB_XINV_E3_BLOCKS 2
 #endif
-constexpr int xinv_min_blocks(int e) { return e % 3 == 0 ? PGB_XINV_E3_BLOCKS : PGB_XINV_MIN_BLOCKS; }
+#ifndef PGB_XINV_PLAIN_BLOCKS
+#define PGB_XINV_PLAIN_BLOCKS 4
+#endif
+// the plain output of lines up to 256 points fits four (64 registers, and the shared memory)
+constexpr int xinv_min_blocks(int n, int e, int mode) {
+  return e % 3 == 0 ? PGB_XINV_E3_BLOCKS
+                    : (e == 8 && n <= 256 && mode == XINV_PLAIN ? PGB_XINV_PLAIN_BLOCKS : PGB_XINV_MIN_BLOCKS);
+}
+constexpr XsAlias xinv_alias(int e, int mode) { return mode == XINV_PLAIN ? xs_alias_float(e) : XS_ALIAS_NONE; }
 template <int N, int E, typename TO, int MODE>
-__global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_s(const float2* __restrict__ spec, TO* __restrict__ out, Geom g,
+__global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(N, E, MODE)) k_xinv_s(const float2* __restrict__ spec, TO* __restrict__ out, Geom g,
                                                       const float2* __restrict__ twx, const float2* __restrict__ twr,
                                                       XinvExtra ex, int ns, unsigned stage_bytes) {
   using C = float2;
   constexpr int nl = N / E, RB = xs_rows(N, E), LS = N;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
-  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, false);
+  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, xinv_alias(E, MODE), true);
   C* tw_s = reinterpret_cast<C*>(smraw);
   C* twr_s = tw_s + N;
   C* lines = twr_s + N + 2;
@@ -63,8 +71,8 @@ __global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_
     }
   const LineSyncT<nl> sync{1 + ty};
   const LineAddr<N> sw{};
-  C* la = lines + (size_t)ty * 2 * LS;
-  C* lb = la + LS;
+  constexpr bool kAlias = xinv_alias(E, MODE) == XS_ALIAS_ONE;   // the staged row is the other buffer
+  C* la = lines + (size_t)ty * (kAlias ? 1 : 2) * LS;
   // per-lane partial sums (even / odd points): delta^2, p^2 and the double-float sum of p
   float2 acc0 = make_float2(0.f, 0.f), acc1 = acc0, sh = acc0, sl = acc0;
   bool ok = true;
@@ -99,7 +107,7 @@ __global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_
         }
       }
     }
-    const C* X = reinterpret_cast<const C*>(stg + (size_t)s * stage_bytes + (size_t)ty * row_bytes);
+    C* X = reinterpret_cast<C*>(stg + (size_t)s * stage_bytes + (size_t)ty * row_bytes);
     C v[E];
 #pragma unroll
     for (int i = 0; i < E; ++i) {
@@ -114,7 +122,8 @@ __global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_
       const C od = cmul(csub(xk, xc), cconj(twr_s[m]));   // * exp(+2 pi i m/n)
       v[i] = make_float2(ev.x - od.y, ev.y + od.x);        // ev + i od
     }
-    st_fft<N, E, +1, true, float>(v, la, lb, sw, lane, tw_s, sync);
+    st_fft<N, E, +1, true, float>(v, la, kAlias ? X : la + LS, sw, lane, tw_s, sync);
+    if constexpr (kAlias) fence_proxy_async_smem();   // generic writes to the staged row come before its refill by TMA
     if (valid) {
 #pragma unroll
       for (int i = 0; i < E; ++i) {
@@ -158,7 +167,7 @@ __global__ void __launch_bounds__(xs_max_threads(E), xinv_min_blocks(E)) k_xinv_
     // deterministic CTA partial sums: fixed-order tree over the CTA's threads, in the
     // line buffers (no longer in use: every thread is past its last transform)
     constexpr int TH = xs_threads(N, E);
-    static_assert((size_t)TH * 40 <= (size_t)RB * 2 * LS * sizeof(C), "reduction does not fit the line buffers");
+    static_assert((size_t)TH * 40 <= (size_t)RB * LS * sizeof(C), "reduction does not fit the line buffers");
     __syncthreads();
     double* redd = reinterpret_cast<double*>(lines);
     float (*red)[TH] = reinterpret_cast<float (*)[TH]>(redd + TH);
@@ -235,7 +244,7 @@ cudaError_t xinv_s(const float2* spec, TO* out, const Geom& g, int N, int E, con
   const int RB = xs_rows(N, E);
   const unsigned row_bytes = (unsigned)xs_align((size_t)(N + 1) * sizeof(float2), 16);
   if ((size_t)g.P * sizeof(float2) < row_bytes || (g.P * sizeof(float2)) % 16 || !aligned16(spec)) return cudaSuccess;
-  const XsConfig c = xs_config(N, E, RB * row_bytes, 0, false);
+  const XsConfig c = xs_config(N, E, RB * row_bytes, 0, xinv_alias(E, MODE), true, xinv_min_blocks(N, E, MODE));
   if (c.ns == 0) return cudaSuccess;
   const long long ngroups = ((long long)g.ny * (g.lev1 - g.lev0) + RB - 1) / RB;
   PGB_XS_E_SWITCH(E, PGB_XS_N_SWITCH(N, {

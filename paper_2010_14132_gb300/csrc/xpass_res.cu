@@ -46,10 +46,10 @@ __global__ void __launch_bounds__(xs_max_threads(E), xres_min_blocks(E, HAS_Q, F
   constexpr int nl = N / E, RB = xs_rows(N, E), LS = N, NX = 2 * N;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
-  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, true);
+  const XsLayout L = xs_layout(N, RB, ns, stage_bytes, XS_ALIAS_TWO, false);
   C* tw_s = reinterpret_cast<C*>(smraw);
   C* twr_s = tw_s + N;
-  C* lines = twr_s + N + 2;
+  C* lines = twr_s + N / 2 + 2;
   unsigned char* stg = smraw + L.off_stage;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + L.off_bar);
 
@@ -254,13 +254,13 @@ cudaError_t xres_s(const ResidualArgs& R, float2* spec, const Geom& g, int N, in
   // stage S, p0 (and q) rows while three CTAs per SM still fit, else S rows only
   const unsigned row_bytes_all = (unsigned)(g.nx * (8 + 4 + (HAS_Q ? 4 : 0)));
   const unsigned row_bytes_s = (unsigned)(g.nx * 8);
-  const XsConfig c_all = xs_config(N, E, RB * row_bytes_all, 0, true);
+  const XsConfig c_all = xs_config(N, E, RB * row_bytes_all, 0, XS_ALIAS_TWO, false, 3);
   const bool stage_p = c_all.ns > 0 && c_all.smem <= 75 * 1024 * (size_t)xs_max_threads(E) / 256;
-  const XsConfig c = stage_p ? c_all : xs_config(N, E, RB * row_bytes_s, 0, true);
+  const XsConfig c = stage_p ? c_all : xs_config(N, E, RB * row_bytes_s, 0, XS_ALIAS_TWO, false, 3);
   const long long ngroups = ((long long)g.ny * (g.lev1 - g.lev0) + RB - 1) / RB;
   if constexpr (HAS_Q) {
     if (R.r0) {   // the first try's r0 - L q: r0 rows staged in slots of an S row's width
-      const XsConfig c0 = xs_config(N, E, RB * row_bytes_s, 0, true);
+      const XsConfig c0 = xs_config(N, E, RB * row_bytes_s, 0, XS_ALIAS_TWO, false, 3);
       if (c0.ns == 0 || !aligned16(R.r0) || (R.r_ld * 4) % 16 || !aligned16(R.p0) || !aligned16(R.q) ||
           (g.nx * 4) % 16)
         return cudaSuccess;
