@@ -312,7 +312,7 @@ int xpass_blocks(const Geom& g, const FftPlan& fx, size_t csize) {
   const int rb = xpass_rows(fx.n, fx.E, csize);
   long long nb = (nrows + rb - 1) / rb;
   if (csize == sizeof(float2) && xpass_static_supported(fx.n)) {
-    const long long rbs = 256 / (fx.n / (fx.n % 3 == 0 ? kE3 : 8));   // rows per group of the persistent kernels
+    const long long rbs = 256 / (fx.n / st_elems(fx.n));   // rows per group of the persistent kernels
     const long long ng = (nrows + rbs - 1) / rbs;
     if (ng > nb) nb = ng;
   }

@@ -31,6 +31,10 @@ constexpr int st_big_log(int e) { return e % 16 == 0 ? 4 : (e % 8 == 0 ? 3 : 2);
 // Elements per thread for lengths with a factor 3: radix 3, then radix 4 (12 values per thread
 // keep a line's data in twice as many threads as the radix-8 schedule's 24, for the same shared memory)
 constexpr int kE3 = 12;
+// ... or radices 3 and 2 with 6, where the length has a single factor 2
+constexpr int kE3Odd = 6;
+// elements per thread by length: 8 for powers of two
+constexpr int st_elems(int n) { return n % 12 == 0 ? kE3 : (n % 6 == 0 ? kE3Odd : 8); }
 constexpr int st_nstages(int n, int e) {
   return st_count(n, 3) + st_count(n, 2) / st_big_log(e) + (st_count(n, 2) % st_big_log(e) ? 1 : 0);
 }

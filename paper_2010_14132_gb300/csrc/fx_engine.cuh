@@ -43,15 +43,15 @@ constexpr int clog2(long long n) {
   while ((1LL << b) < n) ++b;
   return b;
 }
-// elements per thread: radix 8 for powers of two, radices 3 and 4 for lengths with a factor 3
-constexpr int fx_elems(int n) { return n % 3 == 0 ? kE3 : 8; }
+// elements per thread: radix 8 for powers of two, radices 3 and 4 (or 2) for lengths with a factor 3
+constexpr int fx_elems(int n) { return st_elems(n); }
 // lengths the kernels are built for
 constexpr bool fx_length(int n) {
   switch (n) {
     case 16: case 32: case 64: case 128: case 256: case 512: case 1024: case 2048:
     case 24: case 48: case 96: case 192: case 384: case 768:
     case 36: case 72: case 144: case 288: case 576:
-    case 108: case 216: case 432: case 864: case 324:
+    case 18: case 54: case 108: case 216: case 432: case 864: case 324:
       return true;
     default: return false;
   }
@@ -304,6 +304,7 @@ template <typename K> inline cudaError_t fx_allow_smem(K kernel, size_t bytes) {
     PGB_FX_N_CASE(384, __VA_ARGS__) PGB_FX_N_CASE(768, __VA_ARGS__) PGB_FX_N_CASE(36, __VA_ARGS__)              \
     PGB_FX_N_CASE(72, __VA_ARGS__) PGB_FX_N_CASE(144, __VA_ARGS__) PGB_FX_N_CASE(288, __VA_ARGS__)              \
     PGB_FX_N_CASE(576, __VA_ARGS__) PGB_FX_N_CASE(108, __VA_ARGS__) PGB_FX_N_CASE(216, __VA_ARGS__)             \
+    PGB_FX_N_CASE(18, __VA_ARGS__) PGB_FX_N_CASE(54, __VA_ARGS__)                                               \
     PGB_FX_N_CASE(432, __VA_ARGS__) PGB_FX_N_CASE(864, __VA_ARGS__) PGB_FX_N_CASE(324, __VA_ARGS__)             \
     default: return cudaSuccess;                                                                                \
   }

@@ -36,7 +36,7 @@ namespace {
 
 // Rows per CTA of the residual kernels that stage every stencil row (xpass_res_tile.cu), about 128 threads; lines
 // that leave fewer than two (1024 packed points and more) take the kernels that read neighbour rows through L2.
-__host__ __device__ constexpr int xrt_rows(int n) { return 128 / (n / (n % 3 == 0 ? kE3 : 8)); }
+__host__ __device__ constexpr int xrt_rows(int n) { return 128 / (n / st_elems(n)); }
 __host__ __device__ constexpr bool xrt_length(int n) { return xrt_rows(n) >= 2; }
 
 // CTA size: at most 256 threads with 8 or 12 elements per thread, 128 with 16 (one warp per
@@ -187,13 +187,16 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 
 // Elements per thread of the persistent x-pass for a half length N: kE3 when N has
 // a factor 3 (radix 3, then 4), else the plan's 8 or 16.
-inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? kE3 : (plan_e == 16 ? 16 : 8); }
+inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? st_elems(N) : (plan_e == 16 ? 16 : 8); }
 
 // Dispatch to the compile-time (N, E) instance; shapes the engine cannot take are
 // never instantiated (and are not reported supported).
 #define PGB_XS_E_SWITCH(E, ...)                                 \
   if ((E) == kE3) {                                             \
     constexpr int EE = kE3;                                     \
+    __VA_ARGS__;                                                \
+  } else if ((E) == kE3Odd) {                                   \
+    constexpr int EE = kE3Odd;                                  \
     __VA_ARGS__;                                                \
   } else if ((E) == 16) {                                       \
     constexpr int EE = 16;                                      \
@@ -206,11 +209,17 @@ inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? kE3 : (plan_e == 16
   case V: { constexpr int NN = V; if constexpr (st_valid(NN, EE)) { __VA_ARGS__; } } break;
 // Half lengths with compile-time kernels.  The ones with factors 9, 27 and 81 ran the run-time engine (24 elements
 // and 190 registers a thread, index arithmetic by division): 432 x 324 x 37 in FP32, x 42 -> 22 us, inverse x
-// 40 -> 22, and the y-pass of 324 points 24 -> 17.
+// 40 -> 22, and the y-pass of 324 points 24 -> 17.  The short ones (16 to 54) ran it as well, one CTA per row group:
+// FP32 32 x 32 x 32 38 -> 27 us, mixed 181 -> 123; FP32 96 x 768 x 101 237 -> 122.
 #define PGB_XS_N_SWITCH(N, ...)                          \
   switch (N) {                                           \
+    PGB_XS_N_CASE(16, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(18, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(24, __VA_ARGS__)                       \
     PGB_XS_N_CASE(32, __VA_ARGS__)                       \
     PGB_XS_N_CASE(36, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(48, __VA_ARGS__)                       \
+    PGB_XS_N_CASE(54, __VA_ARGS__)                       \
     PGB_XS_N_CASE(64, __VA_ARGS__)                       \
     PGB_XS_N_CASE(72, __VA_ARGS__)                       \
     PGB_XS_N_CASE(96, __VA_ARGS__)                       \

@@ -258,8 +258,8 @@ cudaError_t xinv_s(const float2* spec, TO* out, const Geom& g, int N, int E, con
 
 bool xpass_static_supported(int n_half) {
   switch (n_half) {
-    case 32: case 64: case 128: case 256: case 512: case 1024: case 2048:
-    case 36: case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 768:
+    case 16: case 32: case 64: case 128: case 256: case 512: case 1024: case 2048:
+    case 18: case 24: case 36: case 48: case 54: case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 768:
       return true;
     default: return false;
   }

@@ -205,7 +205,7 @@ cudaError_t xrt_launch(const ResidualArgs& R, float2* spec, const Geom& g, int n
                        unsigned* err, int* nblocks_out, cudaStream_t st, bool* used) {
 #define PGB_XRT_CASE(V)                                                                                              \
   case V: {                                                                                                          \
-    constexpr int EE = V % 3 == 0 ? kE3 : 8, RB = xrt_rows(V);                                                       \
+    constexpr int EE = st_elems(V), RB = xrt_rows(V);                                                                \
     static_assert(xrt_length(V), "two rows a CTA at least");                                                        \
     auto kern = k_xrt<V, EE, ISO, FROM_R0>;                                                                          \
     int cap = 0;                                                                                                     \
@@ -219,6 +219,7 @@ cudaError_t xrt_launch(const ResidualArgs& R, float2* spec, const Geom& g, int n
                       done, err);                                                                                    \
   }
   switch (n) {
+    PGB_XRT_CASE(16) PGB_XRT_CASE(18) PGB_XRT_CASE(24) PGB_XRT_CASE(48) PGB_XRT_CASE(54)
     PGB_XRT_CASE(32) PGB_XRT_CASE(36) PGB_XRT_CASE(64) PGB_XRT_CASE(72) PGB_XRT_CASE(96) PGB_XRT_CASE(108)
     PGB_XRT_CASE(128) PGB_XRT_CASE(144) PGB_XRT_CASE(192) PGB_XRT_CASE(216) PGB_XRT_CASE(256) PGB_XRT_CASE(288)
     PGB_XRT_CASE(324) PGB_XRT_CASE(384) PGB_XRT_CASE(432) PGB_XRT_CASE(512) PGB_XRT_CASE(768)

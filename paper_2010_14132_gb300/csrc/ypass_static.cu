@@ -1,4 +1,4 @@
-// Persistent FP32 y-pass for ny = 2^a 3^b in [64, 2048] (the list in PGB_YS_N_SWITCH; Section 2.1: the
+// Persistent FP32 y-pass for ny = 2^a 3^b in [32, 2048] (the list in PGB_YS_N_SWITCH; Section 2.1: the
 // transform along y of every kx column of every level).
 //
 // A tile is one level and TK consecutive kx columns: ny rows of TK complex
@@ -209,6 +209,10 @@ int largest_divisor_upto(int n, int cap) {
   case V: { constexpr int NN = V; if constexpr (st_valid(NN, E)) { __VA_ARGS__; } } break;
 #define PGB_YS_N_SWITCH(N, ...)        \
   switch (N) {                         \
+    PGB_YS_N_CASE(32, __VA_ARGS__)     \
+    PGB_YS_N_CASE(36, __VA_ARGS__)     \
+    PGB_YS_N_CASE(48, __VA_ARGS__)     \
+    PGB_YS_N_CASE(54, __VA_ARGS__)     \
     PGB_YS_N_CASE(64, __VA_ARGS__)     \
     PGB_YS_N_CASE(72, __VA_ARGS__)     \
     PGB_YS_N_CASE(96, __VA_ARGS__)     \
@@ -321,8 +325,8 @@ cudaError_t ys1_launch(float2* spec, const Geom& g, int N, const float2* twy, in
 
 bool ypass_static_supported(int ny) {
   switch (ny) {
-    case 64: case 128: case 256: case 512: case 1024: case 2048:
-    case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 576: case 768:
+    case 32: case 64: case 128: case 256: case 512: case 1024: case 2048:
+    case 36: case 48: case 54: case 72: case 96: case 108: case 144: case 192: case 216: case 288: case 324: case 384: case 432: case 576: case 768:
     case 864: case 1536:
       return true;
     default: return false;
@@ -335,14 +339,18 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   if (!ypass_static_supported(fy.n)) return cudaSuccess;
   int tk = tile > 0 ? tile : 8;   // 64-byte TMA box rows (measured best untuned at 1024^2 and on small domains)
   if (tk % 2) tk += 1;   // 16-byte inner TMA box
-  // kE3 elements per thread when ny has a factor 3 (radix 3, then 4)
-  const int E = fy.n % 3 == 0 ? kE3 : (fy.E == 16 ? 16 : 8);
-  if (variant == 2 && (E == 16 || E == kE3)) {   // single-buffered, in place, two CTAs per SM
+  // when ny has a factor 3, 12 elements per thread (radix 3, then 4) or 6
+  const int E = fy.n % 3 == 0 ? st_elems(fy.n) : (fy.E == 16 ? 16 : 8);
+  if (variant == 2 && E != 8) {   // single-buffered, in place, two CTAs per SM
     int tk1 = tk;
+    if (tile <= 0 && tk1 * (fy.n / E) < 32) tk1 = 16;   // a warp at least
     while (tk1 > 2 && tk1 * (fy.n / E) > ys1_max_threads(fy.n, E)) tk1 >>= 1;
     float2* sp = (float2*)spec;
     cudaError_t e;
-    if (E == 16)
+    if (E == kE3Odd)
+      e = sign < 0 ? ys1_launch<kE3Odd, -1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used)
+                   : ys1_launch<kE3Odd, +1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used);
+    else if (E == 16)
       e = sign < 0 ? ys1_launch<16, -1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used)
                    : ys1_launch<16, +1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used);
     else
@@ -356,6 +364,7 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
 #define PGB_YS_CALL(EE, SG)                                                                   \
   return inplace ? ys_launch<EE, SG, true>(sp, g, fy.n, tb.twy_f, tk, done, err, st, used)    \
                  : ys_launch<EE, SG, false>(sp, g, fy.n, tb.twy_f, tk, done, err, st, used)
+  if (E == kE3Odd) return cudaSuccess;   // that form only
   if (E == kE3) {
     if (sign < 0) PGB_YS_CALL(kE3, -1);
     PGB_YS_CALL(kE3, +1);

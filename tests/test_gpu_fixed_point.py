@@ -15,7 +15,7 @@ from paper_2010_14132_gb300.solver import Plan
 
 pytestmark = pytest.mark.gpu
 
-LENGTHS = [16, 24, 32, 36, 48, 64, 72, 96, 108, 128, 144, 192, 216, 256, 288, 324, 384, 432, 512, 576, 768, 864,
+LENGTHS = [16, 18, 24, 32, 36, 48, 54, 64, 72, 96, 108, 128, 144, 192, 216, 256, 288, 324, 384, 432, 512, 576, 768, 864,
            1024, 2048]
 
 

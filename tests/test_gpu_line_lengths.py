@@ -1,4 +1,4 @@
-"""FP32 and mixed solves on line lengths with factors 9, 27 and 81 (compile-time transforms).
+"""FP32 and mixed solves on short line lengths and ones with factors 9, 27 and 81 (compile-time transforms).
 
 Each length is taken as the x line (nx = 2 N, lines that do not tile warps among them) and as the y line, with
 row counts that leave the last group of rows short, against the FP64 plan of the same grid.  The tolerances
@@ -13,8 +13,8 @@ from paper_2010_14132_gb300.solver import Plan
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("axis,n", [("x", n) for n in (36, 72, 108, 144, 216, 288, 324, 432)]
-                         + [("y", n) for n in (72, 108, 144, 216, 288, 324, 432, 576, 864)])
+@pytest.mark.parametrize("axis,n", [("x", n) for n in (16, 18, 24, 36, 48, 54, 72, 108, 144, 216, 288, 324, 432)]
+                         + [("y", n) for n in (32, 36, 48, 54, 72, 108, 144, 216, 288, 324, 432, 576, 864)])
 @pytest.mark.parametrize("iso", [True, False])
 def test_ragged_lengths(axis, n, iso):
     nx, ny, nz = (2 * n, 18, 5) if axis == "x" else (48, n, 5)

@@ -14,7 +14,7 @@ from paper_2010_14132_gb300.solver import Plan
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nx,ny,nz", [(64, 4, 2), (64, 36, 3), (64, 54, 2), (128, 48, 5), (192, 18, 2), (256, 27, 3),
+@pytest.mark.parametrize("nx,ny,nz", [(32, 48, 3), (36, 16, 2), (48, 81, 2), (108, 32, 2), (64, 4, 2), (64, 36, 3), (64, 54, 2), (128, 48, 5), (192, 18, 2), (256, 27, 3),
                                       (432, 16, 4), (512, 6, 2), (1024, 4, 2), (1024, 9, 3), (1024, 128, 2),
                                       (1536, 9, 3), (2048, 8, 3)])
 @pytest.mark.parametrize("opts", [{}, {"bc": "dirichlet_top"}, {"verify": 0}, {"level_chunk": 2}])
