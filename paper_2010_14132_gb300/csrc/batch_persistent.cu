@@ -338,7 +338,7 @@ __device__ void item_x(const BDom& D, int type, int pass, int sub, unsigned char
       for (int i = 0; i < E; ++i) v[i] = line[sw(st_in_index<N, E, 0>(lane, i))];
       sync();   // every input is read before the transform overwrites the line
       const float2* fin = st_fft_inplace<N, E, -1, false, float>(v, line, sw, lane, tw_s, sync);
-      r2c_unpack_store<N, E>(fin, twr_s, D.spec + rr * g.P, lane, valid);
+      r2c_unpack_store<N, E, Swizzled>(fin, twr_s, D.spec + rr * g.P, lane, valid);
     } else {
       // C2R: each first-stage input from the bins X_m and X_{N-m} (self-conjugate bins real)
       const float2* X = D.spec + rr * g.P;

@@ -121,11 +121,63 @@ template <int SIGN, typename C, typename T> __device__ __forceinline__ void dft1
     for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = t[4 * k1 + k2];
 }
 
+// multiply by W^m = exp(SIGN 2 pi i m/12)
+template <int SIGN, int M, typename C, typename T> __device__ __forceinline__ C w12(C a) {
+  const T h = (T)0.86602540378443864676, q = (T)0.5;   // cos, sin (pi/6)
+  if constexpr (M == 0) return a;
+  else if constexpr (M == 3) return cmul_si<SIGN>(a);
+  else if constexpr (M == 6) return C{-a.x, -a.y};
+  else {
+    const T cs = M == 1 ? h : (M == 2 ? q : -q), sn = (T)SIGN * (M == 1 ? q : h);   // M in {1, 2, 4}
+    return C{cs * a.x - sn * a.y, cs * a.y + sn * a.x};
+  }
+}
+
+// 12-point DFT as 3 x 4: DFT3 over n1 of x[4 n1 + n2], inner twiddles W^(n2 k1), DFT4 over n2; X[k1 + 3 k2] then sits
+// in slot 4 k1 + k2 and is moved to natural order.  One stage in place of a radix-3 and a radix-4 one.
+template <int SIGN, typename C, typename T> __device__ __forceinline__ void dft12(C* v) {
+  C y[3][4];
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) {
+    C t[3] = {v[n2], v[n2 + 4], v[n2 + 8]};
+    dft3<SIGN, C, T>(t);
+#pragma unroll
+    for (int k1 = 0; k1 < 3; ++k1) y[k1][n2] = t[k1];
+  }
+  y[1][1] = w12<SIGN, 1, C, T>(y[1][1]);
+  y[1][2] = w12<SIGN, 2, C, T>(y[1][2]);
+  y[1][3] = w12<SIGN, 3, C, T>(y[1][3]);
+  y[2][1] = w12<SIGN, 2, C, T>(y[2][1]);
+  y[2][2] = w12<SIGN, 4, C, T>(y[2][2]);
+  y[2][3] = w12<SIGN, 6, C, T>(y[2][3]);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    dft4<SIGN>(y[k1][0], y[k1][1], y[k1][2], y[k1][3]);
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 3 * k2] = y[k1][k2];
+  }
+}
+// 6-point DFT as 3 x 2
+template <int SIGN, typename C, typename T> __device__ __forceinline__ void dft6(C* v) {
+  C a[3] = {v[0], v[2], v[4]}, b[3] = {v[1], v[3], v[5]};
+  dft3<SIGN, C, T>(a);
+  dft3<SIGN, C, T>(b);
+  b[1] = w12<SIGN, 2, C, T>(b[1]);
+  b[2] = w12<SIGN, 4, C, T>(b[2]);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    v[k1] = cadd(a[k1], b[k1]);
+    v[k1 + 3] = csub(a[k1], b[k1]);
+  }
+}
+
 template <int R, int SIGN, typename T> __device__ __forceinline__ void dft_r(typename CT<T>::t* v) {
   if constexpr (R == 2) dft2<SIGN>(v);
   else if constexpr (R == 3) dft3<SIGN, typename CT<T>::t, T>(v);
   else if constexpr (R == 4) dft4<SIGN>(v[0], v[1], v[2], v[3]);
+  else if constexpr (R == 6) dft6<SIGN, typename CT<T>::t, T>(v);
   else if constexpr (R == 8) dft8<SIGN, typename CT<T>::t, T>(v);
+  else if constexpr (R == 12) dft12<SIGN, typename CT<T>::t, T>(v);
   else dft16<SIGN, typename CT<T>::t, T>(v);
 }
 

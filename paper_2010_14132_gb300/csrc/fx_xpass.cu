@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xfwd_fx(cons
                                                                            const int4* __restrict__ twr) {
   constexpr int E = fx_elems(N), nl = N / E, RB = fx_x_rows(N), LS = fx_line_stride(N);
   // one more bit of room than the transform needs: 2 |X_k| <= |Z_k + conj Z_{N-k}| + |Z_k - conj Z_{N-k}|
-  constexpr int T = 60 - clog2(st_radix(N, 0, E));
+  constexpr int T = 60 - clog2(fx_radix(N, 0, E));
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
   Fx2* lines = reinterpret_cast<Fx2*>(smraw);
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xfwd_fx(cons
   const double2* src = reinterpret_cast<const double2*>(in + (valid ? row : 0) * g.nx);
   double2 x[E];
 #pragma unroll
-  for (int i = 0; i < E; ++i) x[i] = valid ? __ldcs(&src[st_in_index<N, E, 0>(lane, i)]) : make_double2(0, 0);
+  for (int i = 0; i < E; ++i) x[i] = valid ? __ldcs(&src[fx_in_index<N, E>(lane, i)]) : make_double2(0, 0);
   sync();
   unsigned h = 0;
 #pragma unroll
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xinv_fx(cons
                                                                            const int4* __restrict__ twr) {
   constexpr int E = fx_elems(N), nl = N / E, RB = fx_x_rows(N), LS = fx_line_stride(N);
   // two more bits of room than the transform needs: |z| <= 2 (|X_m| + |X_{N-m}|)
-  constexpr int T = 59 - clog2(st_radix(N, 0, E));
+  constexpr int T = 59 - clog2(fx_radix(N, 0, E));
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
   Fx2* lines = reinterpret_cast<Fx2*>(smraw);
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xinv_fx(cons
   Fx2 v[E];
 #pragma unroll
   for (int i = 0; i < E; ++i) {
-    const int m = st_in_index<N, E, 0>(lane, i);
+    const int m = fx_in_index<N, E>(lane, i);
     const Fx2 xk = la[sw(m)], xc = la[sw(N - m)];
     const Fx2 ev = {xk.x + xc.x, xk.y - xc.y};
     int4 w = __ldg(&twr[m]);   // its conjugate: exp(+2 pi i m/nx)
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_x_rows(N)) k_xinv_fx(cons
   double2* dst = reinterpret_cast<double2*>(out + row * g.nx);
 #pragma unroll
   for (int i = 0; i < E; ++i)
-    __stcs(&dst[st_out_index<N, E>(lane, i)],
+    __stcs(&dst[fx_out_index<N, E>(lane, i)],
            make_double2(to_d(v[i].y), to_d(v[i].x)));
 }
 
@@ -222,8 +222,8 @@ int4 fx_twiddle(long long m, long long n) {
   auto halves = [](long double v, int& hi, int& lo) {
     const long long f = llrintl(v * 2305843009213693952.0L);   // 2^61
     lo = (int)(unsigned)(unsigned long long)f;
-    if (lo == (int)0x80000000) lo += 1;   // its negative has to exist
-    hi = (int)((f - lo + 0x40000000ll) >> 32);
+    hi = (int)((f - lo) / 4294967296ll);   // exact
+    if (lo == (int)0x80000000) lo += 1;    // its negative has to exist
   };
   int4 w;
   halves(c, w.x, w.y);
@@ -239,8 +239,8 @@ std::vector<int4> fx_stage_table(int n) {
   std::vector<int4> t;
   if (!fx_length(n)) return t;
   const int E = fx_elems(n);
-  for (int s = 0, Ns = 1; s < st_nstages(n, E); ++s) {
-    const int R = st_radix(n, s, E);
+  for (int s = 0, Ns = 1; s < fx_nstages(n, E); ++s) {
+    const int R = fx_radix(n, s, E);
     for (int r = 1; r < R; ++r)
       for (int k = 0; k < Ns; ++k) t.push_back(fx_twiddle((long long)r * k, (long long)Ns * R));
     Ns *= R;

@@ -34,7 +34,7 @@ template <int N>
 __global__ void __launch_bounds__(N / fx_elems(N) * fx_y_cols(N), fx_y_blocks(N)) k_yfft_fx(double2* __restrict__ spec, Geom g,
                                                                            const int4* __restrict__ tw, int inverse) {
   constexpr int E = fx_elems(N), nl = N / E, TK = fx_y_cols(N);
-  constexpr int T = 61 - clog2(st_radix(N, 0, E));
+  constexpr int T = 61 - clog2(fx_radix(N, 0, E));
   constexpr bool kShuffle = (TK * nl) % 32 == 0;
   pdl_trigger();
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_y_cols(N), fx_y_blocks(N)
   double2 x[E];
 #pragma unroll
   for (int i = 0; i < E; ++i)
-    x[i] = vcol ? base[(long long)st_in_index<N, E, 0>(lane, i) * g.P] : make_double2(0, 0);
+    x[i] = vcol ? base[(long long)fx_in_index<N, E>(lane, i) * g.P] : make_double2(0, 0);
   __syncthreads();
   unsigned h = 0;
 #pragma unroll
@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(N / fx_elems(N) * fx_y_cols(N), fx_y_blocks(N)
 #pragma unroll
   for (int i = 0; i < E; ++i) {
     const double a = to_d(v[i].x), b = to_d(v[i].y);
-    base[(long long)st_out_index<N, E>(lane, i) * g.P] = inverse ? make_double2(b, a) : make_double2(a, b);
+    base[(long long)fx_out_index<N, E>(lane, i) * g.P] = inverse ? make_double2(b, a) : make_double2(a, b);
   }
 }
 

@@ -90,14 +90,14 @@ __device__ __forceinline__ void ring_drain(Ring& rg, uint64_t* bar, int ns) {
     for (int c = rg.consumed[s]; c < rg.issued[s]; ++c) mbar_wait_bounded(&bar[s], (unsigned)(c & 1), kWaitPolls);
 }
 
-// R2C unpacking of a transformed line (natural order in fin) and store of the
+// R2C unpacking of a transformed line (natural order in fin, element i at slot Addr(i)) and store of the
 // bins 0..N to dst: each thread takes the bin pairs (k, N - k), k = lane + nl q.
-template <int N, int E>
+template <int N, int E, typename Addr = LineAddr<N>>
 __device__ __forceinline__ void r2c_unpack_store(const float2* fin, const float2* twr_s, float2* dst, int lane,
                                                  bool valid, int kmax = N) {
   using C = float2;
   constexpr int nl = N / E;
-  const LineAddr<N> sw{};
+  const Addr sw{};
 #pragma unroll
   for (int q = 0; q < E / 2; ++q) {
     const int k = lane + nl * q;   // k < N/2
@@ -186,7 +186,7 @@ template <typename K> cudaError_t prepare(K kernel, int threads, size_t smem, in
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 // Elements per thread of the persistent x-pass for a half length N: kE3 when N has
-// a factor 3 (radix 3, then 4), else the plan's 8 or 16.
+// a factor 3 (radix 12 first), else the plan's 8 or 16.
 inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? st_elems(N) : (plan_e == 16 ? 16 : 8); }
 
 // Dispatch to the compile-time (N, E) instance; shapes the engine cannot take are

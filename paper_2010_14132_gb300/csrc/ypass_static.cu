@@ -339,7 +339,7 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   if (!ypass_static_supported(fy.n)) return cudaSuccess;
   int tk = tile > 0 ? tile : 8;   // 64-byte TMA box rows (measured best untuned at 1024^2 and on small domains)
   if (tk % 2) tk += 1;   // 16-byte inner TMA box
-  // when ny has a factor 3, 12 elements per thread (radix 3, then 4) or 6
+  // when ny has a factor 3, 12 elements per thread (radix 12 first) or 6
   const int E = fy.n % 3 == 0 ? st_elems(fy.n) : (fy.E == 16 ? 16 : 8);
   if (variant == 2 && E != 8) {   // single-buffered, in place, two CTAs per SM
     int tk1 = tk;
