@@ -121,6 +121,49 @@ template <int SIGN, typename C, typename T> __device__ __forceinline__ void dft1
     for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = t[4 * k1 + k2];
 }
 
+// cos(pi m/16), m = 0..8
+__host__ __device__ constexpr double cos_pi16(int m) {
+  return m == 0 ? 1.0 : m == 1 ? 0.98078528040323044913 : m == 2 ? 0.92387953251128675613
+         : m == 3 ? 0.83146961230254523708 : m == 4 ? 0.70710678118654752440 : m == 5 ? 0.55557023301960222474
+         : m == 6 ? 0.38268343236508977173 : m == 7 ? 0.19509032201612826785 : 0.0;
+}
+// multiply by W^m = exp(SIGN 2 pi i m/32), 0 <= m <= 21
+template <int SIGN, int M, typename C, typename T> __device__ __forceinline__ C w32(C a) {
+  if constexpr (M == 0) return a;
+  else if constexpr (M == 8) return cmul_si<SIGN>(a);
+  else if constexpr (M == 16) return C{-a.x, -a.y};
+  else {
+    constexpr int q = M / 8, f = M % 8;   // quadrant, angle inside it
+    constexpr double cf = cos_pi16(f), sf = cos_pi16(8 - f);
+    constexpr double cd = q == 0 ? cf : (q == 1 ? -sf : -cf), sd = q == 0 ? sf : (q == 1 ? cf : -sf);
+    const T cs = (T)cd, sn = (T)(SIGN * sd);
+    return C{cs * a.x - sn * a.y, cs * a.y + sn * a.x};
+  }
+}
+
+// 32-point DFT as 8 x 4: DFT8 over n1 of x[4 n1 + n2], inner twiddles W^(n2 k1), DFT4 over n2 gives X[k1 + 8 k2].
+template <int SIGN, typename C, typename T> __device__ __forceinline__ void dft32(C* v) {
+  C y[4][8];
+#pragma unroll
+  for (int n2 = 0; n2 < 4; ++n2) {
+#pragma unroll
+    for (int n1 = 0; n1 < 8; ++n1) y[n2][n1] = v[4 * n1 + n2];
+    dft8<SIGN, C, T>(y[n2]);
+  }
+#define PGB_W32(K1)                                   \
+  y[1][K1] = w32<SIGN, K1, C, T>(y[1][K1]);           \
+  y[2][K1] = w32<SIGN, 2 * K1, C, T>(y[2][K1]);       \
+  y[3][K1] = w32<SIGN, 3 * K1, C, T>(y[3][K1]);
+  PGB_W32(1) PGB_W32(2) PGB_W32(3) PGB_W32(4) PGB_W32(5) PGB_W32(6) PGB_W32(7)
+#undef PGB_W32
+#pragma unroll
+  for (int k1 = 0; k1 < 8; ++k1) {
+    dft4<SIGN>(y[0][k1], y[1][k1], y[2][k1], y[3][k1]);
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 8 * k2] = y[k2][k1];
+  }
+}
+
 // multiply by W^m = exp(SIGN 2 pi i m/12)
 template <int SIGN, int M, typename C, typename T> __device__ __forceinline__ C w12(C a) {
   const T h = (T)0.86602540378443864676, q = (T)0.5;   // cos, sin (pi/6)
@@ -178,6 +221,7 @@ template <int R, int SIGN, typename T> __device__ __forceinline__ void dft_r(typ
   else if constexpr (R == 6) dft6<SIGN, typename CT<T>::t, T>(v);
   else if constexpr (R == 8) dft8<SIGN, typename CT<T>::t, T>(v);
   else if constexpr (R == 12) dft12<SIGN, typename CT<T>::t, T>(v);
+  else if constexpr (R == 32) dft32<SIGN, typename CT<T>::t, T>(v);
   else dft16<SIGN, typename CT<T>::t, T>(v);
 }
 

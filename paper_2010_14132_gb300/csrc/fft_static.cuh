@@ -16,7 +16,7 @@
 
 namespace pgb {
 
-// Radix schedule for n = 2^a 3^b and E elements per thread.  Powers of two: radix 16 (when E is a multiple of 16), 8 (a
+// Radix schedule for n = 2^a 3^b and E elements per thread.  Powers of two: radix 32 (when E is a multiple of 32), 16, 8 (a
 // multiple of 8) or 4, then a final 2, 4 or 8.  Lengths with a factor 3 (E = 12 or 6): the largest of 12, 6, 4, 3, 2 that
 // divides both what is left of n and E, so that 216 = 12 6 3 takes three stages and 384 = 12 4 4 2 four.  Each stage saved
 // is one exchange through shared memory and its barrier less, which is what bounds these lengths: with the stages
@@ -30,7 +30,7 @@ constexpr int st_count(int n, int p) {
   }
   return c;
 }
-constexpr int st_big_log(int e) { return e % 16 == 0 ? 4 : (e % 8 == 0 ? 3 : 2); }   // log2 of the main power-of-two radix
+constexpr int st_big_log(int e) { return e % 32 == 0 ? 5 : (e % 16 == 0 ? 4 : (e % 8 == 0 ? 3 : 2)); }   // log2 of the main power-of-two radix
 constexpr int st_next3(int n, int e) {   // the next radix of a schedule with factors 3
   constexpr int cand[5] = {12, 6, 4, 3, 2};
   for (int i = 0; i < 5; ++i)
@@ -71,6 +71,7 @@ constexpr int st_span(int n, int s, int e) {
 // E elements per thread must be a multiple of every radix of the schedule.
 constexpr bool st_valid(int n, int e) {
   if (n < 2 || e < 1 || n % e != 0) return false;
+  if (e == 32 && n != 512 && n != 1024) return false;   // two stages, where 16 elements take three
   if (n % 3 == 0 && e != st_elems(n)) return false;   // one element count for lengths with a factor 3
   for (int s = 0; s < st_nstages(n, e); ++s)
     if (e % st_radix(n, s, e) != 0) return false;

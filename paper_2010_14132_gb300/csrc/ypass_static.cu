@@ -27,6 +27,18 @@ template <int N> struct SwStrided {
   int es;
   __device__ __forceinline__ int operator()(int idx) const { return LineAddr<N>{}(idx) * es; }
 };
+// ... and with 32 elements per thread: the first stage's stride of 32 keeps the parity, which decides the half of the
+// banks that a row of 8 columns takes, so it is swapped in every other block of 32 (written so that each unrolled
+// access is one of two bases plus a constant)
+struct SwPair {
+  int es;
+  __device__ __forceinline__ int operator()(int idx) const {
+    const int s = (idx >> 5) & 1;
+    return ((idx & 1) ? idx - s : idx + s) * es;
+  }
+};
+template <int N, int E> struct SwOf { using t = SwStrided<N>; };
+template <int N> struct SwOf<N, 32> { using t = SwPair; };
 struct Plain {
   int es;
   __device__ __forceinline__ int operator()(int idx) const { return idx * es; }
@@ -41,7 +53,7 @@ constexpr int ys_max_threads(int E) { return E >= 16 || E % 3 == 0 ? 512 : 1024;
 // the single-buffered kernel runs two CTAs per SM: 256 threads for the 12-element lengths keeps
 // their registers (128) free of spills (288 for 864 points, whose 72 threads a column would leave only two
 // columns otherwise)
-constexpr int ys1_max_threads(int N, int E) { return E % 3 == 0 ? (N == 864 ? 288 : 256) : ys_max_threads(E); }
+constexpr int ys1_max_threads(int N, int E) { return E == 32 ? 256 : E % 3 == 0 ? (N == 864 ? 288 : 256) : ys_max_threads(E); }
 
 template <int N, int E, int SIGN, bool INPLACE>
 __global__ void __launch_bounds__(ys_max_threads(E)) k_ys(const __grid_constant__ CUtensorMap tm, Geom g,
@@ -157,7 +169,7 @@ __global__ void __launch_bounds__(ys1_max_threads(N, E), 2) k_ys1(const __grid_c
   __syncthreads();
   pdl_wait();   // the previous kernels of the stream are complete
   if (done && *done) return;
-  const SwStrided<N> sw{TK};
+  const typename SwOf<N, E>::t sw{TK};
   int it = 0, pending = 0;
   bool ok = true;
   auto issue = [&](int tt) {
@@ -341,6 +353,19 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   if (tk % 2) tk += 1;   // 16-byte inner TMA box
   // when ny has a factor 3, 12 elements per thread (radix 12 first) or 6
   const int E = fy.n % 3 == 0 ? st_elems(fy.n) : (fy.E == 16 ? 16 : 8);
+  // 512 = 32 16 and 1024 = 32 32: with 32 elements per thread these two lengths take two stages instead of three, one
+  // exchange through shared memory and two barriers less, which is what the pass waits for (one tile per CTA: load,
+  // stages and stores follow each other).  1024 x 1024 x 128: 216 -> 167 us a pass (4.97 -> 6.4 TB/s); 512 x 512 x 64:
+  // 31 -> 24.7.  128 registers, no spills, two CTAs of 256 threads at 1024 and four of 128 at 512.  256 points are two
+  // stages with 16 elements already, 2048 three with either.
+  if (variant == 2 && E == 16 && (fy.n == 512 || fy.n == 1024)) {
+    int tk1 = tk;
+    while (tk1 > 2 && tk1 * (fy.n / 32) > ys1_max_threads(fy.n, 32)) tk1 >>= 1;
+    float2* sp = (float2*)spec;
+    const cudaError_t e = sign < 0 ? ys1_launch<32, -1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used)
+                                   : ys1_launch<32, +1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used);
+    if (e != cudaSuccess || *used) return e;
+  }
   if (variant == 2 && E != 8) {   // single-buffered, in place, two CTAs per SM
     int tk1 = tk;
     if (tile <= 0 && tk1 * (fy.n / E) < 32) tk1 = 16;   // a warp at least
