@@ -97,8 +97,10 @@ typedef enum {
                                     stage, a third less shared memory); 4 (default) = one tile per CTA,
                                     in place, two CTAs per SM, the next tile's load overlapping this
                                     tile's stores (16 elements per thread; otherwise as 0) */
-  POISSON_OPT_X_ELEMS = 6,       /* x-pass elements per thread for power-of-two lines: 8 (default) or 16 */
-  POISSON_OPT_Y_ELEMS = 7,       /* y-pass elements per thread for power-of-two lines: 8 or 16 (default) */
+  POISSON_OPT_X_ELEMS = 6,       /* x-pass elements per thread for power-of-two lines: 8 or 16; unset: 8, and 16
+                                    for the FP32 plan's longer lines where that is faster */
+  POISSON_OPT_Y_ELEMS = 7,       /* y-pass elements per thread for power-of-two lines: 8 or 16 (default; kernel 4
+                                    then takes 32 for 512 and 1024 points) */
   POISSON_OPT_LEVEL_CHUNK = 8,   /* levels per transform chunk (x-pass and y-pass of a chunk run back to
                                     back so its spectrum stays in L2); 0 = all levels in one chunk
                                     (default: the persistent kernels lose more to per-launch start-up

@@ -523,6 +523,7 @@ int poisson_plan_set_option(poisson_plan* pl, int option, double value) {
       FftPlan f{};
       const bool x = option == POISSON_OPT_X_ELEMS;
       if (!make_fft_plan(x ? pl->nx / 2 : pl->ny, f, (int)value)) return POISSON_ERR_UNSUPPORTED;
+      f.e_set = 1;
       if (x) {
         pl->xelems = (int)value;
         pl->fx = f;

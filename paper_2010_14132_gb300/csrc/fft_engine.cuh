@@ -20,6 +20,7 @@ struct FftPlan {
   int nstages;
   int E;                   // elements per thread (multiple of every radix used)
   int radix[kMaxStages];
+  int e_set;               // E was set as an option: the compile-time kernels keep it too
 };
 
 template <int SIGN, typename C> __device__ __forceinline__ void dft2(C* v) {

@@ -188,6 +188,14 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 // Elements per thread of the persistent x-pass for a half length N: kE3 when N has
 // a factor 3 (radix 12 first), else the plan's 8 or 16.
 inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? st_elems(N) : (plan_e == 16 ? 16 : 8); }
+// ... of the FP32 transforms without the mixed path's conversions and epilogues, where no option chose it: 16 from 256
+// points on for the forward pass and from 512 on for the inverse one, whose registers then fit three CTAs per SM.  256
+// points take two stages (16 16) instead of three, 512 as many, with one warp per line instead of two and no barrier
+// between warps.  FP32 1024 x 1024 x 64 492 us with 8 in both, 483 with 16 in the forward pass, 476 in both;
+// 512 x 512 x 64 139 with 8, 136 with 16 in the forward pass, 139 in both; 256 x 256 x 64 (128 points) 47.9 and 51.8.
+inline int xs_elems_fp32(const FftPlan& fx, bool inverse) {
+  return fx.e_set || fx.n % 3 == 0 || fx.n < (inverse ? 512 : 256) ? xs_elems(fx.n, fx.E) : 16;
+}
 
 // Dispatch to the compile-time (N, E) instance; shapes the engine cannot take are
 // never instantiated (and are not reported supported).
