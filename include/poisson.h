@@ -99,8 +99,8 @@ typedef enum {
                                     tile's stores (16 elements per thread; otherwise as 0) */
   POISSON_OPT_X_ELEMS = 6,       /* x-pass elements per thread for power-of-two lines: 8 or 16; unset: 8, and 16
                                     for the FP32 plan's longer lines where that is faster */
-  POISSON_OPT_Y_ELEMS = 7,       /* y-pass elements per thread for power-of-two lines: 8 or 16 (default; kernel 4
-                                    then takes 32 for 512 and 1024 points) */
+  POISSON_OPT_Y_ELEMS = 7,       /* y-pass elements per thread for power-of-two lines: 8 or 16; unset: 16, and with
+                                    kernel 4 32 for 1024 points and for the FP32 plan's 512 */
   POISSON_OPT_LEVEL_CHUNK = 8,   /* levels per transform chunk (x-pass and y-pass of a chunk run back to
                                     back so its spectrum stays in L2); 0 = all levels in one chunk
                                     (default: the persistent kernels lose more to per-launch start-up

@@ -27,8 +27,10 @@ from .solver import Plan
 CACHE = os.environ.get("POISSON_AUTOTUNE_CACHE",
                        os.path.join(os.path.expanduser("~"), ".cache", "poisson_gb300_autotune.json"))
 
-Y_CANDIDATES = [dict(y_kernel=k, y_tile=t, y_elems=e) for k in (0, 4, 3, 1, 2) for t in (2, 4, 8, 16) for e in (8, 16)]
-X_CANDIDATES = [dict(x_kernel=k, x_elems=e) for k in (0, 1) for e in (8, 16)]
+# the first ones leave the elements per thread to the library's own rule
+Y_CANDIDATES = [dict(y_kernel=4, y_tile=t) for t in (4, 8)] + [
+    dict(y_kernel=k, y_tile=t, y_elems=e) for k in (0, 4, 3, 1, 2) for t in (2, 4, 8, 16) for e in (8, 16)]
+X_CANDIDATES = [dict(x_kernel=0)] + [dict(x_kernel=k, x_elems=e) for k in (0, 1) for e in (8, 16)]
 CHUNK_CANDIDATES = [dict(level_chunk=c) for c in (0, 1, 2, 4, 8, 16, 4096)]
 COL_CANDIDATES = [dict(col_tile=c) for c in (0, 1, 4, 3, 16, 32)]
 OPT_IDS = {"y_kernel": N.POISSON_OPT_Y_KERNEL, "y_tile": N.POISSON_OPT_Y_TILE, "y_elems": N.POISSON_OPT_Y_ELEMS,
@@ -95,6 +97,9 @@ def autotune(nx, ny, nz, dx, dy, dz, rho0, dtype="mixed", reps=3, verbose=False)
             print("y", cand, f"{ty:.3f} ms")
         if ty < best_yt:
             best_y, best_yt = dict(cand), ty
+    if "y_elems" not in best_y:   # a set option cannot be taken back
+        plan.close()
+        plan = Plan(nx, ny, nz, dx, dy, dz, rho0, dtype=dtype)
     for k, v in best_y.items():
         plan.set_option(OPT_IDS[k], v)
     best_x, best_xt = {}, float("inf")
@@ -111,6 +116,11 @@ def autotune(nx, ny, nz, dx, dy, dz, rho0, dtype="mixed", reps=3, verbose=False)
             print("x", cand, f"{tx:.3f} ms")
         if tx < best_xt:
             best_x, best_xt = dict(cand), tx
+    if "x_elems" not in best_x:
+        plan.close()
+        plan = Plan(nx, ny, nz, dx, dy, dz, rho0, dtype=dtype)
+        for k, v in best_y.items():
+            plan.set_option(OPT_IDS[k], v)
     for k, v in best_x.items():
         plan.set_option(OPT_IDS[k], v)
     # levels per transform chunk: timed on the whole solve (it trades L2 reuse against launch count)

@@ -61,8 +61,8 @@ template <> __device__ __forceinline__ float to_f<double>(double x) { return d2f
 // buffers of its own row (XS_ALIAS_TWO); a row of nx floats, or of n/2 + 1 spectrum bins, holds one of them, the
 // one that the second stage writes, when every input has long been read (XS_ALIAS_ONE; lines with a factor 3, whose
 // registers allow two CTAs per SM either way, keep both buffers).  What that saves makes room for a fourth
-// CTA per SM or a deeper ring (FP32 solve of 256 x 256 x 64: 53.1 -> 50.3 us; forward pass at 1024 x 1024 x 128 232 ->
-// 211).  The mixed path's inverse epilogues are held to three CTAs by their registers and keep both buffers.
+// CTA per SM or a deeper ring (FP32 solve of 256 x 256 x 64: 53.1 -> 50.3 us; forward pass at 1024 x 1024 x 128, 8 elements per
+// thread, 232 -> 211).  The mixed path's inverse epilogues are held to three CTAs by their registers and keep both buffers.
 enum XsAlias { XS_ALIAS_NONE = 0, XS_ALIAS_ONE = 1, XS_ALIAS_TWO = 2 };
 struct XsLayout {
   size_t off_stage, off_bar, total;
@@ -216,9 +216,9 @@ inline int xs_elems_fp32(const FftPlan& fx, bool inverse) {
 #define PGB_XS_N_CASE(V, ...) \
   case V: { constexpr int NN = V; if constexpr (st_valid(NN, EE)) { __VA_ARGS__; } } break;
 // Half lengths with compile-time kernels.  The ones with factors 9, 27 and 81 ran the run-time engine (24 elements
-// and 190 registers a thread, index arithmetic by division): 432 x 324 x 37 in FP32, x 42 -> 22 us, inverse x
-// 40 -> 22, and the y-pass of 324 points 24 -> 17.  The short ones (16 to 54) ran it as well, one CTA per row group:
-// FP32 32 x 32 x 32 38 -> 27 us, mixed 181 -> 123; FP32 96 x 768 x 101 237 -> 122.
+// and 190 registers a thread, index arithmetic by division): 432 x 324 x 37 in FP32 145 -> 77 us (x 42 -> 22, inverse
+// x 40 -> 22, the y-pass of 324 points 24 -> 17), 70 with radix 12.  The short ones (16 to 54) ran it as well, one CTA
+// per row group: FP32 32 x 32 x 32 38 -> 27 us, mixed 181 -> 123; FP32 96 x 768 x 101 237 -> 122, 108 with radix 12.
 #define PGB_XS_N_SWITCH(N, ...)                          \
   switch (N) {                                           \
     PGB_XS_N_CASE(16, __VA_ARGS__)                       \

@@ -358,7 +358,7 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   // stages and stores follow each other).  1024 x 1024 x 128: 216 -> 167 us a pass (4.97 -> 6.4 TB/s); 512 x 512 x 64:
   // 31 -> 24.7.  128 registers, no spills, two CTAs of 256 threads at 1024 and four of 128 at 512.  256 points are two
   // stages with 16 elements already, 2048 three with either.
-  if (variant == 2 && E == 16 && (fy.n == 512 || fy.n == 1024)) {
+  if (variant == 2 && E == 16 && !fy.e_set && (fy.n == 512 || fy.n == 1024)) {
     int tk1 = tk;
     while (tk1 > 2 && tk1 * (fy.n / 32) > ys1_max_threads(fy.n, 32)) tk1 >>= 1;
     float2* sp = (float2*)spec;
