@@ -2,8 +2,8 @@
 // r0 = S - mu_W - L p0, and the verification's first try r0 - L q (the same values, in the same arithmetic, as the
 // kernels of xpass_res.cu, which keep the residual with q and the lines too long for two rows a CTA).
 //
-// Bound by instruction issue (3.9 instructions a point: the double-float stencil in packed pairs, and the transform)
-// once the operands are at hand.  Read row by row through L2, the y and z neighbours kept 24 warps an SM
+// Bound by instruction issue (3.3 and 3.7 warp instructions a point for the two: the double-float stencil in packed
+// pairs, and the transform) once the operands are at hand.  Read row by row through L2, the y and z neighbours kept 24 warps an SM
 // waiting instead (long-scoreboard stalls 4 to 6 per instruction, issue slots 50-55% used; bringing the
 // upper rows into L2 ahead of time changed nothing).  Here a CTA of about 128 threads takes RB rows of one level
 // and stages, by bulk copies on two mbarriers, their operand rows (S, or r0 and p0) and the field's rows: the RB
