@@ -355,7 +355,7 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   const int E = fy.n % 3 == 0 ? st_elems(fy.n) : (fy.E == 16 ? 16 : 8);
   // 512 = 32 16 and 1024 = 32 32: with 32 elements per thread these two lengths take two stages instead of three, one
   // exchange through shared memory and two barriers less, which is what the pass waits for (one tile per CTA: load,
-  // stages and stores follow each other).  1024 x 1024 x 128: 216 -> 167 us a pass (4.97 -> 6.4 TB/s); 512 x 512 x 64:
+  // stages and stores follow each other).  1024 x 1024 x 128: 225 -> 181 us a pass (cold; 4.8 -> 5.9 TB/s); 512 x 512 x 64:
   // 31 -> 24.7.  128 registers, no spills, two CTAs of 256 threads at 1024 and four of 128 at 512.  256 points are two
   // stages with 16 elements already, 2048 three with either.
   if (variant == 2 && E == 16 && !fy.e_set && (fy.n == 512 || fy.n == 1024)) {
