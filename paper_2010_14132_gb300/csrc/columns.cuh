@@ -4,6 +4,7 @@
 // (Section 2.1).  The pivot algebra is stated at the top of thomas_kernels.cu.
 #pragma once
 #include "kernels.cuh"
+#include "launch_rules.hpp"
 
 namespace pgb {
 
@@ -165,10 +166,15 @@ __device__ __forceinline__ void lowk_recurrence(TCm* zx, TCm* zy, TCm* w, int ld
 // Shared memory (in doubles) of one low-|k| column solved by a block.
 __host__ __device__ constexpr size_t lowk_smem_elems(int nz) { return 6 * (size_t)nz + 96; }
 
-// Fixed-order sum over the block (every thread gets the result): a shuffle tree in each warp, then the warps in
-// order.  scratch: a double per warp.
+// Fixed-order sum over the block (every thread gets the result): a shuffle tree over the existing lanes of each warp
+// (a block may be half a warp), then the warps in order.  scratch: a double per warp.
 __device__ __forceinline__ double lowk_block_sum(double v, double* scratch) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  const int lane = threadIdx.x & 31, lanes = warp_lanes(threadIdx.x, blockDim.x);
+  const unsigned mask = warp_mask(threadIdx.x, blockDim.x);
+  for (int o = 16; o > 0; o >>= 1) {
+    const double u = __shfl_down_sync(mask, v, o);
+    if (lane + o < lanes) v += u;
+  }
   const int wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   __syncthreads();   // scratch may still be read from an earlier sum
   if ((threadIdx.x & 31) == 0) scratch[wid] = v;
@@ -201,7 +207,7 @@ __device__ __forceinline__ void lowk_column_tab(unsigned char* smraw, typename C
   double* z = reinterpret_cast<double*>(smraw);   // [2][nz]: real parts, imaginary parts
   double* F = z + 2 * nz;                          // elimination factors
   double* w = F + nz;                              // back-substitution factors
-  double* scratch = w + nz;                        // [3 per warp]
+  double* scratch = w + nz;                        // [1 per warp]
   const int kx = colk.x, ky = colk.y;
   const bool singular = singular00 && kx == 0 && ky == 0;   // nonsingular with p = 0 on the top face
   CS* colp = spec + (long long)ky * g.P + kx;
@@ -237,7 +243,8 @@ __device__ __forceinline__ void lowk_column_tab(unsigned char* smraw, typename C
     w[k] = k == m ? (ADJ ? r : (k + 1 < nz ? r : 0.0)) : r * u;
   }
   __syncthreads();
-  if (t < 32) {   // lanes 0-3: (part, direction); the others keep the shuffles whole
+  if (t < 32) {   // lanes 0-3: (part, direction); the others keep the shuffles whole (a block has 16 threads at least)
+    const unsigned mask = warp_mask(t, nt);
     const int part = t & 1, up = (t >> 1) & 1, n = t < 4 ? (up ? nz - 1 - m : m) : 0;
     double* zp = z + part * nz;
     const int k0 = up ? nz - 1 : 0, dk = up ? -1 : 1;
@@ -254,9 +261,9 @@ __device__ __forceinline__ void lowk_column_tab(unsigned char* smraw, typename C
       }
     }
     const double term = (up ? w[m] : F[m]) * y;
-    const double both = term + __shfl_xor_sync(0xffffffffu, term, 2);
+    const double both = term + __shfl_xor_sync(mask, term, 2);
     double x = (zp[m] + both) * __ldg(inv_col + m);
-    __syncwarp();
+    __syncwarp(mask);
     if (t < 2) zp[m] = x;
     if (n > 0) {
       int k = k0 + (n - 1) * dk;
