@@ -38,7 +38,6 @@
 #include <algorithm>
 #include <cstddef>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 #include "columns.cuh"
@@ -910,26 +909,14 @@ int batch_persistent_build(BatchPersistent* bp, const std::vector<BatchDomIn>& d
 
 cudaError_t batch_persistent_launch(const BatchPersistent& bp, cudaStream_t st) {
   if (!bp.doms || bp.nitems <= 0) return cudaErrorInvalidValue;
-  static std::mutex mu;
-  static int per_sm = -1;
-  static size_t granted = 0;
   int ctas = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (per_sm < 0 || granted < bp.smem) {
-      cudaError_t e = cudaFuncSetAttribute(k_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.smem);
-      if (e != cudaSuccess) return e;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch, kBT, bp.smem);
-      if (e != cudaSuccess) return e;
-      granted = bp.smem;
-    }
-    ctas = per_sm;
-  }
+  cudaError_t e = allow_smem(k_batch, bp.smem, kBT, &ctas);
+  if (e != cudaSuccess) return e;
   if (ctas < 1) return cudaErrorInvalidConfiguration;
   long long grid = (long long)ctas * sm_count();
   if (grid > bp.nitems) grid = bp.nitems;
   k_batch_init<<<bp.n, kBT, 0, st>>>(reinterpret_cast<const BDom*>(bp.doms), bp.ticket);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_batch<<<(unsigned)grid, kBT, bp.smem, st>>>(reinterpret_cast<const BDom*>(bp.doms),
                                                 reinterpret_cast<const uint2*>(bp.items), bp.nitems, bp.ticket,

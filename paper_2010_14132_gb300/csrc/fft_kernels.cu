@@ -13,11 +13,10 @@
 //    bins kx = 0 and kx = nx/2 contribute their real parts only.  Its epilogue
 //    writes the output field and, in the mixed-precision path, performs the
 //    refinement update and the norm partial sums.
-#include <mutex>
-#include <unordered_map>
 
 #include "kernels.cuh"
 #include "fft_static.cuh"
+#include "kernel_grants.cuh"
 #include "residual.cuh"
 
 namespace pgb {
@@ -284,19 +283,6 @@ bool fft_e_supported(int E) {
   }
 
 static constexpr int kMaxDynSmem = 227 * 1024;
-
-// Opt a kernel in to `bytes` of dynamic shared memory.  Always done (not only
-// above 48 KB): static shared memory counts against the same default limit.
-template <typename K> static cudaError_t allow_smem(K kernel, size_t bytes) {
-  static std::mutex mu;
-  static std::unordered_map<const void*, size_t> granted;
-  std::lock_guard<std::mutex> lock(mu);
-  size_t& have = granted[reinterpret_cast<const void*>(kernel)];
-  if (have >= bytes) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) have = bytes;
-  return e;
-}
 
 // rows per CTA for the x-pass
 static int xpass_rows(int n, int E, size_t csize) {

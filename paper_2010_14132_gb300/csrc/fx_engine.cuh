@@ -25,10 +25,9 @@
 // xl yl (below one unit of the result).  The inverse transform is the forward one with real and imaginary
 // parts exchanged on the way in and out.
 #pragma once
-#include <mutex>
-#include <unordered_map>
 
 #include "fft_static.cuh"
+#include "kernel_grants.cuh"
 
 namespace pgb {
 
@@ -305,18 +304,6 @@ __device__ __forceinline__ Fx2* fx_run_from(Fx2 (&v)[E], Fx2* cur, Fx2* nxt, Add
       return fx_run_from<N, E, FINAL_IN_REGS, S + 1, INPLACE>(v, nxt, cur, addr, lane, tw, sync, l1, l1b);
     }
   }
-}
-
-// opt a kernel in to its dynamic shared memory, once
-template <typename K> inline cudaError_t fx_allow_smem(K kernel, size_t bytes) {
-  static std::mutex mu;
-  static std::unordered_map<const void*, size_t> granted;
-  std::lock_guard<std::mutex> lock(mu);
-  size_t& have = granted[reinterpret_cast<const void*>(kernel)];
-  if (have >= bytes) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) have = bytes;
-  return e;
 }
 
 #define PGB_FX_N_CASE(V, ...) \

@@ -259,7 +259,7 @@ cudaError_t launch_xfwd_fx(const double* in, double2* spec, const Geom& g, int n
   *used = false;
   if (!tb.twx_q || !tb.twr_q) return cudaSuccess;
   PGB_FX_N_SWITCH(n, {
-    const cudaError_t e = fx_allow_smem(k_xfwd_fx<NN>, FxX<NN>::smem);
+    const cudaError_t e = allow_smem(k_xfwd_fx<NN>, FxX<NN>::smem);
     if (e != cudaSuccess) return e;
     *used = true;
     return pdl_launch(k_xfwd_fx<NN>, FxX<NN>::grid(g), dim3(FxX<NN>::nl, FxX<NN>::RB), FxX<NN>::smem, st, in, spec, g,
@@ -272,7 +272,7 @@ cudaError_t launch_xinv_fx(const double2* spec, double* out, const Geom& g, int 
   *used = false;
   if (!tb.twx_q || !tb.twr_q) return cudaSuccess;
   PGB_FX_N_SWITCH(n, {
-    const cudaError_t e = fx_allow_smem(k_xinv_fx<NN>, FxX<NN>::smem);
+    const cudaError_t e = allow_smem(k_xinv_fx<NN>, FxX<NN>::smem);
     if (e != cudaSuccess) return e;
     *used = true;
     return pdl_launch(k_xinv_fx<NN>, FxX<NN>::grid(g), dim3(FxX<NN>::nl, FxX<NN>::RB), FxX<NN>::smem, st, spec, out, g,

@@ -107,7 +107,7 @@ cudaError_t launch_yfft_fx(int sign, double2* spec, const Geom& g, int n, const 
   PGB_FX_N_SWITCH(n, {
     constexpr int TK = fx_y_cols(NN);
     constexpr size_t smem = (size_t)TK * NN * sizeof(Fx2);
-    const cudaError_t e = fx_allow_smem(k_yfft_fx<NN>, smem);
+    const cudaError_t e = allow_smem(k_yfft_fx<NN>, smem);
     if (e != cudaSuccess) return e;
     *used = true;
     return pdl_launch(k_yfft_fx<NN>, dim3((g.nxh + TK - 1) / TK, g.lev1 - g.lev0), dim3(TK, NN / fx_elems(NN)), smem,

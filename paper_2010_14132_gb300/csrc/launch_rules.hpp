@@ -2,6 +2,11 @@
 // too, so that they are tested on the host.
 #pragma once
 
+#include <cstddef>
+#include <functional>
+#include <mutex>
+#include <unordered_map>
+
 #ifdef __CUDACC__
 #define PGB_HD __host__ __device__ __forceinline__
 #else
@@ -20,5 +25,45 @@ PGB_HD unsigned warp_mask(int t, int n) {
   const int lanes = warp_lanes(t, n);
   return lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
 }
+
+// What the kernels have been granted, for all devices of the process: a kernel's shared memory limit is an attribute of
+// the kernel on one device, and its CTAs per SM depend on the device and on the shared memory it is launched with.
+class KernelGrants {
+ public:
+  // CTAs per SM of (device, kernel, smem) in *per_sm (0 if threads is 0: not asked for).  allow(smem) raises the limit,
+  // called where the device's is lower; occupancy(per_sm) is called once per entry.  Both return 0 or an error, passed on.
+  template <typename Allow, typename Occupancy>
+  int get(int device, const void* kernel, size_t smem, int threads, Allow allow, Occupancy occupancy, int* per_sm) {
+    std::lock_guard<std::mutex> lock(mu_);
+    size_t& limit = limit_[{device, kernel, 0}];
+    if (limit < smem) {
+      if (const int e = allow(smem)) return e;
+      limit = smem;
+    }
+    *per_sm = 0;
+    if (threads <= 0) return 0;
+    int& n = ctas_[{device, kernel, smem}];
+    if (n == 0)
+      if (const int e = occupancy(&n)) return e;
+    *per_sm = n;
+    return 0;
+  }
+
+ private:
+  struct Key {
+    int device;
+    const void* kernel;
+    size_t smem;
+    bool operator==(const Key& o) const { return device == o.device && kernel == o.kernel && smem == o.smem; }
+  };
+  struct Hash {
+    size_t operator()(const Key& k) const {
+      return std::hash<const void*>()(k.kernel) * 31 + k.smem * 131 + (size_t)k.device;
+    }
+  };
+  std::mutex mu_;
+  std::unordered_map<Key, size_t, Hash> limit_;
+  std::unordered_map<Key, int, Hash> ctas_;
+};
 
 }  // namespace pgb

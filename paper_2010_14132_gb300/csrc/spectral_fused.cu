@@ -28,13 +28,12 @@
 // of polls sets ERR_WAIT_TIMEOUT, skips its item and still counts it done, so the
 // items behind it are not held up; the solve then reports POISSON_ERR_TIMEOUT.
 #include <cstring>
-#include <mutex>
-#include <unordered_map>
 #include <vector>
 
 #include "async_copy.cuh"
 #include "columns.cuh"
 #include "fft_static.cuh"
+#include "kernel_grants.cuh"
 #include "kernels.cuh"
 
 namespace pgb {
@@ -322,23 +321,11 @@ cudaError_t launch_spectral_fused(const ThomasArgs& T, const Geom& g, const FftP
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  static std::mutex mu;
-  static std::unordered_map<const void*, std::pair<size_t, int>> granted;
   cudaError_t e = cudaSuccess;
   auto run = [&](auto kern, int nthreads) -> cudaError_t {
     int per_sm = 0;
-    {
-      std::lock_guard<std::mutex> lock(mu);
-      auto& ent = granted[reinterpret_cast<const void*>(kern)];
-      if (ent.first < smem || ent.second == 0) {
-        cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (r != cudaSuccess) return r;
-        r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nthreads, smem);
-        if (r != cudaSuccess) return r;
-        ent = {smem, per_sm};
-      }
-      per_sm = ent.second;
-    }
+    const cudaError_t r = allow_smem(kern, smem, nthreads, &per_sm);
+    if (r != cudaSuccess) return r;
     if (per_sm < 1) return cudaSuccess;
     long long grid = (long long)sms * per_sm;
     if (grid > nitems) grid = nitems;

@@ -28,6 +28,7 @@
 
 #include "async_copy.cuh"
 #include "fft_static.cuh"
+#include "kernel_grants.cuh"
 #include "kernels.cuh"
 #include "residual2.cuh"
 
@@ -167,20 +168,10 @@ XsConfig xs_config(int N, int E, unsigned stage_bytes, size_t static_smem, XsAli
 }
 
 template <typename K> cudaError_t prepare(K kernel, int threads, size_t smem, int& grid_cap) {
-  static std::mutex mu;
-  static std::unordered_map<const void*, std::pair<size_t, int>> done;   // smem granted, CTAs per SM
-  std::lock_guard<std::mutex> lock(mu);
-  auto& ent = done[reinterpret_cast<const void*>(kernel)];
-  if (ent.first < smem || ent.second == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-    if (e != cudaSuccess) return e;
-    ent = {smem, per_sm};
-  }
-  grid_cap = ent.second * sm_count();
-  return cudaSuccess;
+  int per_sm = 0;
+  const cudaError_t e = allow_smem(kernel, smem, threads, &per_sm);
+  if (e == cudaSuccess) grid_cap = per_sm * sm_count();
+  return e;
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

@@ -10,11 +10,10 @@
 // tile and the (by then consumed) input tile in a swizzled layout, and the last
 // stage's outputs go from registers straight to global memory (each warp writes
 // row segments of TK contiguous values).
-#include <mutex>
-#include <unordered_map>
 
 #include "async_copy.cuh"
 #include "fft_static.cuh"
+#include "kernel_grants.cuh"
 #include "kernels.cuh"
 
 namespace pgb {
@@ -263,8 +262,6 @@ cudaError_t ys_launch(float2* spec, const Geom& g, int N, const float2* twy, int
   const int tiles_per_level = (g.nxh + tk - 1) / tk;
   const int ntiles = tiles_per_level * g.lev1;
   const int chunk_tiles = tiles_per_level * (g.lev1 - g.lev0);
-  static std::mutex mu;
-  static std::unordered_map<const void*, std::pair<size_t, int>> granted;   // per kernel: smem, CTAs per SM
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -272,18 +269,8 @@ cudaError_t ys_launch(float2* spec, const Geom& g, int N, const float2* twy, int
   PGB_YS_N_SWITCH(N, {
     auto kern = k_ys<NN, E, SIGN, INPLACE>;
     int per_sm = 0;
-    {
-      std::lock_guard<std::mutex> lock(mu);
-      auto& ent = granted[reinterpret_cast<const void*>(kern)];
-      if (ent.first != smem || ent.second == 0) {
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nthreads, smem);
-        if (e != cudaSuccess) return e;
-        ent = {smem, per_sm};
-      }
-      per_sm = ent.second;
-    }
+    e = allow_smem(kern, smem, nthreads, &per_sm);
+    if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaSuccess;
     const int grid = chunk_tiles < sms * per_sm ? chunk_tiles : sms * per_sm;
     if (grid <= 0) return cudaSuccess;

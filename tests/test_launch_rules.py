@@ -29,3 +29,45 @@ def test_warp_masks_name_existing_lanes_only(tmp_path):
         exists = [32 * (t // 32) + b < n for b in range(32)]
         assert lanes == sum(exists)
         assert mask == sum(1 << b for b in range(32) if exists[b]), line
+
+
+def test_kernel_grants_are_kept_per_device(tmp_path):
+    """A shared memory limit is raised on each device once, never lowered, and asked for again only above it; the CTAs per
+    SM are those of the device and of the size launched; errors come back and leave no grant behind."""
+    lines = _run(tmp_path, """
+  KernelGrants g;
+  int k1, k2, n = -1;
+  auto ask = [&](int device, const void* kernel, size_t smem, int threads, int fail = 0) {
+    size_t allowed = 0;
+    int counted = 0;
+    const int e = g.get(device, kernel, smem, threads, [&](size_t b) { allowed = b; return fail; },
+                        [&](int* out) { ++counted; *out = 100 * device + (int)(smem / 1024); return 0; }, &n);
+    printf("%d %zu %d %d\\n", e, allowed, counted, n);
+  };
+  ask(0, &k1, 65536, 0);
+  ask(0, &k1, 65536, 0);
+  ask(1, &k1, 65536, 0);     // the second device has not been asked
+  ask(1, &k1, 65536, 0);
+  ask(0, &k2, 65536, 0);
+  ask(0, &k1, 32768, 0);     // below the limit
+  ask(0, &k1, 131072, 0);
+  ask(0, &k1, 65536, 256);   // CTAs per SM, of each size and device
+  ask(0, &k1, 65536, 256);
+  ask(0, &k1, 131072, 256);
+  ask(0, &k1, 65536, 256);
+  ask(1, &k1, 65536, 256);
+  ask(1, &k1, 131072, 256, 7);   // refused
+  ask(1, &k1, 131072, 256);
+""")
+    assert [tuple(map(int, line.split())) for line in lines] == [
+        (0, 65536, 0, 0), (0, 0, 0, 0), (0, 65536, 0, 0), (0, 0, 0, 0), (0, 65536, 0, 0), (0, 0, 0, 0), (0, 131072, 0, 0),
+        (0, 0, 1, 64), (0, 0, 0, 64), (0, 0, 1, 128), (0, 0, 0, 64), (0, 0, 1, 164),
+        (7, 131072, 0, 164), (0, 131072, 1, 228)]
+
+
+def test_launchers_keep_no_grants_of_their_own():
+    """Every remembered cudaFuncSetAttribute goes through the per-device table; the other launchers set it each time."""
+    for name in sorted(os.listdir(CSRC)):
+        text = open(os.path.join(CSRC, name)).read()
+        if "cudaFuncSetAttribute" in text and name != "kernel_grants.cuh":
+            assert "unordered_map" not in text and "static size_t" not in text, name
