@@ -439,18 +439,20 @@ __global__ void __launch_bounds__(256) k_cg_dir(const typename CgVec<TT>::t* __r
   }
 }
 
-// the last step's p (STEP as above; 3: p = 0), and sum p
+// the last step's p (STEP as above; 3: p = 0), and sum p.  A direction with no step (d . K d not positive: d in the
+// null space, or not finite) leaves p as it was.
 template <int STEP>
 __global__ void __launch_bounds__(256) k_cg_last(const double2* __restrict__ d, double2* __restrict__ p, CgDims D,
                                                  CgState* c, double* __restrict__ partials) {
   const double alpha = c->alpha;
+  const bool step = STEP != 3 && c->dq > 0;
   double s = 0;
 #pragma unroll 2
   CG_PAIRS(i, D) {
     double2 v = make_double2(0.0, 0.0);
-    if (STEP != 3) {
+    if (STEP == 2) v = p[i];
+    if (step) {
       const double2 dv = d[i];
-      if (STEP == 2) v = p[i];
       v = STEP == 2 ? make_double2(fma(alpha, dv.x, v.x), fma(alpha, dv.y, v.y))
                     : make_double2(alpha * dv.x, alpha * dv.y);
     }
