@@ -14,8 +14,8 @@
 //  * Accuracy: with n elements, ||X||_rms = ||x||_2 and sum |x| <= sqrt(n) ||x||_2, the rounding of the last
 //    stages, about 2^-62 of that sum, is within a few 2^-62 sqrt(n) of the result's norm: 2^-56 for n = 1024,
 //    where FP64 butterflies leave some 2^-52.5.  The conversion back rounds to 53 bits.
-//  * A line that holds an infinity or a NaN gives NaN throughout (`bad`); exponents outside the double range
-//    give infinities or zeros.
+//  * A line that holds an infinity or a NaN gives NaN throughout (`bad`); results above the double range
+//    are infinities, those below the normal range subnormal numbers.
 //
 // What it gave (GB300, 512 x 512 x 64, one pass over the field): forward x 584 -> 85 us, y 440 -> 94, inverse x
 // 560 -> 91.  The passes are now bound by the integer pipe (65% busy, about 230 instructions a complex point)
@@ -210,18 +210,20 @@ struct FxIn {
     return __double2ll_rn(__hiloint2double(keep ? hi + add : 0, keep ? __double2loint(x) : 0));
   }
 };
-// v 2^q rounded to the nearest double (below the normal range: 0, above: infinity); bad: NaN
+// v 2^q rounded to the nearest double (subnormal below the normal range, infinity above); bad: NaN
 static __device__ __noinline__ double fx_to_double_any(i64 v, int q, bool bad) {
   const i64 s = v >> 63;
   unsigned long long m = (unsigned long long)((v ^ s) - s);
   const int z = __clzll((i64)m);
   m <<= (z & 63);
   const int be = 1086 + q - z;   // biased exponent of the leading bit
-  const unsigned rest = (unsigned)m & 0x7ffu;
-  const unsigned up = (rest > 0x400u || (rest == 0x400u && ((m >> 11) & 1))) ? 1u : 0u;
-  unsigned long long r = ((unsigned long long)(unsigned)(be - 1) << 52) + (m >> 11) + up;
+  const int d = be >= 1 ? 11 : 12 - be;   // bits below the last one kept: 11, more for a subnormal number
+  unsigned long long r = d < 64 ? m >> d : 0ull;
+  const unsigned long long rest = d < 64 ? m << (64 - d) : (d == 64 ? m : 0ull), half = 1ull << 63;
+  r += (rest > half || (rest == half && (r & 1))) ? 1u : 0u;
+  if (be >= 1) r += (unsigned long long)(unsigned)(be - 1) << 52;   // the leading bit is the exponent's last unit
   r = be >= 2047 ? 0x7ff0000000000000ull : r;
-  r = (z == 64 || be < 1) ? 0ull : r;
+  r = z == 64 ? 0ull : r;
   r |= (unsigned long long)s & 0x8000000000000000ull;
   r = bad ? 0x7ff8000000000000ull : r;
   return __longlong_as_double((i64)r);
