@@ -545,8 +545,10 @@ struct GrhoSumF {   // float products, sums as float pairs
     one(p0.x, p1.x, g0.x, g1.x);
     one(p0.y, p1.y, g0.y, g1.y);
   }
-  __device__ __forceinline__ double lo() const { return (double)lh + (double)ll; }
-  __device__ __forceinline__ double up() const { return (double)uh + (double)ul; }
+  // past the float range h is the infinity (or NaN) of a plain sum, and the two-sums' low parts mean nothing
+  static __device__ __forceinline__ double value(float h, float l) { return (double)h + (isfinite(h) ? (double)l : 0.0); }
+  __device__ __forceinline__ double lo() const { return value(lh, ll); }
+  __device__ __forceinline__ double up() const { return value(uh, ul); }
 };
 struct GrhoSumM : GrhoSumF {   // mixed: double fields, rounded to float with integer operations
   using V = double2;
