@@ -115,9 +115,9 @@ struct poisson_plan {
   float2 cx{}, cy{};
   // workspace layout
   size_t off_spec = 0, off_stats = 0, off_sched = 0, stats_bytes = 0, off_part = 0, off_rpart = 0, off_sqn = 0,
-         off_r = 0, off_lz = 0, off_lw = 0, off_p0 = 0, off_q = 0,
+         off_r = 0, off_p0 = 0, off_q = 0,
          off_gp = 0, off_fa = 0, off_fb = 0, ws_bytes = 0;
-  int xinv_blocks = 1, grho_nb = 1;
+  int xinv_blocks = 1, grho_nb = 1, rpart_slots = 0;
   PhaseProfiler prof;
   bool mixed() const { return dtype == POISSON_MIXED; }
   bool fp64() const { return dtype == POISSON_FP64; }
@@ -209,18 +209,14 @@ void layout_workspace(poisson_plan* pl) {
   pl->off_sched = off + ((sizeof(Stats) + 15) & ~(size_t)15);
   pl->stats_bytes = pl->off_sched - pl->off_stats + 4 * sizeof(unsigned) * (size_t)pl->sched_words;
   off = align256(off + pl->stats_bytes);
-  pl->off_part = off;
-  off = align256(off + 3 * sizeof(double) * (size_t)(pl->xinv_blocks + pl->nz));   // + one per level chunk
-  pl->off_rpart = off;   // residual norms: per row group of the tiled kernel, or as above
-  off = align256(off + 2 * sizeof(double) *
-                           (size_t)std::max(pl->xinv_blocks + pl->nz, xres_tile_groups(pl->ny, pl->nz, pl->nx / 2)));
-  pl->off_sqn = off;   // per-CTA squared norms of a verification solve (column tiles of >= 16 columns)
-  off = align256(off + sizeof(double) * (size_t)(pl->g.plane / 16 + 1 + pl->n_lowk));
-  pl->off_lz = off;
-  off = align256(off + sizeof(double2) * (size_t)pl->nz * pl->n_lowk);
-  pl->off_lw = off;
-  off = align256(off + sizeof(double) * (size_t)pl->nz * pl->n_lowk);
-  if (pl->mixed()) {
+  if (pl->mixed()) {   // the sums of the refinement's stopping rule
+    pl->off_part = off;
+    off = align256(off + 3 * sizeof(double) * (size_t)(pl->xinv_blocks + pl->nz));   // + one per level chunk
+    pl->off_rpart = off;   // residual norms: likewise, or the tiled kernel's blocks in one launch
+    pl->rpart_slots = std::max(pl->xinv_blocks + pl->nz, xres_tile_blocks(pl->ny, pl->nz, pl->nx / 2));
+    off = align256(off + 2 * sizeof(double) * (size_t)pl->rpart_slots);
+    pl->off_sqn = off;   // per-CTA squared norms of a verification solve (column tiles of >= 16 columns)
+    off = align256(off + sizeof(double) * (size_t)(pl->g.plane / 16 + 1 + pl->n_lowk));
     pl->off_p0 = off;
     off = align256(off + sizeof(float) * (size_t)N);
     pl->off_q = off;
@@ -698,6 +694,8 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
       bool used = false;
       ResidualArgs Rc = *R;
       Rc.part0 = R->part0 + rparts;
+      // what the later chunks' launches need is left to them: a block each at least
+      Rc.slots = pl->rpart_slots - Rc.part0 - (pl->nz - gc.lev1 + lc - 1) / lc;
       int nb = 0;
       if (pl->respass && pl->off_r && pl->xkernel == 0 && lc >= pl->nz) {
         // the residual as its own pass into a float field, then the plain R2C x-pass of it
@@ -749,8 +747,6 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
   A.lowk_inv = pl->lowk_inv_d + (size_t)pl->n_lowk * pl->nz;   // the twisted ones
   A.singular00 = !pl->top_dirichlet();
   A.n_lowk = pl->n_lowk;
-  A.lowk_z = (double2*)(ws + pl->off_lz);
-  A.lowk_w = (double*)(ws + pl->off_lw);
   A.stats = stats;
   A.done = done;
   A.target_mean = target_mean;
@@ -975,7 +971,6 @@ static int solve_fields(poisson_plan* pl, const void* S, void* p, char* ws, cuda
   PGB_CUDA(launch_zero_words(stats, pl->stats_bytes, st));
   const bool t_double = pl->fp64();
   XinvExtra ex{};
-  ex.partials = (double*)(ws + pl->off_part);
   if (!pl->mixed()) {
     bool mid = false;
     PGB_CUDA(forward_columns(pl, S, t_double, ws, st, 0, nullptr, nullptr, nullptr, nullptr, 0, &mid));
@@ -984,6 +979,7 @@ static int solve_fields(poisson_plan* pl, const void* S, void* p, char* ws, cuda
     const int* done = &stats->done;
     float* p0 = (float*)(ws + pl->off_p0);
     float* q = (float*)(ws + pl->off_q);
+    ex.partials = (double*)(ws + pl->off_part);
     int nb = 0;
     // first solve: double source, float transforms, double low-|k| columns
     bool mid = false;

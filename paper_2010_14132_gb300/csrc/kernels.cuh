@@ -188,6 +188,7 @@ struct XinvExtra {
 struct ResidualArgs {
   double* partials;      // per-block sums of r^2 and S^2 (2 per block), from slot part0 on
   int part0;
+  int slots;             // the most blocks that the tiled residual pass may launch (it takes any number)
   double* p_out;         // nullable: the residual x-pass with q also stores the iterate p0 + q here (as
                          // the double the inverse x-pass would write), so that a verification stop
                          // needs no separate pass to form it
@@ -251,8 +252,6 @@ struct ThomasArgs {
   int lowk_r2;            // columns with kx^2+ky'^2 <= lowk_r2 go to the low-k kernel (>= 0)
   const int2* lowk_cols;  // (kx, ky) list, (0,0) first
   int n_lowk;
-  double2* lowk_z;        // scratch nz * n_lowk
-  double* lowk_w;         // scratch nz * n_lowk
   Stats* stats;
   const int* done;
   const double* target_mean;  // nullable: the (0,0) column then gives the solution mean -(*target_mean)
@@ -429,8 +428,8 @@ cudaError_t launch_xfwd_static(int ti_is_double, const void* in, void* spec, con
                                const Tables& tb, const int* done, unsigned* err, cudaStream_t st, bool* used);
 cudaError_t launch_xres_tile(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
                              const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used);
-// Row groups of that kernel over all levels (0: lines it does not take), an upper bound of its partial sums.
-int xres_tile_groups(int ny, int nz, int n_half);
+// Blocks that kernel launches for all levels at once (0: lines it does not take).
+int xres_tile_blocks(int ny, int nz, int n_half);
 cudaError_t launch_xres_static(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
                                const int* done, unsigned* err, int* nblocks_out, cudaStream_t st, bool* used);
 cudaError_t launch_xinv_static(int to_is_double, int mode, const void* spec, void* out, const Geom& g,

@@ -212,7 +212,8 @@ cudaError_t xrt_launch(const ResidualArgs& R, float2* spec, const Geom& g, int n
     const cudaError_t e = prepare(kern, RB * (V / EE), XrtLayout<V>::total, cap);                                    \
     if (e != cudaSuccess || cap <= 0) return e;                                                                      \
     const long long groups = (long long)((g.ny + RB - 1) / RB) * (g.lev1 - g.lev0);                                  \
-    const int grid = (int)(groups < cap ? groups : cap);                                                             \
+    int grid = (int)(groups < cap ? groups : cap);                                                                   \
+    if (grid > R.slots) grid = R.slots;                                                                              \
     if (nblocks_out) *nblocks_out = grid;                                                                            \
     *used = true;                                                                                                    \
     return pdl_launch(kern, dim3(grid), dim3(V / EE, RB), XrtLayout<V>::total, st, R, spec, g, tb.twx_f, tb.twr_f,   \
@@ -251,9 +252,11 @@ cudaError_t launch_xrt_iso(const ResidualArgs& R, float2* spec, const Geom& g, i
 cudaError_t launch_xrt_iso(const ResidualArgs& R, float2* spec, const Geom& g, int n, const Tables& tb, const int* done,
                            unsigned* err, int* nblocks_out, cudaStream_t st, bool* used);
 
-int xres_tile_groups(int ny, int nz, int n) {
+int xres_tile_blocks(int ny, int nz, int n) {
   if (!xpass_static_supported(n) || !xrt_length(n)) return 0;
-  return (ny + xrt_rows(n) - 1) / xrt_rows(n) * nz;
+  const int groups = (ny + xrt_rows(n) - 1) / xrt_rows(n) * nz;
+  const int resident = (st_elems(n) == kE3 ? 3 : 4) * sm_count();   // by its registers (160-168, 112-128)
+  return groups < resident ? groups : resident;
 }
 
 cudaError_t launch_xres_tile(const ResidualArgs& R, void* spec, const Geom& g, const FftPlan& fx, const Tables& tb,
