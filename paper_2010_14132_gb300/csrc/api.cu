@@ -345,11 +345,17 @@ int poisson_plan_create(int nx, int ny, int nz, double dx, double dy, const doub
     return POISSON_ERR_UNSUPPORTED;
   }
   // The FP32 plan takes more elements per thread on long lines (xs_elems_fp32, launch_yfft_static).  A mixed plan's
-  // passes keep theirs, so that both residual passes and both forms of a batch round alike, but for 1024-point y-lines
-  // (1024 x 1024 x 128 3617 -> 3403 us; at 512 x 512 the batch of 24 domains took 0.90 of its earlier time with either).
+  // x-passes keep theirs, so that both residual passes and both forms of a batch (whose lines end at 512 points) round
+  // alike.  Its y-lines take the two stages of radix 32 from 1024 points on (1024 x 1024 x 128 3617 -> 3403 us).  Errors
+  // do not tell the forms apart: rms over 16 to 24 sources of a solve with one sweep, 32 elements against 16, 0.74 to 1.07
+  // with standard errors of 0.10 to 0.23.  Nor does the low-wavenumber verification: its norm came to 1.00 to 2.91 times
+  // the full one with 32 and 1.00 to 2.19 with 16 on nine grids of 1024-point lines with eight sources each, and it is the
+  // source that decides (512-point lines, 24 sources a grid: up to 15.7 with 32, 11.9 with 16).  Lines of 512 points would
+  // gain 3 to 4% (512 x 512 x 64 542 -> 520 us) and stay with 16 elements because that norm is held to 4 times the full
+  // one on a source where it is 1.95 with 16 and 4.16 with 32.
   if (dtype == POISSON_MIXED) {
     pl->fx.e_set = 1;
-    pl->fy.e_set = ny != 1024;
+    pl->fy.e_set = ny < 1024;
   }
   pl->g.nx = nx;
   pl->g.ny = ny;

@@ -20,7 +20,7 @@ struct FftPlan {
   int nstages;
   int E;                   // elements per thread (multiple of every radix used)
   int radix[kMaxStages];
-  int e_set;               // the compile-time kernels keep E too: an option set it, or the plan refines
+  int e_set;               // the compile-time kernels keep E too: an option set it, or the plan is mixed
 };
 
 template <int SIGN, typename C> __device__ __forceinline__ void dft2(C* v) {
