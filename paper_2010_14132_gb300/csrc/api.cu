@@ -11,6 +11,7 @@
 
 #include "../../include/poisson.h"
 #include "kernels.cuh"
+#include "launch_rules.hpp"
 
 using namespace pgb;
 
@@ -212,7 +213,7 @@ void layout_workspace(poisson_plan* pl) {
   if (pl->mixed()) {   // the sums of the refinement's stopping rule
     pl->off_part = off;
     off = align256(off + 3 * sizeof(double) * (size_t)(pl->xinv_blocks + pl->nz));   // + one per level chunk
-    pl->off_rpart = off;   // residual norms: likewise, or the tiled kernel's blocks in one launch
+    pl->off_rpart = off;   // residual norms: likewise, or the tiled kernel's blocks in one launch (chunks share them)
     pl->rpart_slots = std::max(pl->xinv_blocks + pl->nz, xres_tile_blocks(pl->ny, pl->nz, pl->nx / 2));
     off = align256(off + 2 * sizeof(double) * (size_t)pl->rpart_slots);
     pl->off_sqn = off;   // per-CTA squared norms of a verification solve (column tiles of >= 16 columns)
@@ -700,8 +701,6 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
       bool used = false;
       ResidualArgs Rc = *R;
       Rc.part0 = R->part0 + rparts;
-      // what the later chunks' launches need is left to them: a block each at least
-      Rc.slots = pl->rpart_slots - Rc.part0 - (pl->nz - gc.lev1 + lc - 1) / lc;
       int nb = 0;
       if (pl->respass && pl->off_r && pl->xkernel == 0 && lc >= pl->nz) {
         // the residual as its own pass into a float field, then the plain R2C x-pass of it
@@ -715,7 +714,14 @@ static cudaError_t forward_columns(poisson_plan* pl, const void* in, int in_doub
       }
       bool stat = false;
       if (e == cudaSuccess && !used && pl->xkernel == 0) {
-        e = launch_xres_tile(Rc, spec, gc, pl->fx, pl->tb, done, &stats->err, &nb, st, &used);
+        // the tiled pass's chunks add to the slots of the first one's blocks, so that none has fewer blocks for them
+        ResidualArgs Rt = Rc;
+        Rt.part0 = R->part0;
+        Rt.part_add = l0 > 0;
+        Rt.slots = pl->rpart_slots - R->part0;
+        int nt = 0;
+        e = launch_xres_tile(Rt, spec, gc, pl->fx, pl->tb, done, &stats->err, &nt, st, &used);
+        if (e == cudaSuccess && used) nb = added_slots(rparts, nt);
         if (e == cudaSuccess && !used)
           e = launch_xres_static(Rc, spec, gc, pl->fx, pl->tb, done, &stats->err, &nb, st, &used);
         stat = used;

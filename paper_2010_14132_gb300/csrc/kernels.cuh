@@ -189,6 +189,7 @@ struct ResidualArgs {
   double* partials;      // per-block sums of r^2 and S^2 (2 per block), from slot part0 on
   int part0;
   int slots;             // the most blocks that the tiled residual pass may launch (it takes any number)
+  int part_add;          // the tiled pass adds to its slots: another chunk's launch of the same pass wrote them
   double* p_out;         // nullable: the residual x-pass with q also stores the iterate p0 + q here (as
                          // the double the inverse x-pass would write), so that a verification stop
                          // needs no separate pass to form it

@@ -26,6 +26,16 @@ PGB_HD unsigned warp_mask(int t, int n) {
   return lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
 }
 
+// Blocks of one launch of the tiled residual pass: all groups of rows that are resident at once, up to the slots for
+// their sums.  The launches of a pass's level chunks use the same slots, one after the other (each chunk's blocks in
+// slots of its own left the last chunks one block: 256 x 256 x 48 in chunks of five levels 635 -> 2247 us).
+inline int tile_pass_blocks(long long groups, int resident, int slots) {
+  const int n = groups < resident ? (int)groups : resident;
+  return n < slots ? n : slots;
+}
+// Slots that a launch of n blocks adds to those in use.
+inline int added_slots(int in_use, int n) { return n > in_use ? n - in_use : 0; }
+
 // What the kernels have been granted, for all devices of the process: a kernel's shared memory limit is an attribute of
 // the kernel on one device, and its CTAs per SM depend on the device and on the shared memory it is launched with.
 class KernelGrants {

@@ -194,9 +194,9 @@ __global__ void __launch_bounds__(xrt_rows(N) * (N / E), xrt_blocks(N))
     __syncthreads();
   }
   if (tid == 0 && R.partials) {
-    const long long slot = R.part0 + blockIdx.x;
-    R.partials[2 * slot] = (double)red[0][0];
-    R.partials[2 * slot + 1] = (double)red[1][0];
+    double* out = R.partials + 2 * (R.part0 + (long long)blockIdx.x);
+    out[0] = (double)red[0][0] + (R.part_add ? out[0] : 0.0);
+    out[1] = (double)red[1][0] + (R.part_add ? out[1] : 0.0);
   }
 }
 
@@ -212,8 +212,7 @@ cudaError_t xrt_launch(const ResidualArgs& R, float2* spec, const Geom& g, int n
     const cudaError_t e = prepare(kern, RB * (V / EE), XrtLayout<V>::total, cap);                                    \
     if (e != cudaSuccess || cap <= 0) return e;                                                                      \
     const long long groups = (long long)((g.ny + RB - 1) / RB) * (g.lev1 - g.lev0);                                  \
-    int grid = (int)(groups < cap ? groups : cap);                                                                   \
-    if (grid > R.slots) grid = R.slots;                                                                              \
+    const int grid = tile_pass_blocks(groups, cap, R.slots);                                                         \
     if (nblocks_out) *nblocks_out = grid;                                                                            \
     *used = true;                                                                                                    \
     return pdl_launch(kern, dim3(grid), dim3(V / EE, RB), XrtLayout<V>::total, st, R, spec, g, tb.twx_f, tb.twr_f,   \

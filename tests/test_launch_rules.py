@@ -71,3 +71,29 @@ def test_launchers_keep_no_grants_of_their_own():
         text = open(os.path.join(CSRC, name)).read()
         if "cudaFuncSetAttribute" in text and name != "kernel_grants.cuh":
             assert "unordered_map" not in text and "static size_t" not in text, name
+
+
+def test_level_chunks_of_the_tiled_pass_have_all_their_blocks(tmp_path):
+    """Slots for the blocks of one launch over all levels (or for the larger count of another pass) are enough for every
+    chunk: each launches all groups of rows that are resident at once, and the slots in use never pass their number."""
+    lines = _run(tmp_path, """
+  const int resident = 608;
+  for (int per_level : {1, 3, 32, 128, 700})
+    for (int nz : {2, 37, 48, 128})
+      for (int spare : {0, 100})
+        for (int chunk : {1, 5, 19, 128}) {
+          const int lc = chunk < nz ? chunk : nz;
+          const int slots = tile_pass_blocks((long long)per_level * nz, resident, 1 << 30) + spare;
+          int used = 0;
+          for (int l0 = 0; l0 < nz; l0 += lc) {
+            const long long groups = (long long)per_level * (l0 + lc < nz ? lc : nz - l0);
+            const int n = tile_pass_blocks(groups, resident, slots);
+            used += added_slots(used, n);
+            printf("%lld %d %d %d\\n", groups, n, used, slots);
+          }
+        }
+""")
+    assert len(lines) > 1000
+    for line in lines:
+        groups, n, used, slots = map(int, line.split())
+        assert n == min(groups, 608) and n <= used <= slots
