@@ -184,8 +184,14 @@ inline int xs_elems(int N, int plan_e) { return N % 3 == 0 ? st_elems(N) : (plan
 // points take two stages (16 16) instead of three, 512 as many, with one warp per line instead of two and no barrier
 // between warps.  FP32 1024 x 1024 x 64 492 us with 8 in both, 483 with 16 in the forward pass, 476 in both;
 // 512 x 512 x 64 139 with 8, 136 with 16 in the forward pass, 139 in both; 256 x 256 x 64 (128 points) 47.9 and 51.8.
-inline int xs_elems_fp32(const FftPlan& fx, bool inverse) {
-  return fx.e_set || fx.n % 3 == 0 || fx.n < (inverse ? 512 : 256) ? xs_elems(fx.n, fx.E) : 16;
+// Up to 4096 lines a pass leaves warp slots empty, and what counts is the time of one line, which twice the threads
+// shorten: solves with 8 and with 16 take 41.3 and 46.5 us at 4096 x 64 x 8 (512 lines), 36.5 and 38.2 at 2048 x 128 x 8,
+// 36.6 and 39.2 at 1024 x 64 x 32 (2048 lines), 34.3 and 35.5 at 512 x 128 x 32 (4096), but 133.4 and 126.1 at
+// 2048 x 256 x 32, 46.4 and 45.0 at 512 x 256 x 32 (8192).  The lines of all levels count, so that chunks of them round
+// alike.
+inline int xs_elems_fp32(const FftPlan& fx, const Geom& g, bool inverse) {
+  const bool more = !fx.e_set && fx.n % 3 != 0 && fx.n >= (inverse ? 512 : 256) && (long long)g.ny * g.nz > 4096;
+  return more ? 16 : xs_elems(fx.n, fx.E);
 }
 
 // Dispatch to the compile-time (N, E) instance; shapes the engine cannot take are

@@ -127,7 +127,7 @@ cudaError_t launch_xfwd_static(int ti_is_double, const void* in, void* spec, con
                                const Tables& tb, const int* done, unsigned* err, cudaStream_t st, bool* used) {
   *used = false;
   if (!xpass_static_supported(fx.n)) return cudaSuccess;
-  const int E = ti_is_double ? xs_elems(fx.n, fx.E) : xs_elems_fp32(fx, false);
+  const int E = ti_is_double ? xs_elems(fx.n, fx.E) : xs_elems_fp32(fx, g, false);
   if (ti_is_double) return xfwd_s<double>((const double*)in, (float2*)spec, g, fx.n, E, tb, done, err, st, used);
   return xfwd_s<float>((const float*)in, (float2*)spec, g, fx.n, E, tb, done, err, st, used);
 }

@@ -271,7 +271,7 @@ cudaError_t launch_xinv_static(int to_is_double, int mode, const void* spec, voi
   *used = false;
   if (!xpass_static_supported(fx.n)) return cudaSuccess;
   const float2* sp = (const float2*)spec;
-  const int E = mode != XINV_PLAIN || to_is_double ? xs_elems(fx.n, fx.E) : xs_elems_fp32(fx, true);
+  const int E = mode != XINV_PLAIN || to_is_double ? xs_elems(fx.n, fx.E) : xs_elems_fp32(fx, g, true);
   if (mode == XINV_P0) return xinv_s<float, XINV_P0>(sp, (float*)out, g, fx.n, E, tb, ex, nblocks_out, st, used);
   if (mode == XINV_UPDATE)
     return xinv_s<float, XINV_UPDATE>(sp, (float*)out, g, fx.n, E, tb, ex, nblocks_out, st, used);
