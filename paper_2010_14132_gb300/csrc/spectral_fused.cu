@@ -86,8 +86,13 @@ __host__ __device__ constexpr size_t mid_buf_bytes(int N, int nz, int TC, size_t
   return y > c ? (y > l ? y : l) : (c > l ? c : l);
 }
 
+// CTAs per SM asked of the compiler: at 256 points three (of 128 threads) hide more of the items' waits than two (FP32
+// 256 x 256 x 48 with this option 56.8 -> 53.2 us, mixed 262 -> 253; unasked, the double low-|k| column takes the kernel to 182 registers,
+// two CTAs)
+constexpr int mid_min_blocks(int n) { return n <= 256 ? 3 : 2; }
+
 template <int N, int TC>
-__global__ void __launch_bounds__(kMidTK * (N / kMidE), 2)
+__global__ void __launch_bounds__(kMidTK * (N / kMidE), mid_min_blocks(N))
     k_mid(const __grid_constant__ CUtensorMap tmy, const __grid_constant__ CUtensorMap tmc, MidArgs A) {
   using C = float2;
   constexpr int E = kMidE, TK = kMidTK, NT = TK * (N / E), TY = TC / TK;
