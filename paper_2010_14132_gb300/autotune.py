@@ -5,9 +5,9 @@ For one grid (nx, ny, nz, dtype) it times candidate settings of the y-pass
 x-pass (persistent bulk-copy-staged kernel, or one CTA per row group with 8 or
 16 elements per thread), using the library's own per-phase CUDA events
 (POISSON_OPT_PROFILE) on the launching stream, and keeps the fastest setting of
-each pass.  Results are cached in a JSON file keyed by GPU name, sizes and
-dtype, so a plan is tuned once and the choice reused every solve (the
-plan-once idea of Section 2.1).
+each pass.  Results are cached in a JSON file keyed by GPU name, sizes, dtype
+and the library's sources, so a plan is tuned once and the choice reused every
+solve (the plan-once idea of Section 2.1).
 
     from paper_2010_14132_gb300.autotune import tuned_options
     opts = tuned_options(nx, ny, nz, dx, dy, dz, rho0, "mixed")
@@ -15,6 +15,9 @@ plan-once idea of Section 2.1).
 """
 from __future__ import annotations
 
+import functools
+import glob
+import hashlib
 import json
 import os
 
@@ -22,6 +25,7 @@ import numpy as np
 import torch
 
 from . import _native as N
+from .build import CSRC, INCLUDE
 from .solver import Plan
 
 CACHE = os.environ.get("POISSON_AUTOTUNE_CACHE",
@@ -39,9 +43,20 @@ OPT_IDS = {"y_kernel": N.POISSON_OPT_Y_KERNEL, "y_tile": N.POISSON_OPT_Y_TILE, "
            "spectral_fused": N.POISSON_OPT_SPECTRAL_FUSED, "residual_pass": N.POISSON_OPT_RESIDUAL_PASS}
 
 
+@functools.lru_cache(maxsize=None)
+def _sources():
+    """Fingerprint of the kernels and their launchers, the option ids and the candidates here: a choice holds for the code it
+    was measured with (one kept from before a default changed would go on setting the old one)."""
+    h = hashlib.sha256()
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.*")) + glob.glob(os.path.join(INCLUDE, "*.h"))) + [__file__]:
+        with open(path, "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _key(nx, ny, nz, dtype):
     name = torch.cuda.get_device_name()
-    return f"{name}|{nx}x{ny}x{nz}|{dtype}"
+    return f"{name}|{nx}x{ny}x{nz}|{dtype}|{_sources()}"
 
 
 def _load_cache():
@@ -157,7 +172,7 @@ def autotune(nx, ny, nz, dx, dy, dz, rho0, dtype="mixed", reps=3, verbose=False)
 
 
 def tuned_options(nx, ny, nz, dx, dy, dz, rho0, dtype="mixed", retune=False):
-    """Cached autotune result for this GPU, size and dtype (tunes on first use)."""
+    """Cached autotune result for this GPU, size, dtype and build of the library (tunes on first use)."""
     cache = _load_cache()
     key = _key(nx, ny, nz, dtype)
     if key in cache and not retune:
