@@ -36,6 +36,16 @@ inline int tile_pass_blocks(long long groups, int resident, int slots) {
 // Slots that a launch of n blocks adds to those in use.
 inline int added_slots(int in_use, int n) { return n > in_use ? n - in_use : 0; }
 
+// FP64 column kernel: values a lane carries, of a pair of columns (4), one column (2) or one real or imaginary part (1),
+// for 19, 13 or 10 FP64 instructions per level of every warp (16 lanes of columns, both halves) that one of the FP64 units,
+// four an SM, has to run; the least of the three (128 x 128 x 64 on 608 units: one column, 97 -> 77 us for the solve).
+inline int fp64_column_values(long long pairs, long long cols, int sms) {
+  const long long units = sms > 0 ? 4ll * sms : 1;
+  auto cost = [units](long long lanes, int per_level) { return ((lanes + 15) / 16 + units - 1) / units * per_level; };
+  const long long c4 = cost(pairs, 19), c2 = cost(cols, 13), c1 = cost(2 * cols, 10);
+  return c4 <= c2 && c4 <= c1 ? 4 : (c2 <= c1 ? 2 : 1);
+}
+
 // What the kernels have been granted, for all devices of the process: a kernel's shared memory limit is an attribute of
 // the kernel on one device, and its CTAs per SM depend on the device and on the shared memory it is launched with.
 class KernelGrants {

@@ -1,6 +1,7 @@
 // Refinement control, correction rebuild, coefficient tables, rho0-gradient reductions and
 // the field-layout conversion.
 #include "columns.cuh"
+#include "kernel_grants.cuh"
 #include "kernels.cuh"
 #include "residual2.cuh"
 
@@ -623,7 +624,7 @@ cudaError_t launch_grho(int kind, const void* g, const void* p, const Geom& g_, 
   // kGrhoPoints points a thread, fewer while that leaves less than about four blocks per SM
   const int faces = g_.nz - 1;
   long long nb = (2 * half + 256 * kGrhoPoints - 1) / (256 * kGrhoPoints);
-  const long long fill = (608 + faces - 1) / faces, most = (half + 255) / 256;
+  const long long fill = (4ll * sm_count() + faces - 1) / faces, most = (half + 255) / 256;
   if (nb < fill) nb = fill;
   if (nb > most) nb = most;
   if (nb > nparts_max) nb = nparts_max;

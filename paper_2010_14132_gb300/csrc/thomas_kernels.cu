@@ -20,6 +20,7 @@
 #include "kernels.cuh"
 #include "async_copy.cuh"
 #include "columns.cuh"
+#include "kernel_grants.cuh"
 
 namespace pgb {
 
@@ -612,23 +613,21 @@ static cudaError_t thomas_d_nr(const ThomasArgs& A, const Geom& g, const Tables&
   // that finish first, and this kernel needs its warps spread evenly over the FP64 units (256 x 256 x 64 solve: 226 us
   // with the early launch, 162 without; 54 x 54 x 48: 110 and 70; 32 x 32 x 32: 34.6 and 36.9).
   const dim3 grid((unsigned)((lanes + 15) / 16 + A.n_lowk));
-  if (grid.x <= 152)
+  if (grid.x <= (unsigned)sm_count())
     return pdl_launch(kern, grid, dim3(32), smem, st, (double2*)A.spec, g, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d,
                       A.lowk_r2, A.stats, L);
   kern<<<grid, 32, smem, st>>>((double2*)A.spec, g, tb.a_d, tb.c_d, tb.lamx_d, tb.lamy_d, A.lowk_r2, A.stats, L);
   return cudaGetLastError();
 }
 
-// Two columns, one column or one part a lane: 19, 13 or 10 FP64 instructions per level for every warp that one of the
-// 608 FP64 units has to run; the least of the three (128 x 128 x 64: one column, 97 -> 77 us for the solve).
 template <bool ADJ>
 static cudaError_t thomas_d_launch(const ThomasArgs& A, const Geom& g, const Tables& tb, cudaStream_t st) {
   const long long pairs = (long long)(g.ny / 2 + 1) * g.nxh, cols = (long long)g.ny * g.nxh;
-  auto cost = [](long long lanes, int per_level) { return ((lanes + 15) / 16 + 607) / 608 * per_level; };
-  const long long c4 = cost(pairs, 19), c2 = cost(cols, 13), c1 = cost(2 * cols, 10);
-  if (c4 <= c2 && c4 <= c1) return thomas_d_nr<4, ADJ>(A, g, tb, pairs, st);
-  if (c2 <= c1) return thomas_d_nr<2, ADJ>(A, g, tb, cols, st);
-  return thomas_d_nr<1, ADJ>(A, g, tb, 2 * cols, st);
+  switch (fp64_column_values(pairs, cols, sm_count())) {
+    case 4: return thomas_d_nr<4, ADJ>(A, g, tb, pairs, st);
+    case 2: return thomas_d_nr<2, ADJ>(A, g, tb, cols, st);
+    default: return thomas_d_nr<1, ADJ>(A, g, tb, 2 * cols, st);
+  }
 }
 
 template <typename T, bool ADJ>

@@ -23,9 +23,6 @@
 // xpass_inv.cu) share: the shared-memory layout, the staging-ring bookkeeping,
 // the R2C unpacking and the launch configuration.
 #pragma once
-#include <mutex>
-#include <unordered_map>
-
 #include "async_copy.cuh"
 #include "fft_static.cuh"
 #include "kernel_grants.cuh"
@@ -125,20 +122,6 @@ __device__ __forceinline__ void r2c_unpack_store(const float2* fin, const float2
 // ---------------------------------------------------------------------------
 // launch configuration
 // ---------------------------------------------------------------------------
-
-int sm_count() {
-  static std::mutex mu;
-  static std::unordered_map<int, int> cache;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = cache.find(dev);
-  if (it != cache.end()) return it->second;
-  int n = 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 0;
-  cache[dev] = n;
-  return n;
-}
 
 struct XsConfig {
   int ns = 0;

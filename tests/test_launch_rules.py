@@ -1,5 +1,6 @@
 """The launch rules of csrc/launch_rules.hpp, compiled by the host compiler (no GPU, no CUDA header)."""
 import os
+import re
 import shutil
 import subprocess
 
@@ -97,3 +98,30 @@ def test_level_chunks_of_the_tiled_pass_have_all_their_blocks(tmp_path):
     for line in lines:
         groups, n, used, slots = map(int, line.split())
         assert n == min(groups, 608) and n <= used <= slots
+
+
+def test_fp64_column_form_by_the_device(tmp_path):
+    """Values a lane for the least FP64 work of the busiest of four units an SM, on devices of several sizes (also one whose
+    SM count could not be told)."""
+    sizes = [(nx // 2 + 1, ny) for nx in (4, 16, 32, 54, 64, 128, 256, 512, 1024, 4096) for ny in (4, 27, 32, 81, 128, 512, 4096)]
+    lines = _run(tmp_path, "".join(
+        f'  for (int sms : {{0, 1, 76, 148, 152}}) printf("%d %d\\n", sms, fp64_column_values({(ny // 2 + 1) * nxh}ll, {ny * nxh}ll, sms));\n'
+        for nxh, ny in sizes))
+    assert len(lines) == 5 * len(sizes)
+    seen = set()
+    for i, line in enumerate(lines):
+        nxh, ny = sizes[i // 5]
+        sms, values = map(int, line.split())
+        warps = lambda lanes: -(-lanes // 16)  # noqa: E731
+        cost = {v: -(-warps(lanes) // max(1, 4 * sms)) * per_level
+                for v, lanes, per_level in ((4, (ny // 2 + 1) * nxh, 19), (2, ny * nxh, 13), (1, 2 * ny * nxh, 10))}
+        assert values == min((4, 2, 1), key=lambda v: cost[v]), (nxh, ny, sms)
+        seen.add((sms, values))
+    assert {(76, 1), (76, 4), (152, 1), (152, 2), (152, 4)} <= seen
+
+
+def test_no_launcher_counts_the_sms_of_one_device():
+    for name in sorted(os.listdir(CSRC)):
+        for n, line in enumerate(open(os.path.join(CSRC, name))):
+            code = line.split("//")[0]
+            assert not re.search(r"\b(152|304|608|607)\b", code), f"{name}:{n + 1}"
