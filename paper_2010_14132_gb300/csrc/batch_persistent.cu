@@ -451,9 +451,8 @@ __device__ void item_lowk(const BDom& D, int pass, int sub, unsigned char* sm) {
   if (tid < ncol) {
     const int2 ck = __ldg(&D.lowk_cols[j0 + tid]);
     const bool singular = D.singular00 && ck.x == 0 && ck.y == 0;
-    lowk_recurrence<double, false>(zx + tid, zy + tid, w + tid, kBLowk, a, c, W, nz, ck.x, ck.y, singular, D.lamx_d,
-                                   D.lamy_d, D.scale_d, target_mean, D.stats, red + 5 * tid, sq + tid,
-                                   D.lowk_inv != nullptr);
+    lowk_recurrence(zx + tid, zy + tid, w + tid, kBLowk, a, c, W, nz, ck.x, ck.y, singular, D.lamx_d, D.lamy_d,
+                    D.scale_d, target_mean, D.stats, red + 5 * tid, sq + tid, D.lowk_inv != nullptr);
   }
   __syncthreads();
   for (int i = tid; i < nz * kBLowk; i += kBT) {

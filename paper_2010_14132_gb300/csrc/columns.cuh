@@ -36,19 +36,12 @@ struct LowkArgs {
 // One step of the low-|k| pivot recurrence (rounded step by step, so that the table built ahead by
 // k_lowk_pivots and a column solve computing its own pivots agree bit for bit):
 // g_k = s + a_k g_{k-1}/u_{k-1} (g_0 = s), u_k = g_k + c_k, returns 1/u_k (0 for the pinned singular top).
-template <typename TCm> __device__ __forceinline__ TCm rn_mul(TCm x, TCm y);
-template <> __device__ __forceinline__ double rn_mul<double>(double x, double y) { return __dmul_rn(x, y); }
-template <> __device__ __forceinline__ float rn_mul<float>(float x, float y) { return __fmul_rn(x, y); }
-template <typename TCm> __device__ __forceinline__ TCm rn_add(TCm x, TCm y);
-template <> __device__ __forceinline__ double rn_add<double>(double x, double y) { return __dadd_rn(x, y); }
-template <> __device__ __forceinline__ float rn_add<float>(float x, float y) { return __fadd_rn(x, y); }
-template <typename TCm>
-__device__ __forceinline__ TCm lowk_pivot_step(int k, TCm s, TCm ak, TCm ck, TCm& g_prev, TCm inv_prev,
-                                               bool last_singular) {
-  const TCm gk = (k == 0) ? s : rn_add(s, rn_mul(rn_mul(ak, g_prev), inv_prev));
-  const TCm u = rn_add(gk, ck);
+__device__ __forceinline__ double lowk_pivot_step(int k, double s, double ak, double ck, double& g_prev, double inv_prev,
+                                                  bool last_singular) {
+  const double gk = (k == 0) ? s : __dadd_rn(s, __dmul_rn(__dmul_rn(ak, g_prev), inv_prev));
+  const double u = __dadd_rn(gk, ck);
   g_prev = gk;
-  return last_singular ? (TCm)0 : (TCm)1 / u;   // the singular top pivot is pinned
+  return last_singular ? 0.0 : 1.0 / u;   // the singular top pivot is pinned
 }
 
 // ---------------------------------------------------------------------------
@@ -59,27 +52,26 @@ __device__ __forceinline__ TCm lowk_pivot_step(int k, TCm s, TCm ak, TCm ck, TCm
 //   adjoint: remove the plain mean of the right-hand side, pin v_{nz-1} = 0,
 //            back-substitute, remove the W direction (x -= W sum(x)/sum(W)).
 // ---------------------------------------------------------------------------
-// The sequential recurrence of one low-|k| or singular column, run by one thread
+// The sequential recurrence of one low-|k| or singular column (forward solve), run by one thread
 // out of shared memory: the right-hand side at zx[k ld], zy[k ld] (real and
 // imaginary parts; overwritten by the solution before any mean shift), the
 // back-substitution factors in w[k ld], the level tables a, c, W (stride 1).
-// red receives (shift_x, shift_y, sum W, sum x, sum y) for the caller's output
-// pass; sq_out (nullable, forward only) the sum of |x_k|^2 of the output.
+// red receives (shift_x, shift_y, 1, sum x, sum y) for the caller's output
+// pass; sq_out (nullable) the sum of |x_k|^2 of the output.
 // tab: w[k ld] holds the column's pivot reciprocals 1/u_k on entry (staged by the caller from the
 // plan's table, in parallel): the chain then loads them from shared memory instead of forming
 // pivots, and the back substitution forms its factors from them (the same products as when they are
 // stored by the forward sweep, so both ways give the same bits).
-template <typename TCm, bool ADJ>
-__device__ __forceinline__ void lowk_recurrence(TCm* zx, TCm* zy, TCm* w, int ld, const TCm* a, const TCm* c,
-                                                const TCm* W, int nz, int kx, int ky, bool singular,
+__device__ __forceinline__ void lowk_recurrence(double* zx, double* zy, double* w, int ld, const double* a,
+                                                const double* c, const double* W, int nz, int kx, int ky, bool singular,
                                                 const double* __restrict__ lamx, const double* __restrict__ lamy,
                                                 double scale, const double* __restrict__ target_mean,
-                                                Stats* stats, TCm* red, double* sq_out, bool tab = false) {
-  TCm mean_x = 0, mean_y = 0;
+                                                Stats* stats, double* red, double* sq_out, bool tab) {
+  double mean_x = 0, mean_y = 0;
   if (singular) {
-    TCm sw = 0;
+    double sw = 0;
     for (int k = 0; k < nz; ++k) {
-      const TCm wk = ADJ ? (TCm)1 : (TCm)W[k];
+      const double wk = W[k];
       mean_x += wk * zx[k * ld];
       mean_y += wk * zy[k * ld];
       sw += wk;
@@ -87,48 +79,34 @@ __device__ __forceinline__ void lowk_recurrence(TCm* zx, TCm* zy, TCm* w, int ld
     mean_x /= sw;
     mean_y /= sw;
     // only the first solve records mu_W (a refinement correction solve has a target mean)
-    if (!ADJ && stats && !target_mean) stats->mu_w = (double)mean_x * scale;
+    if (stats && !target_mean) stats->mu_w = mean_x * scale;
   }
-  const TCm s = singular ? (TCm)0 : -((TCm)lamx[kx] + (TCm)lamy[ky]);
-  const TCm ms = -(TCm)scale;
-  TCm g_prev = s, inv_prev = 0, yx = 0, yy = 0;
+  const double s = singular ? 0.0 : -(lamx[kx] + lamy[ky]);
+  const double ms = -scale;
+  double g_prev = s, inv_prev = 0, yx = 0, yy = 0;
   for (int k = 0; k < nz; ++k) {
-    const TCm bx = ms * (zx[k * ld] - mean_x), by = ms * (zy[k * ld] - mean_y);
+    const double bx = ms * (zx[k * ld] - mean_x), by = ms * (zy[k * ld] - mean_y);
     // the pivots depend on the column's wavenumbers and the levels only: staged from the plan's
     // table when it has them (no division on the chain), else computed here
-    const TCm inv = tab ? w[k * ld]
-                        : lowk_pivot_step<TCm>(k, s, (TCm)a[k], (TCm)c[k], g_prev, inv_prev,
-                                               singular && (k == nz - 1));
-    if (!ADJ) {
-      TCm nx_ = bx, ny_ = by;
-      if (k > 0) {
-        const TCm f = (TCm)a[k] * inv_prev;
-        nx_ += f * yx;
-        ny_ += f * yy;
-      }
-      yx = nx_;
-      yy = ny_;
-      zx[k * ld] = yx * inv;
-      zy[k * ld] = yy * inv;
-      if (!tab) w[k * ld] = (TCm)c[k] * inv;
-    } else {
-      TCm nx_ = bx, ny_ = by;
-      if (k > 0) {
-        nx_ += (TCm)c[k - 1] * yx;
-        ny_ += (TCm)c[k - 1] * yy;
-      }
-      yx = nx_ * inv;
-      yy = ny_ * inv;
-      zx[k * ld] = yx;
-      zy[k * ld] = yy;
-      if (!tab) w[k * ld] = (k + 1 < nz) ? (TCm)a[k + 1] * inv : (TCm)0;
+    const double inv =
+        tab ? w[k * ld] : lowk_pivot_step(k, s, a[k], c[k], g_prev, inv_prev, singular && (k == nz - 1));
+    double nx_ = bx, ny_ = by;
+    if (k > 0) {
+      const double f = a[k] * inv_prev;
+      nx_ += f * yx;
+      ny_ += f * yy;
     }
+    yx = nx_;
+    yy = ny_;
+    zx[k * ld] = yx * inv;
+    zy[k * ld] = yy * inv;
+    if (!tab) w[k * ld] = c[k] * inv;
     inv_prev = inv;
   }
-  TCm xx = zx[(nz - 1) * ld], xy = zy[(nz - 1) * ld];
-  TCm sx = xx, sy = xy;
+  double xx = zx[(nz - 1) * ld], xy = zy[(nz - 1) * ld];
+  double sx = xx, sy = xy;
   for (int k = nz - 2; k >= 0; --k) {
-    const TCm wk = !tab ? w[k * ld] : (ADJ ? (TCm)a[k + 1] * w[k * ld] : (TCm)c[k] * w[k * ld]);
+    const double wk = !tab ? w[k * ld] : c[k] * w[k * ld];
     xx = zx[k * ld] + wk * xx;
     xy = zy[k * ld] + wk * xy;
     zx[k * ld] = xx;
@@ -136,30 +114,25 @@ __device__ __forceinline__ void lowk_recurrence(TCm* zx, TCm* zy, TCm* w, int ld
     sx += xx;
     sy += xy;
   }
-  TCm shx = 0, shy = 0, swt = 1;
+  double shx = 0, shy = 0;
   if (singular) {
-    if (!ADJ) {
-      shx = sx / (TCm)nz;
-      shy = sy / (TCm)nz;
-      // refinement sweep: the correction also removes the mean of the current iterate
-      if (target_mean) shx += (TCm)__ldcg(target_mean);
-    } else {
-      swt = 0;
-      for (int k = 0; k < nz; ++k) swt += (TCm)W[k];
-    }
+    shx = sx / (double)nz;
+    shy = sy / (double)nz;
+    // refinement sweep: the correction also removes the mean of the current iterate
+    if (target_mean) shx += __ldcg(target_mean);
   }
   red[0] = shx;
   red[1] = shy;
-  red[2] = swt;
+  red[2] = 1;
   red[3] = sx;
   red[4] = sy;
-  if (!ADJ && sq_out) {
-    TCm sq = 0;
+  if (sq_out) {
+    double sq = 0;
     for (int k = 0; k < nz; ++k) {
-      const TCm ox = singular ? zx[k * ld] - shx : zx[k * ld], oy = singular ? zy[k * ld] - shy : zy[k * ld];
+      const double ox = singular ? zx[k * ld] - shx : zx[k * ld], oy = singular ? zy[k * ld] - shy : zy[k * ld];
       sq += ox * ox + oy * oy;
     }
-    *sq_out = (double)sq;
+    *sq_out = sq;
   }
 }
 

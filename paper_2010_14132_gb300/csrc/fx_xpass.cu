@@ -233,8 +233,6 @@ int4 fx_twiddle(long long m, long long n) {
 
 }  // namespace
 
-bool fx_supported(int n) { return fx_length(n); }
-
 std::vector<int4> fx_stage_table(int n) {
   std::vector<int4> t;
   if (!fx_length(n)) return t;

@@ -220,8 +220,7 @@ cudaError_t launch_xfwd_residual(const ResidualArgs& R, void* spec, const Geom& 
 cudaError_t launch_yfft(int t_is_double, int sign, void* spec, const Geom& g, const FftPlan& fy,
                         const Tables& tb, int tile, const int* done, cudaStream_t st);
 // FP64 passes in 64-bit block fixed point (fx_xpass.cu, fx_ypass.cu); *used = false when the plan has no
-// tables for them (a line length outside fx_supported).
-bool fx_supported(int n);
+// tables for them (a line length outside fx_length, fx_engine.cuh).
 std::vector<int4> fx_stage_table(int n);
 std::vector<int4> fx_unpack_table(int nx);
 cudaError_t launch_xfwd_fx(const double* in, double2* spec, const Geom& g, int n, const Tables& tb, cudaStream_t st,

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(64) k_lowk_pivots(const int2* __restrict__ col
   } else if (t == 0) {
     double g_prev = s, inv_prev = 0.0;
     for (int k = 0; k < nz; ++k) {
-      const double inv = lowk_pivot_step<double>(k, s, a[k], c[k], g_prev, inv_prev, false);
+      const double inv = lowk_pivot_step(k, s, a[k], c[k], g_prev, inv_prev, false);
       lower[k] = inv;
       inv_prev = inv;
       if (k == m - 1) meet[0] = g_prev * inv;
