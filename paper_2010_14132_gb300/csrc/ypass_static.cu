@@ -344,14 +344,20 @@ cudaError_t launch_yfft_static(int sign, void* spec, const Geom& g, const FftPla
   // exchange through shared memory and two barriers less, which is what the pass waits for (one tile per CTA: load,
   // stages and stores follow each other).  1024 x 1024 x 128: 225 -> 181 us a pass (cold; 4.8 -> 5.9 TB/s); 512 x 512 x 64:
   // 31 -> 24.7.  128 registers, no spills, two CTAs of 256 threads at 1024 and four of 128 at 512.  256 points are two
-  // stages with 16 elements already, 2048 three with either.
+  // stages with 16 elements already, 2048 three with either.  512 points with no more tiles than SMs keep 16: one tile is
+  // all an SM then has to do, and twice the threads shorten it by more than the stage saved (FP32 solves with 32 and 16:
+  // 64 x 512 x 8, 40 tiles, 29.7 and 27.7 us; 128 x 512 x 16, 144, 33.1 and 31.4; 64 x 512 x 32, 160, 36.8 and 36.5;
+  // 1024 x 512 x 3, 195, 36.0 and 36.5; 128 x 512 x 24, 216, 35.0 and 37.1), where 1024 points gain with any number.  The
+  // tiles of all levels count, so that chunks of them round alike.
   if (variant == 2 && E == 16 && !fy.e_set && (fy.n == 512 || fy.n == 1024)) {
     int tk1 = tk;
     while (tk1 > 2 && tk1 * (fy.n / 32) > ys1_max_threads(fy.n, 32)) tk1 >>= 1;
-    float2* sp = (float2*)spec;
-    const cudaError_t e = sign < 0 ? ys1_launch<32, -1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used)
-                                   : ys1_launch<32, +1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used);
-    if (e != cudaSuccess || *used) return e;
+    if (fy.n == 1024 || (long long)((g.nxh + tk1 - 1) / tk1) * g.nz > sm_count()) {
+      float2* sp = (float2*)spec;
+      const cudaError_t e = sign < 0 ? ys1_launch<32, -1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used)
+                                     : ys1_launch<32, +1>(sp, g, fy.n, tb.twy_f, tk1, done, err, st, used);
+      if (e != cudaSuccess || *used) return e;
+    }
   }
   if (variant == 2 && E != 8) {   // single-buffered, in place, two CTAs per SM
     int tk1 = tk;
