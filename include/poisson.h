@@ -98,9 +98,10 @@ typedef enum {
                                     in place, two CTAs per SM, the next tile's load overlapping this
                                     tile's stores (16 elements per thread; otherwise as 0) */
   POISSON_OPT_X_ELEMS = 6,       /* x-pass elements per thread for power-of-two lines: 8 or 16; unset: 8, and 16
-                                    for the FP32 plan's longer lines where that is faster */
+                                    for the FP32 plan's longer lines where it has more than 4096 of them */
   POISSON_OPT_Y_ELEMS = 7,       /* y-pass elements per thread for power-of-two lines: 8 or 16; unset: 16, and with
-                                    kernel 4 32 for 1024 points and for the FP32 plan's 512 */
+                                    kernel 4 32 for 1024 points and for the FP32 plan's 512 where it has more
+                                    tiles of a level's columns than the device has SMs */
   POISSON_OPT_LEVEL_CHUNK = 8,   /* levels per transform chunk (x-pass and y-pass of a chunk run back to
                                     back so its spectrum stays in L2); 0 = all levels in one chunk
                                     (default: the persistent kernels lose more to per-launch start-up

@@ -13,7 +13,10 @@
 //    rounding to nearest.  A line dominated by one bin is not shifted at all, noise by about log2(n) - 2 bits.
 //  * Accuracy: with n elements, ||X||_rms = ||x||_2 and sum |x| <= sqrt(n) ||x||_2, the rounding of the last
 //    stages, about 2^-62 of that sum, is within a few 2^-62 sqrt(n) of the result's norm: 2^-56 for n = 1024,
-//    where FP64 butterflies leave some 2^-52.5.  The conversion back rounds to 53 bits.
+//    where FP64 butterflies leave some 2^-52.5.  The conversion back rounds to 53 bits.  Whole solves with
+//    lines of 16 to 2048 points, measured against extended precision: errors 0.62 of the butterflies' for noise,
+//    0.7 to 0.8 for fields with a dominant bin, an outlier or a weak level, 0.02 where low wavenumbers amplify
+//    what the transforms leave in them.
 //  * A line that holds an infinity or a NaN gives NaN throughout (`bad`); results above the double range
 //    are infinities, those below the normal range subnormal numbers.
 //
