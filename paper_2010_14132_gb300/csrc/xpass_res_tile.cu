@@ -195,8 +195,9 @@ __global__ void __launch_bounds__(xrt_rows(N) * (N / E), xrt_blocks(N))
   }
   if (tid == 0 && R.partials) {
     double* out = R.partials + 2 * (R.part0 + (long long)blockIdx.x);
-    out[0] = (double)red[0][0] + (R.part_add ? out[0] : 0.0);
-    out[1] = (double)red[1][0] + (R.part_add ? out[1] : 0.0);
+    // at L2: blocks of the chunk before, on other SMs, wrote these lines
+    out[0] = (double)red[0][0] + (R.part_add ? __ldcg(out) : 0.0);
+    out[1] = (double)red[1][0] + (R.part_add ? __ldcg(out + 1) : 0.0);
   }
 }
 
